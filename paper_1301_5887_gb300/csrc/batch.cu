@@ -36,6 +36,7 @@ namespace {
 struct BatchGraph {
   GraphView g;
   const uint64_t* lo;     // bin table of the request's bins
+  const GuideBin* gtab;   // and their guide table
   uint32_t nb, pow2;
   uint32_t seed_lo, seed_hi;
   wedge_record* records;  // global-stream records or nullptr
@@ -72,6 +73,7 @@ __global__ __launch_bounds__(THREADS, 1024 / THREADS) void k_sample_batch(const 
   __shared__ BatchStream s_st;
   __shared__ BatchGraph s_g;
   __shared__ uint64_t s_lo[WEDGE_MAX_BINS];
+  __shared__ GuideBin s_gtab[WEDGE_MAX_BINS];
   __shared__ uint32_t s_stats[STAT_N];
   __shared__ uint32_t s_q[WARPS][4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -101,11 +103,15 @@ __global__ __launch_bounds__(THREADS, 1024 / THREADS) void k_sample_batch(const 
     const BatchStream st = s_st;
     const BatchGraph g = s_g;
     const bool global = st.tag != 0;
-    for (int i = tid; i < (int)g.nb; i += THREADS) s_lo[i] = g.lo[i];
+    for (int i = tid; i < (int)g.nb; i += THREADS) {
+      s_lo[i] = g.lo[i];
+      s_gtab[i] = g.gtab[i];
+    }
     if (global)
       for (int i = tid; i < STAT_N; i += THREADS) s_stats[i] = 0;
     __syncthreads();
     const BinTable bt{s_lo, g.nb, g.pow2};
+    const GuideRange gr{s_gtab, global ? 2u : st.bin, global ? g.nb : st.bin + 1u};
     uint32_t q0 = 0, q1 = 0, q2 = 0, q3 = 0;
     const bool per_warp = st.mapping == WEDGE_MAP_WARP;
     const int step = per_warp ? WARPS : THREADS;
@@ -152,16 +158,21 @@ __global__ __launch_bounds__(THREADS, 1024 / THREADS) void k_sample_batch(const 
     } else {
       // two samples per thread in lockstep (j and j + step), so two chains of
       // dependent loads are in flight; an odd last one draws a copy of itself
-      for (int j = me; j < (int)tile_count; j += 2 * step) {
-        const bool two = j + step < (int)tile_count;
-        const uint64_t la = tile_first + (uint64_t)j, lb = two ? la + (uint64_t)step : la;
-        const uint64_t sa = st.first + la, sb = st.first + lb;
-        const Philox4 ra = philox4x32_10((uint32_t)sa, (uint32_t)(sa >> 32), st.bin, st.tag, g.seed_lo, g.seed_hi);
-        const Philox4 rb = philox4x32_10((uint32_t)sb, (uint32_t)(sb >> 32), st.bin, st.tag, g.seed_lo, g.seed_hi);
-        Wedge wa, wb;
-        draw_wedge_thread2(g.g, st.start, st.len, st.p, st.wbase, ra, rb, wa, wb);
-        record(wa, la);
-        if (two) record(wb, lb);
+      bool guess = true;
+      for (int j = me; j - lane < (int)tile_count; j += 2 * step) {
+        bool useful = guess;
+        if (j < (int)tile_count) {
+          const bool two = j + step < (int)tile_count;
+          const uint64_t la = tile_first + (uint64_t)j, lb = two ? la + (uint64_t)step : la;
+          const uint64_t sa = st.first + la, sb = st.first + lb;
+          const Philox4 ra = philox4x32_10((uint32_t)sa, (uint32_t)(sa >> 32), st.bin, st.tag, g.seed_lo, g.seed_hi);
+          const Philox4 rb = philox4x32_10((uint32_t)sb, (uint32_t)(sb >> 32), st.bin, st.tag, g.seed_lo, g.seed_hi);
+          Wedge wa, wb;
+          draw_wedge_thread2(g.g, gr, st.p, st.wbase, ra, rb, wa, wb, useful);
+          record(wa, la);
+          if (two) record(wb, lb);
+        }
+        guess = warp_guesses(guess, guess && !useful);
       }
     }
     {
@@ -329,8 +340,9 @@ extern "C" wedge_status wedge_batch_create(const wedge_request* reqs, int n_reqs
     if (sp.records && !want_glob) return bail(fail(WEDGE_EINVAL, "wedge_batch_create: request %d: records need the global stream", r));
     const wedge_bins_info& inf = q.bins->info;
     BatchGraph& G = graphs[(size_t)r];
-    G.g = GraphView{q.graph->off, q.graph->adj, q.bins->L, q.bins->W};
+    G.g = GraphView{q.graph->off, q.graph->adj, q.bins->L, q.bins->W, q.bins->guide, 1.0f / (float)q.graph->n};
     G.lo = q.bins->lo_dev;
+    G.gtab = q.bins->gtab;
     G.nb = inf.n_bins;
     G.pow2 = q.bins->pow2;
     G.seed_lo = (uint32_t)sp.seed;

@@ -451,6 +451,10 @@ struct BuildBuffers {
   }
 };
 
+// Entries to allocate for an adjacency array: whole 32-byte sectors, which
+// the closure search reads as a whole.
+size_t adj_alloc(int64_t n_adj) { return ((size_t)(n_adj > 0 ? n_adj : 1) + 7) & ~(size_t)7; }
+
 void free_graph(wedge_graph* g, cudaStream_t s) {
   if (!g) return;
   dfree(g->off, s);
@@ -563,7 +567,7 @@ extern "C" wedge_status wedge_graph_build(const int32_t* src, const int32_t* dst
   if ((st = dalloc_n(&bb.scalars, 4, s, "wedge_graph_build")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&g->off, (size_t)n_vertices + 1, s, "wedge_graph_build: offsets")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&g->deg, (size_t)n_vertices, s, "wedge_graph_build: degrees")) != WEDGE_OK) return bail(st);
-  if ((st = dalloc_n(&g->adj, (size_t)(nkeys > 0 ? nkeys : 1), s, "wedge_graph_build: adjacency")) != WEDGE_OK)
+  if ((st = dalloc_n(&g->adj, adj_alloc(nkeys), s, "wedge_graph_build: adjacency")) != WEDGE_OK)
     return bail(st);
   BUILD_TRY(cudaMemsetAsync(bb.derr, 0, 64 * sizeof(uint32_t), s), "wedge_graph_build");
   BUILD_TRY(cudaMemsetAsync(bb.scalars, 0, 4 * sizeof(int64_t), s), "wedge_graph_build");
@@ -851,7 +855,7 @@ extern "C" wedge_status wedge_graph_from_csr(const int64_t* off, const int32_t* 
   wedge_status st;
   if ((st = dalloc_n(&g->off, (size_t)n_vertices + 1, s, "wedge_graph_from_csr")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&g->deg, (size_t)n_vertices, s, "wedge_graph_from_csr")) != WEDGE_OK) return bail(st);
-  if ((st = dalloc_n(&g->adj, (size_t)(n_adj > 0 ? n_adj : 1), s, "wedge_graph_from_csr")) != WEDGE_OK) return bail(st);
+  if ((st = dalloc_n(&g->adj, adj_alloc(n_adj), s, "wedge_graph_from_csr")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&derr, 2, s, "wedge_graph_from_csr")) != WEDGE_OK) return bail(st);
   cudaError_t e = cudaMemcpyAsync(g->off, off, ((size_t)n_vertices + 1) * sizeof(int64_t), cudaMemcpyDefault, s);
   if (e == cudaSuccess && n_adj > 0)

@@ -19,6 +19,20 @@ struct wedge_graph {
   int32_t* deg;  // n
 };
 
+namespace wedge {
+
+// Where the centres of one bin lie in the guide over the wedge prefix W: the
+// bin's wedges are cut into cells of 2^shift, and guide[at + c] is the last j
+// with W[j] <= wlo + c 2^shift (guide[at + cells], one past the last cell: the
+// bin's last j). Written by k_bin_bounds, read by the samplers.
+struct GuideBin {
+  uint64_t wlo;    // W at the bin's start
+  uint32_t at;     // first guide entry
+  uint32_t shift;
+};
+
+}  // namespace wedge
+
 struct wedge_bins {
   int device;
   uint64_t graph_uid;
@@ -27,6 +41,8 @@ struct wedge_bins {
   int32_t* L;               // n_wedge_vertices
   uint64_t* W;              // n_wedge_vertices + 1
   uint64_t* lo_dev;         // bin table: n_bins entries
+  wedge::GuideBin* gtab;    // n_bins entries
+  uint32_t* guide;          // first vertices of the wedge cells
 };
 
 namespace wedge {

@@ -117,6 +117,7 @@ struct DrawArgs {
   const uint64_t* lo;
   uint32_t nb, pow2;
   uint32_t seed_lo, seed_hi;
+  float ids_inv;  // 1 / n
   unsigned long long* q_out;  // [n_streams][4]
 };
 
@@ -141,37 +142,42 @@ __global__ __launch_bounds__(ROUND_THREADS) void k_round_draw(DrawArgs a) {
   const BinTable bt{s_lo, a.nb, a.pow2};
   const uint64_t first = ((uint64_t)blockIdx.x - desc.tile_begin) * DRAW_TILE;
   uint32_t q0 = 0, q1 = 0, q2 = 0, q3 = 0;
+  bool guess = true;
   for (int it = 0; it < DRAW_PER_THREAD; ++it) {
     const uint64_t local = first + (uint64_t)it * ROUND_THREADS + tid;
-    if (local >= desc.count) break;
-    const uint64_t s = desc.qbase + local;
-    int64_t lo = desc.start, hi = desc.start + desc.len;  // Q[lo] <= s < Q[hi]
-    while (hi - lo > 1) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
-      if (__ldg(a.Q + mid) <= s) lo = mid; else hi = mid;
+    if (local - lane >= desc.count) break;  // the whole warp
+    bool useful = guess;
+    if (local < desc.count) {
+      const uint64_t s = desc.qbase + local;
+      int64_t lo = desc.start, hi = desc.start + desc.len;  // Q[lo] <= s < Q[hi]
+      while (hi - lo > 1) {
+        const int64_t mid = lo + ((hi - lo) >> 1);
+        if (__ldg(a.Q + mid) <= s) lo = mid; else hi = mid;
+      }
+      const uint64_t l = s - __ldg(a.Q + lo);  // the l-th wedge at this centre
+      const int32_t v0 = __ldg(a.L + lo);
+      const int64_t o0 = __ldg(a.off + v0);
+      const int64_t d0 = __ldg(a.off + v0 + 1) - o0;
+      const Philox4 r = philox4x32_10((uint32_t)l, (uint32_t)(l >> 32), (uint32_t)v0, TAG_DRAW, a.seed_lo, a.seed_hi);
+      const uint64_t dm1 = (uint64_t)(d0 - 1);
+      const uint64_t u = mulhi64((uint64_t)r.r0 | ((uint64_t)r.r1 << 32), (uint64_t)d0 * dm1);
+      const uint64_t i = div_small(u, dm1);
+      const uint64_t jp = u - i * dm1;
+      const uint64_t jj = jp + (jp >= i ? 1ULL : 0ULL);
+      const int32_t v1 = __ldg(a.adj + o0 + (int64_t)i);
+      const int32_t v2 = __ldg(a.adj + o0 + (int64_t)jj);
+      const int64_t o1 = __ldg(a.off + v1), d1 = __ldg(a.off + v1 + 1) - o1;
+      const int64_t o2 = __ldg(a.off + v2), d2 = __ldg(a.off + v2 + 1) - o2;
+      if (!closed_wedge(a.adj, v1, v2, o1, d1, o2, d2, a.ids_inv, useful)) {
+        q0 += 1;
+      } else {
+        const uint32_t cls = 1u + (bin_of(bt, (uint64_t)d1) == desc.bin) + (bin_of(bt, (uint64_t)d2) == desc.bin);
+        q1 += cls == 1u;
+        q2 += cls == 2u;
+        q3 += cls == 3u;
+      }
     }
-    const uint64_t l = s - __ldg(a.Q + lo);  // the l-th wedge at this centre
-    const int32_t v0 = __ldg(a.L + lo);
-    const int64_t o0 = __ldg(a.off + v0);
-    const int64_t d0 = __ldg(a.off + v0 + 1) - o0;
-    const Philox4 r = philox4x32_10((uint32_t)l, (uint32_t)(l >> 32), (uint32_t)v0, TAG_DRAW, a.seed_lo, a.seed_hi);
-    const uint64_t dm1 = (uint64_t)(d0 - 1);
-    const uint64_t u = mulhi64((uint64_t)r.r0 | ((uint64_t)r.r1 << 32), (uint64_t)d0 * dm1);
-    const uint64_t i = u / dm1;
-    const uint64_t jp = u - i * dm1;
-    const uint64_t jj = jp + (jp >= i ? 1ULL : 0ULL);
-    const int32_t v1 = __ldg(a.adj + o0 + (int64_t)i);
-    const int32_t v2 = __ldg(a.adj + o0 + (int64_t)jj);
-    const int64_t o1 = __ldg(a.off + v1), d1 = __ldg(a.off + v1 + 1) - o1;
-    const int64_t o2 = __ldg(a.off + v2), d2 = __ldg(a.off + v2 + 1) - o2;
-    if (!closed_wedge(a.adj, v1, v2, o1, d1, o2, d2)) {
-      q0 += 1;
-    } else {
-      const uint32_t cls = 1u + (bin_of(bt, (uint64_t)d1) == desc.bin) + (bin_of(bt, (uint64_t)d2) == desc.bin);
-      q1 += cls == 1u;
-      q2 += cls == 2u;
-      q3 += cls == 3u;
-    }
+    guess = warp_guesses(guess, guess && !useful);
   }
   const uint32_t w0 = __reduce_add_sync(FULL_MASK, q0), w1 = __reduce_add_sync(FULL_MASK, q1);
   const uint32_t w2 = __reduce_add_sync(FULL_MASK, q2), w3 = __reduce_add_sync(FULL_MASK, q3);
@@ -305,6 +311,7 @@ wedge_status sample_rounding(const wedge_graph* g, const wedge_bins* b, uint64_t
   da.streams = d_streams;
   da.n_streams = (int)streams.size();
   da.off = g->off;
+  da.ids_inv = 1.0f / (float)g->n;
   da.adj = g->adj;
   da.L = b->L;
   da.Q = Q;

@@ -47,6 +47,8 @@ struct SampleArgs {
   const int32_t* adj;
   const int32_t* L;
   const uint64_t* W;
+  const uint32_t* guide;
+  const GuideBin* gtab;
   const uint64_t* lo;
   uint32_t nb;
   uint32_t pow2;
@@ -62,6 +64,7 @@ __global__ __launch_bounds__(SAMPLE_THREADS) void k_sample(SampleArgs a) {
   __shared__ StreamDesc s_desc;
   __shared__ int s_stream;
   __shared__ uint64_t s_lo[WEDGE_MAX_BINS];
+  __shared__ GuideBin s_gtab[WEDGE_MAX_BINS];
   __shared__ uint32_t s_stats[WEDGE_STAT_BINS * WEDGE_STAT_BINS];
   __shared__ uint32_t s_q[SAMPLE_THREADS / 32][4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -74,54 +77,65 @@ __global__ __launch_bounds__(SAMPLE_THREADS) void k_sample(SampleArgs a) {
     s_stream = lo;
     s_desc = a.streams[lo];
   }
-  for (int i = tid; i < (int)a.nb; i += SAMPLE_THREADS) s_lo[i] = a.lo[i];
+  for (int i = tid; i < (int)a.nb; i += SAMPLE_THREADS) {
+    s_lo[i] = a.lo[i];
+    s_gtab[i] = a.gtab[i];
+  }
   for (int i = tid; i < WEDGE_STAT_BINS * WEDGE_STAT_BINS; i += SAMPLE_THREADS) s_stats[i] = 0;
   __syncthreads();
   const StreamDesc desc = s_desc;
   const BinTable bt{s_lo, a.nb, a.pow2};
-  const GraphView gv{a.off, a.adj, a.L, a.W, a.n, a.n_adj, a.n_L, a.err};
+  const GraphView gv{a.off, a.adj, a.L, a.W, a.guide, 1.0f / (float)a.n, a.n, a.n_adj, a.n_L, a.err};
   const bool global = desc.tag != 0;
+  const GuideRange gr{s_gtab, global ? 2u : desc.bin, global ? a.nb : desc.bin + 1u};
   const uint64_t first = ((uint64_t)blockIdx.x - desc.tile_begin) * SAMPLE_TILE;
   uint32_t q0 = 0, q1 = 0, q2 = 0, q3 = 0;
+  bool guess = true;
   for (int j = 0; j < SAMPLE_PER_THREAD; ++j) {
     const uint64_t local = first + (uint64_t)j * SAMPLE_THREADS + tid;
-    if (local >= desc.k) break;
-    const uint64_t s = desc.first + local;  // sample index in the stream
-    const Philox4 r = philox4x32_10((uint32_t)s, (uint32_t)(s >> 32), desc.bin, desc.tag, a.seed_lo, a.seed_hi);
-    const Wedge w = draw_wedge_thread(gv, desc.start, desc.len, desc.p, desc.wbase, r);
-    const int32_t v0 = w.v0, v1 = w.v1, v2 = w.v2;
-    const int64_t d0 = w.d0, d1 = w.d1, d2 = w.d2;
-    const bool closed = w.closed;
-    if (!global) {
-      if (!closed) {
-        q0 += 1;
+    if (local - lane >= desc.k) break;  // the whole warp
+    bool lost = false;
+    if (local < desc.k) {
+      const uint64_t s = desc.first + local;  // sample index in the stream
+      const Philox4 r = philox4x32_10((uint32_t)s, (uint32_t)(s >> 32), desc.bin, desc.tag, a.seed_lo, a.seed_hi);
+      bool useful = guess;
+      const Wedge w = draw_wedge_thread(gv, gr, desc.p, desc.wbase, r, useful);
+      lost = guess && !useful;
+      const int32_t v0 = w.v0, v1 = w.v1, v2 = w.v2;
+      const int64_t d0 = w.d0, d1 = w.d1, d2 = w.d2;
+      const bool closed = w.closed;
+      if (!global) {
+        if (!closed) {
+          q0 += 1;
+        } else {
+          const uint32_t cls = 1u + (bin_of(bt, (uint64_t)d1) == desc.bin) + (bin_of(bt, (uint64_t)d2) == desc.bin);
+          q1 += cls == 1u;
+          q2 += cls == 2u;
+          q3 += cls == 3u;
+        }
       } else {
-        const uint32_t cls = 1u + (bin_of(bt, (uint64_t)d1) == desc.bin) + (bin_of(bt, (uint64_t)d2) == desc.bin);
-        q1 += cls == 1u;
-        q2 += cls == 2u;
-        q3 += cls == 3u;
-      }
-    } else {
-      // one bin of every degree: a closed wedge has all three vertices in it (q3)
-      q0 += closed ? 0u : 1u;
-      q3 += closed ? 1u : 0u;
-      if (closed) {
-        const int64_t dmin = min(d0, min(d1, d2)), dmax = max(d0, max(d1, d2));
-        atomicAdd(&s_stats[stat_bin((uint64_t)dmin) * WEDGE_STAT_BINS + stat_bin((uint64_t)dmax)], 1u);
-      }
-      if (a.records) {
-        wedge_record rec;
-        rec.v0 = v0;
-        rec.v1 = v1;
-        rec.v2 = v2;
-        rec.closed = closed ? 1 : 0;
-        rec.d0 = (int32_t)d0;
-        rec.d1 = (int32_t)d1;
-        rec.d2 = (int32_t)d2;
-        rec.reserved = 0;
-        a.records[local] = rec;
+        // one bin of every degree: a closed wedge has all three vertices in it (q3)
+        q0 += closed ? 0u : 1u;
+        q3 += closed ? 1u : 0u;
+        if (closed) {
+          const int64_t dmin = min(d0, min(d1, d2)), dmax = max(d0, max(d1, d2));
+          atomicAdd(&s_stats[stat_bin((uint64_t)dmin) * WEDGE_STAT_BINS + stat_bin((uint64_t)dmax)], 1u);
+        }
+        if (a.records) {
+          wedge_record rec;
+          rec.v0 = v0;
+          rec.v1 = v1;
+          rec.v2 = v2;
+          rec.closed = closed ? 1 : 0;
+          rec.d0 = (int32_t)d0;
+          rec.d1 = (int32_t)d1;
+          rec.d2 = (int32_t)d2;
+          rec.reserved = 0;
+          a.records[local] = rec;
+        }
       }
     }
+    guess = warp_guesses(guess, lost);
   }
   {
     const uint32_t w0 = __reduce_add_sync(FULL_MASK, q0), w1 = __reduce_add_sync(FULL_MASK, q1);
@@ -167,7 +181,8 @@ __global__ __launch_bounds__(256) void k_classify(const int64_t* __restrict__ of
     const int64_t o2 = off[v2], d2 = off[v2 + 1] - o2;
     const uint32_t b = bin_of(bt, (uint64_t)d0);
     uint8_t cls = 0;
-    if (closed_wedge(adj, v1, v2, o1, d1, o2, d2))
+    bool guess = true;
+    if (closed_wedge(adj, v1, v2, o1, d1, o2, d2, 1.0f / (float)n, guess))
       cls = (uint8_t)(1u + (bin_of(bt, (uint64_t)d1) == b) + (bin_of(bt, (uint64_t)d2) == b));
     q[w] = cls;
   }
@@ -269,6 +284,8 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
   a.adj = g->adj;
   a.L = b->L;
   a.W = b->W;
+  a.guide = b->guide;
+  a.gtab = b->gtab;
   a.lo = b->lo_dev;
   a.nb = inf.n_bins;
   a.pow2 = b->pow2;

@@ -49,6 +49,8 @@ struct KeyArgs {
   const int32_t* adj;
   const int32_t* L;
   const uint64_t* W;
+  const uint32_t* guide;
+  const GuideBin* gtab;
   const uint64_t* lo;
   uint32_t nb, pow2;
   uint32_t seed_lo, seed_hi;
@@ -59,6 +61,7 @@ struct KeyArgs {
 __global__ __launch_bounds__(KEY_THREADS) void k_sample_keys(KeyArgs a) {
   __shared__ KeyStream s_desc;
   __shared__ uint64_t s_lo[WEDGE_MAX_BINS];
+  __shared__ GuideBin s_gtab[WEDGE_MAX_BINS];
   const int tid = threadIdx.x;
   if (tid == 0) {
     int lo = 0, hi = a.n_streams;  // last stream with tile_begin <= blockIdx.x
@@ -68,11 +71,15 @@ __global__ __launch_bounds__(KEY_THREADS) void k_sample_keys(KeyArgs a) {
     }
     s_desc = a.streams[lo];
   }
-  for (int i = tid; i < (int)a.nb; i += KEY_THREADS) s_lo[i] = a.lo[i];
+  for (int i = tid; i < (int)a.nb; i += KEY_THREADS) {
+    s_lo[i] = a.lo[i];
+    s_gtab[i] = a.gtab[i];
+  }
   __syncthreads();
   const KeyStream desc = s_desc;
   const BinTable bt{s_lo, a.nb, a.pow2};
-  const GraphView gv{a.off, a.adj, a.L, a.W};
+  const GraphView gv{a.off, a.adj, a.L, a.W, a.guide, 0.0f};
+  const GuideRange gr{s_gtab, desc.bin, desc.bin + 1u};
   const uint64_t first = ((uint64_t)blockIdx.x - desc.tile_begin) * KEY_TILE;
   for (int j = 0; j < KEY_PER_THREAD; ++j) {
     const uint64_t local = first + (uint64_t)j * KEY_THREADS + tid;
@@ -80,7 +87,7 @@ __global__ __launch_bounds__(KEY_THREADS) void k_sample_keys(KeyArgs a) {
     const uint64_t s = desc.first + local;
     const Philox4 r = philox4x32_10((uint32_t)s, (uint32_t)(s >> 32), desc.bin, 0u, a.seed_lo, a.seed_hi);
     int64_t o1, o2;
-    const Wedge w = draw_pair_thread(gv, desc.start, desc.len, desc.p, desc.wbase, r, o1, o2);
+    const Wedge w = draw_pair_thread(gv, gr, desc.p, desc.wbase, r, o1, o2);
     const uint32_t cls = 1u + (bin_of(bt, (uint64_t)w.d1) == desc.bin) + (bin_of(bt, (uint64_t)w.d2) == desc.bin);
     const bool first_row = w.d1 < w.d2 || (w.d1 == w.d2 && w.v1 < w.v2);  // search the smaller (degree, id) row
     const uint64_t x = (uint64_t)(first_row ? w.v1 : w.v2), y = (uint64_t)(first_row ? w.v2 : w.v1);
@@ -223,6 +230,8 @@ wedge_status sample_sorted_closure(const wedge_graph* g, const wedge_bins* b, ui
   ka.adj = g->adj;
   ka.L = b->L;
   ka.W = b->W;
+  ka.guide = b->guide;
+  ka.gtab = b->gtab;
   ka.lo = b->lo_dev;
   ka.nb = nb;
   ka.pow2 = b->pow2;
