@@ -106,13 +106,14 @@ size_t scan_scratch_bytes(int64_t n);
 // If maxv != nullptr, atomicMax(maxv, max input) (inputs interpreted as int32).
 wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, int32_t* maxv, void* scratch,
                              uint32_t* derr, cudaStream_t s);
-wedge_status scan_u32_to_i64(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
-                             cudaStream_t s);
-wedge_status scan_u64_to_u64(const uint64_t* in, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
-                             cudaStream_t s);
 // out[i] = sum in[0..i) for i < n and out[n] = the total (out holds n + 1).
+wedge_status scan_u32_with_total(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
+                                 cudaStream_t s);
 wedge_status scan_u64_with_total(const uint64_t* in, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s, const char* name);
+// The same over C(deg[i], 2), deg[i] >= 0.
+wedge_status scan_pairs_with_total(const int32_t* deg, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
+                                   cudaStream_t s, const char* name);
 
 // Per-bin samples allocated per vertex by probabilistic rounding and drawn per
 // centre (rounding.cu). k_of_bin: host, n_bins budgets. Fills out->k_b (the

@@ -23,6 +23,12 @@ constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
 __device__ __forceinline__ int pad(int i) { return i + (i >> 5); }
 
+// A degree that counts as its C(d,2) wedges.
+struct Pairs {
+  int32_t d;
+  __device__ __forceinline__ operator uint64_t() const { return (uint64_t)d * (uint64_t)(d - 1) / 2ULL; }
+};
+
 // CHECK: inputs must be >= 0 (DERR_NEGATIVE otherwise) and every prefix must
 // fit the look-back words' 58-bit value field (DERR_OVERFLOW otherwise).
 template <typename Tin, typename Tout, bool CHECK = false>
@@ -58,8 +64,8 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restric
     if (g < n) {
       const Tin x = in[g];
       v = (Tout)x;
-      if (maxv) local_max = max(local_max, (int32_t)x);
-      if (CHECK && x < (Tin)0) atomicOr(err, DERR_NEGATIVE);
+      if (maxv) local_max = max(local_max, (int32_t)v);
+      if (CHECK && v < (Tout)0) atomicOr(err, DERR_NEGATIVE);
     }
     s_buf[pad(idx)] = v;
   }
@@ -155,19 +161,20 @@ wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t
   return run_scan<int32_t, int64_t>(in, out, n, total, maxv, scratch, derr, s, "scan_degrees");
 }
 
-wedge_status scan_u32_to_i64(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
-                             cudaStream_t s) {
-  return run_scan<uint32_t, int64_t>(in, out, n, nullptr, nullptr, scratch, derr, s, "scan_bin_counts");
-}
-
-wedge_status scan_u64_to_u64(const uint64_t* in, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
-                             cudaStream_t s) {
-  return run_scan<uint64_t, uint64_t>(in, out, n, nullptr, nullptr, scratch, derr, s, "scan_bin_wedges");
+wedge_status scan_u32_with_total(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
+                                 cudaStream_t s) {
+  return run_scan<uint32_t, int64_t>(in, out, n, out + n, nullptr, scratch, derr, s, "scan_bin_counts");
 }
 
 wedge_status scan_u64_with_total(const uint64_t* in, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s, const char* name) {
   return run_scan<uint64_t, uint64_t>(in, out, n, out + n, nullptr, scratch, derr, s, name);
+}
+
+wedge_status scan_pairs_with_total(const int32_t* deg, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
+                                   cudaStream_t s, const char* name) {
+  return run_scan<Pairs, uint64_t>(reinterpret_cast<const Pairs*>(deg), out, n, out + n, nullptr, scratch, derr, s,
+                                   name);
 }
 
 // ---------------------------------------------------------------------------
