@@ -19,6 +19,7 @@ loudly; there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 
 import numpy as np
@@ -411,6 +412,14 @@ def bin(graph: Graph, tau: int = 1, omega: int = 2, stream=None) -> Bins:  # noq
     return Bins(h.value, graph)
 
 
+def _words(struct, field, *shape):
+    """A copy of a struct's uint64 array field (or of its first rows), as numpy.
+    Taken from the struct's memory at once: element by element through ctypes
+    the statistics histogram alone takes longer than a small sampling kernel."""
+    d = getattr(type(struct), field)
+    return np.frombuffer(struct, np.uint64, math.prod(shape), d.offset).reshape(shape).copy()
+
+
 class Counts:
     """Host copy of wedge_counts as numpy arrays."""
 
@@ -418,14 +427,14 @@ class Counts:
         self.raw = c
         nb = c.n_bins
         self.n_bins = nb
-        self.k_b = np.array(c.k_b[:nb], np.uint64)
-        self.q = np.array([list(c.q[i]) for i in range(nb)], np.uint64).reshape(nb, 4)
-        self.n_b = np.array(c.n_b[:nb], np.uint64)
-        self.p_b = np.array(c.p_b[:nb], np.uint64)
+        self.k_b = _words(c, "k_b", nb)
+        self.q = _words(c, "q", nb, 4)
+        self.n_b = _words(c, "n_b", nb)
+        self.p_b = _words(c, "p_b", nb)
         self.p_total = int(c.p_total)
         self.k_global = int(c.k_global)
         self.closed_global = int(c.closed_global)
-        self.stats = np.array([list(c.stats[i]) for i in range(STAT_BINS)], np.uint64)
+        self.stats = _words(c, "stats", STAT_BINS, STAT_BINS)
 
     def counts_matrix(self):
         """(n_bins, 5) = (k_b, q0, q1, q2, q3), the oracle's layout."""
@@ -486,9 +495,8 @@ def exact(graph: Graph, bins: Bins, t_i=None, stream=None) -> dict:
             raise ValueError("t_i needs n_vertices entries")
     _check(lib.wedge_exact(graph.handle, bins.handle, pt, _stream_handle(stream), ctypes.byref(out)))
     nb = out.n_bins
-    pbq = np.array([list(out.pbq[i]) for i in range(nb)], np.uint64).reshape(nb, 4)
-    return {"triangles": int(out.triangles), "p_total": int(out.p_total), "p_b": np.array(out.p_b[:nb], np.uint64),
-            "pbq": pbq}
+    return {"triangles": int(out.triangles), "p_total": int(out.p_total), "p_b": _words(out, "p_b", nb),
+            "pbq": _words(out, "pbq", nb, 4)}
 
 
 BOX_FIELDS = ("count", "min", "q1", "median", "q3", "max", "whisker_lo", "whisker_hi", "outliers")
@@ -509,9 +517,9 @@ def triangle_stats(graph: Graph, bins: Bins, seed: int, k: int, records=None, st
             raise ValueError("records needs k * 8 int32 entries")
     _check(lib.wedge_triangle_stats(graph.handle, bins.handle, seed, k, pr, _stream_handle(stream),
                                     ctypes.byref(out)))
-    box = np.array([[getattr(out.box[i], f) for f in BOX_FIELDS] for i in range(STAT_BINS)], np.uint64)
+    box = _words(out, "box", STAT_BINS, len(BOX_FIELDS))  # (a box is its fields, in order)
     return {"k": int(out.k), "closed": int(out.closed), "box": box, "ratio_q": np.array(out.ratio_q[:], np.float64),
-            "hist": np.array([list(out.hist[i]) for i in range(STAT_BINS)], np.uint64)}
+            "hist": _words(out, "hist", STAT_BINS, STAT_BINS)}
 
 
 NOALLOC_MAX_VERTICES = 536870912
