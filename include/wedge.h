@@ -477,8 +477,8 @@ WEDGE_API wedge_status wedge_classify(const wedge_graph* g, const wedge_bins* b,
 /* --------------------------------------------------------------------------
  * Exact counts (Sec. 2.1, 2.2): the quantities the sampler estimates, by
  * enumerating every triangle once on the device (each edge oriented from
- * the smaller to the larger (degree, id); the oriented rows of an edge's two
- * endpoints are intersected). For every bin b: p_b (wedges centred in b) and
+ * the smaller to the larger (degree, id); for each edge (u, v), the rest of
+ * u's oriented row is looked up in v's). For every bin b: p_b (wedges centred in b) and
  * pbq[b][q], the closed wedges centred in b whose two endpoints include
  * q - 1 vertices of b (q = 1, 2, 3; Alg. Phase 4c's classes), with
  * pbq[b][0] = p_b - pbq[b][1] - pbq[b][2] - pbq[b][3] (open wedges). Then
@@ -486,8 +486,9 @@ WEDGE_API wedge_status wedge_classify(const wedge_graph* g, const wedge_bins* b,
  * global c = 3t/p (Eq. (CC)).
  *   t_i: optional device uint64[n_vertices] receiving the closed wedges
  *     centred at each vertex (triangles at i); NULL skips them.
- *   Synchronises s. Needs about 4m + 12n bytes of device memory beyond the
- *   graph (m undirected edges).
+ *   Synchronises s. Needs about 4m + 44n bytes of device memory beyond the
+ *   graph (m undirected edges), and about 22 bytes for each of m, but at most
+ *   2^27 (or the largest degree, if that is more), edges.
  *   Errors: EINVAL for NULL handles or bins of another graph; ENOMEM;
  *   ECUDA; ETIMEOUT (a bounded look-back wait gave up).
  * ------------------------------------------------------------------------ */

@@ -3,25 +3,29 @@
 // The quantities sampling estimates (Sec. 2.1, 2.2): t, t_i and p_{b,q}, the
 // closed wedges centred in bin b whose endpoints have q - 1 vertices in b
 // (Alg. Phase 4c's classes), so that c_b = (p_{b,1} + p_{b,2} + p_{b,3}) / p_b.
-// The paper obtains them by enumeration on a CPU; here:
-//   1. k_orient: every adjacency entry (u, v) is kept iff (d_v, v) > (d_u, u)
-//      (degree order); kept entries are compacted in order (one pass,
-//      decoupled look-back) into the oriented rows adj+, which stay sorted,
-//      and out-degrees are counted per row;
-//   2. a scan of the out-degrees gives the oriented row offsets;
-//   3. k_tri_hash_warp: one warp per vertex u with 2 <= d+(u) <= 128 puts
-//      N+(u) into a hash table in shared memory and streams the rows N+(v) of
-//      all v in N+(u) as one flattened list split across the lanes; each
-//      entry w found in the table closes the triangle u < v < w, counted
-//      exactly once. Vertices with longer oriented rows are queued for
-//      k_tri_hash_cta (one CTA per vertex by ticket; 2048 table slots for rows
-//      up to 1024, 8192 beyond). Table entries carry their vertex's bin, and
-//      closed wedges at u and v are tallied in registers, so a found
-//      triangle costs one shared-memory atomic.
-//      Degree order bounds every d+ by sqrt(2m), so the streamed work is the
-//      number of oriented wedges (u, v, w). Each triangle adds one closed
-//      wedge per vertex to p_{bin(centre), class}; CTAs tally in shared
-//      memory and flush once.
+// The paper obtains them by enumeration on a CPU; here vertices are ranked by
+// (degree, id), N+(u) are u's neighbours of higher rank, and every triangle
+// u < v < w is found once, as the edge (u, v) and a w after v in N+(u) that is
+// in N+(v):
+//   1. ranks: a radix sort of the degrees;
+//   2. exact_orient: counts, per vertex, the neighbours of lower and of higher
+//      rank; scans give the in-lists (the u of every v) and the rows N+;
+//   3. exact_edges: the oriented edges by v, in rank order; a stable radix sort
+//      by u then yields the rows N+(u) in rank order, and exact_rows records
+//      for every edge of an in-list how many entries of N+(u) come after v;
+//   4. exact_hash_warp / exact_hash_cta: for every v, a hash table of N+(v) in
+//      shared memory, and the tails of N+(u) after v streamed against it for
+//      all u of v's in-list, a warp per tail.
+// The tails of all edges are the pairs of N+(u), sum C(d+, 2); streaming the
+// whole N+(v) of every v in N+(u) against a table of N+(u) instead reads 3.6
+// times as many entries (Kronecker scale 20: 4.4e9 against 1.2e9; 34.4 ms in
+// all that way, 5.2 ms this way; scale 24: 1.11 s and 0.25 s). The count is
+// bound by instructions and, where N+ rows are short, by the chain of loads per
+// vertex; graphs with next to no triangles pay the ranks and the sort for
+// nothing (uniform, 16 M edges: 2.1 and 2.3 ms).
+// Vertices are taken in groups of at most GROUP_EDGES in-edges, highest ranks
+// first, so that the edges' scratch is bounded; rows fill from their ends, and
+// the tails that a group reads are there when it is counted.
 #include <string.h>
 
 #include <algorithm>
@@ -34,14 +38,10 @@
 namespace wedge {
 namespace {
 
-constexpr int OR_THREADS = 256;
-constexpr int OR_ITEMS = 16;
-constexpr int OR_TILE = OR_THREADS * OR_ITEMS;
-constexpr int TC_THREADS = 256;
-
-__device__ __forceinline__ bool above(int32_t dv, int32_t v, int32_t du, int32_t u) {
-  return dv > du || (dv == du && v > u);
-}
+constexpr int EX_THREADS = 256;
+constexpr int EX_WARPS = EX_THREADS / 32;
+constexpr int OR_STEPS = 16;                            // 32-entry steps of a warp at most
+constexpr int64_t GROUP_EDGES = int64_t(1) << 27;       // in-edges of a group (unless one vertex has more)
 
 // Largest u in [0, n) with off[u] <= e (off ascending, off[0] = 0 <= e).
 __device__ __forceinline__ int32_t row_of(const int64_t* __restrict__ off, int32_t n, int64_t e) {
@@ -71,453 +71,551 @@ __device__ __forceinline__ int32_t next_row(const int64_t* __restrict__ off, int
   return lo;
 }
 
+__global__ __launch_bounds__(EX_THREADS) void k_degree_keys(const int32_t* __restrict__ deg, int32_t n,
+                                                            uint64_t* __restrict__ keys) {
+  const int64_t v = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
+  if (v < n) keys[v] = ((uint64_t)(uint32_t)deg[v] << 32) | (uint64_t)v;
+}
+
+// order[r] = the vertex of rank r, rank its inverse.
+__global__ __launch_bounds__(EX_THREADS) void k_ranks(const uint64_t* __restrict__ sorted, int32_t n,
+                                                      int32_t* __restrict__ order, int32_t* __restrict__ rank) {
+  const int64_t r = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
+  if (r < n) {
+    const int32_t v = (int32_t)(uint32_t)sorted[r];
+    order[r] = v;
+    rank[v] = (int32_t)r;
+  }
+}
+
+// The ranks of few vertices, by comparing each with all: one launch instead of
+// a sort's eight (9 us for 256 vertices, some 25 us less than the sort; at
+// 8,192 the comparisons take about as long).
+constexpr int32_t FEW_VERTICES = 8192;
+
+__global__ __launch_bounds__(EX_THREADS) void k_ranks_few(const int32_t* __restrict__ deg, int32_t n,
+                                                          int32_t* __restrict__ order, int32_t* __restrict__ rank) {
+  // a CTA takes 32 vertices, one a lane; its warps share out the others
+  __shared__ int32_t s_sum[EX_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t v = blockIdx.x * 32 + lane;
+  const int32_t d = v < n ? __ldg(deg + v) : 0;
+  int32_t less = 0;
+  for (int32_t x0 = warp * 32; x0 < n; x0 += EX_THREADS) {
+    const int32_t mine = x0 + lane < n ? __ldg(deg + x0 + lane) : INT32_MAX;
+#pragma unroll 8
+    for (int j = 0; j < 32; ++j) {
+      const int32_t o = __shfl_sync(FULL_MASK, mine, j);
+      less += o < d || (o == d && x0 + j < v);
+    }
+  }
+  s_sum[warp][lane] = less;
+  __syncthreads();
+  if (warp == 0 && v < n) {
+    int32_t r = 0;
+    for (int w = 0; w < EX_WARPS; ++w) r += s_sum[w][lane];
+    rank[v] = r;
+    order[r] = v;
+  }
+}
+
 struct OrientArgs {
   const int64_t* off;
   const int32_t* adj;
-  const int32_t* deg;
+  const int32_t* rank;
   int32_t n;
   int64_t n_adj;
-  uint64_t* status;
-  uint32_t* tile_ctr;
-  uint32_t* err;
-  int32_t* adjp;   // kept entries, in order
-  int32_t* dplus;  // out-degree per vertex (zeroed)
+  int steps;              // 32-entry steps of a warp
+  int32_t* lower;         // by rank: neighbours of lower rank (EMIT: taken so far)
+  int32_t* higher;        // by rank: neighbours of higher rank
+  const int64_t* in_off;  // EMIT: in-list offsets by rank
+  int32_t r0, r1;         // EMIT: the group's ranks
+  uint64_t* keys;         // EMIT: u << 32 | place in the group's in-lists
+  uint32_t* v_of;         // EMIT: v by place
+  uint64_t edges;         // EMIT: places
 };
 
-__global__ __launch_bounds__(OR_THREADS) void k_orient(OrientArgs a) {
-  __shared__ uint32_t s_tile;
-  __shared__ uint32_t s_wsum[OR_THREADS / 32];
-  __shared__ uint64_t s_excl;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_tile = atomicAdd(a.tile_ctr, 1u);
-  __syncthreads();
-  const int64_t tile = s_tile;
-  const int64_t base = tile * OR_TILE + (int64_t)tid * OR_ITEMS;
-  // pass 1: keep flags of this thread's 16 consecutive entries
-  uint32_t keep = 0;
-  int32_t u0 = 0;
-  if (base < a.n_adj) {
-    u0 = row_of(a.off, a.n, base);
-    int32_t u = u0;
-    int64_t row_end = __ldg(a.off + u + 1);
-    int32_t du = __ldg(a.deg + u);
-    for (int i = 0; i < OR_ITEMS; ++i) {
-      const int64_t e = base + i;
-      if (e >= a.n_adj) break;
-      if (e >= row_end) {
-        u = next_row(a.off, a.n, u, e);
-        row_end = __ldg(a.off + u + 1);
-        du = __ldg(a.deg + u);
+// Every adjacency entry (v, u) with rank(u) < rank(v): counted for both ends,
+// or (EMIT) given a place in v's in-list, if v is of the group. A warp takes up to
+// 512 consecutive entries, 32 at a time; the lanes of a row share one atomic.
+template <bool EMIT>
+__global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t le = lanemask_lt() | (1u << lane);
+  const int64_t base = ((int64_t)blockIdx.x * EX_WARPS + (threadIdx.x >> 5)) * (32 * a.steps);
+  if (base >= a.n_adj) return;
+  int32_t x = row_of(a.off, a.n, min(base + lane, a.n_adj - 1)), rx = __ldg(a.rank + x);
+  for (int i = 0; i < a.steps; ++i) {
+    const int64_t e = base + i * 32 + lane;
+    if (e - lane >= a.n_adj) break;  // the whole warp
+    bool keep = false;
+    int32_t ry = 0;
+    if (e < a.n_adj) {
+      if (e >= __ldg(a.off + x + 1)) {
+        x = next_row(a.off, a.n, x, e);
+        rx = __ldg(a.rank + x);
       }
-      const int32_t v = __ldg(a.adj + e);
-      if (above(__ldg(a.deg + v), v, du, u)) keep |= 1u << i;
+      ry = __ldg(a.rank + __ldcs(a.adj + e));
+      keep = ry < rx && (!EMIT || (rx >= a.r0 && rx < a.r1));
     }
-  }
-  const uint32_t cnt = __popc(keep);
-  // block exclusive scan of counts
-  uint32_t incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(FULL_MASK, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) s_wsum[warp] = incl;
-  __syncthreads();
-  uint32_t wpre = 0, tile_total = 0;
-#pragma unroll
-  for (int w = 0; w < OR_THREADS / 32; ++w) {
-    if (w < warp) wpre += s_wsum[w];
-    tile_total += s_wsum[w];
-  }
-  if (warp == 0) {
-    uint64_t* st = a.status + tile;
-    uint64_t excl = 0;
-    if (tile == 0) {
-      if (lane == 0) st_relaxed(st, lb_pack(1, LB_INC, tile_total));
+    const uint32_t kept = __ballot_sync(FULL_MASK, keep);
+    if (kept == 0) continue;
+    const int32_t before = __shfl_up_sync(FULL_MASK, rx, 1);
+    const uint32_t starts = __ballot_sync(FULL_MASK, lane == 0 || before != rx);
+    const int start = 31 - __clz(starts & le);
+    const uint32_t later = starts & ~le;
+    const uint32_t run = (later ? (1u << (__ffs(later) - 1)) - 1u : FULL_MASK) & ~((1u << start) - 1u);
+    const uint32_t mine = kept & run;  // the row's kept entries among these 32
+    int32_t at = 0;
+    if (lane == start && mine) at = atomicAdd(a.lower + rx, __popc(mine));
+    if (!EMIT) {
+      if (keep) atomicAdd(a.higher + ry, 1);
     } else {
-      if (lane == 0) st_relaxed(st, lb_pack(1, LB_AGG, tile_total));
-      excl = lookback_warp(a.status, tile, 1, a.err, lane);
-      if (lane == 0) st_relaxed(st, lb_pack(1, LB_INC, excl + tile_total));
-    }
-    if (lane == 0) s_excl = excl;
-  }
-  __syncthreads();
-  if (keep == 0) return;
-  // pass 2: write kept entries in order; count them per row
-  uint64_t pos = s_excl + wpre + incl - cnt;
-  int32_t u = u0;
-  int64_t row_end = __ldg(a.off + u + 1);
-  uint32_t run = 0;
-  for (int i = 0; i < OR_ITEMS; ++i) {
-    const int64_t e = base + i;
-    if (e >= a.n_adj) break;
-    if (e >= row_end) {
-      if (run) atomicAdd(a.dplus + u, (int32_t)run);
-      run = 0;
-      u = next_row(a.off, a.n, u, e);
-      row_end = __ldg(a.off + u + 1);
-    }
-    if (keep & (1u << i)) {
-      a.adjp[pos++] = __ldg(a.adj + e);
-      ++run;
+      at = __shfl_sync(FULL_MASK, at, start);
+      if (keep) {
+        const uint64_t pos = (uint64_t)(__ldg(a.in_off + rx) - __ldg(a.in_off + a.r0)) + (uint32_t)at +
+                             __popc(mine & lanemask_lt());
+        if (pos < a.edges) {  // (always, unless the graph is not symmetric)
+          a.keys[pos] = ((uint64_t)(uint32_t)ry << 32) | pos;
+          a.v_of[pos] = (uint32_t)rx;
+        }
+      }
     }
   }
-  if (run) atomicAdd(a.dplus + u, (int32_t)run);
 }
+
+// Last place of each u's run in the group's edges sorted by u.
+// (u < n here and below: always, unless the graph is not symmetric and places
+// were left empty.)
+__global__ __launch_bounds__(EX_THREADS) void k_run_ends(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
+                                                         uint32_t* __restrict__ run_end) {
+  const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
+  if (i >= m) return;
+  const uint32_t u = (uint32_t)(keys[i] >> 32);
+  if (u >= n) return;
+  if (i + 1 == m || (uint32_t)(keys[i + 1] >> 32) != u) run_end[u] = (uint32_t)(i + 1);
+}
+
+// After a group: how many entries each row holds now.
+__global__ __launch_bounds__(EX_THREADS) void k_run_add(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
+                                                        const uint32_t* __restrict__ run_end,
+                                                        uint32_t* __restrict__ filled) {
+  const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
+  if (i >= m) return;
+  const uint32_t u = (uint32_t)(keys[i] >> 32);
+  if (u >= n) return;
+  if (i == 0 || (uint32_t)(keys[i - 1] >> 32) != u) filled[u] += run_end[u] - (uint32_t)i;
+}
+
+// Rows N+(u), from their ends: sorted edge i (u, and by its place the v) goes
+// before the entries of higher rank, and its in-list place learns how many
+// these are. WHOLE: the group is all there is, so i is the place in the rows.
+template <bool WHOLE>
+__global__ __launch_bounds__(EX_THREADS) void k_rows(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
+                                                     const uint32_t* __restrict__ v_of,
+                                                     const int64_t* __restrict__ row_off,
+                                                     const uint32_t* __restrict__ run_end,
+                                                     const uint32_t* __restrict__ filled, uint32_t* __restrict__ rows,
+                                                     int64_t n_rows, uint2* __restrict__ rec) {
+  const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
+  if (i >= m) return;
+  const uint64_t key = __ldcs(keys + i);
+  const uint32_t u = (uint32_t)(key >> 32), pos = (uint32_t)key;
+  if (u >= n || pos >= m) return;
+  const int64_t row_end = __ldg(row_off + u + 1);
+  const uint32_t after = WHOLE ? (uint32_t)(row_end - 1 - i)
+                               : __ldg(filled + u) + (__ldg(run_end + u) - 1u - (uint32_t)i);
+  const int64_t at = row_end - 1 - (int64_t)after;
+  if (at < n_rows) rows[at] = __ldg(v_of + pos);  // (always, unless the graph is not symmetric)
+  rec[pos] = make_uint2(u, after);
+}
+
+// ----------------------------------------------------------------- count --
 
 struct CountArgs {
-  const int64_t* offp;  // n + 1 oriented row offsets
-  const int32_t* adjp;
-  const int32_t* deg;
-  int32_t n;
-  const uint64_t* lo;
-  uint32_t nb, pow2;
-  unsigned long long* pbq;   // [nb][4] (class 1..3 used)
-  unsigned long long* t_i;   // per-vertex closed wedges or nullptr
-  unsigned int* next;        // work counter of the warp kernel
-  int32_t* big;              // n entries: medium rows from the front, long rows from the back
-  unsigned int* big_n;       // [0] medium, [1] long
+  const int64_t* row_off;  // n + 1, by rank
+  const uint32_t* rows;
+  const int64_t* in_off;   // n + 1, by rank
+  const uint2* rec;        // the group's in-lists: u, entries of N+(u) after v
+  const int32_t* order;
+  const uint32_t* bin_lo;  // first rank of each bin, then n
+  uint32_t nb;
+  uint32_t n;
+  int64_t m;               // entries of rows
+  int64_t edges;           // entries of rec
+  uint32_t grab;           // vertices a warp takes per ticket
+  int32_t r0, r1;          // the group's ranks
+  unsigned long long* pbq; // [nb][4] (class 1..3 used)
+  unsigned long long* t_i; // per-vertex closed wedges or nullptr
+  unsigned int* next;      // work counter of the warp kernel
+  uint2* units;            // (v, part of its in-list) for the CTA kernels: medium rows from the front, long from the back
+  uint32_t max_units;
+  unsigned int* n_units;   // [0] medium, [1] long
 };
 
-constexpr int WARP_DEG = 128;       // oriented rows up to this length: one warp, table in shared memory
-constexpr int WARP_SLOTS = 256;     // table slots per warp (2 x WARP_DEG)
-constexpr int MID_ROW = 1024;       // longest row of the medium CTA kernel
-constexpr int GRAB = 32;            // vertices a warp takes per ticket
+constexpr int WARP_ROW = 128;        // rows N+(v) up to this length ...
+constexpr int WARP_IN = 64;          // ... with in-lists up to this: one warp
+constexpr int WARP_SLOTS = 512;
+constexpr int MEMORY_ROW = 8;        // rows up to this length are searched where they are
+constexpr int MID_ROW = 1024;        // longest row of the medium CTA kernel
+constexpr int UNIT_IN = 512;         // in-edges of a unit of the CTA kernels
+constexpr uint32_t GRAB = 8;         // vertices a warp takes per ticket at most
 
-__device__ __forceinline__ uint32_t slot_of(int32_t w, uint32_t mask) {
-  return ((uint32_t)w * 0x9E3779B1u) >> 7 & mask;
+__device__ __forceinline__ uint32_t slot_of(uint32_t w, uint32_t mask) { return (w * 0x9E3779B1u) >> 7 & mask; }
+
+// Insert key w (absent); the table has free slots (load <= 1/2).
+__device__ __forceinline__ void insert_key(uint32_t* table, uint32_t mask, uint32_t w) {
+  uint32_t h = slot_of(w, mask);
+  while (atomicCAS(table + h, ~0u, w) != ~0u) h = (h + 1) & mask;
 }
 
-// Insert key w (absent) with its bin; the table has free slots (load <= 1/2).
-__device__ __forceinline__ void insert_key(int32_t* table, uint8_t* tbin, uint32_t mask, int32_t w, uint32_t bw) {
-  uint32_t h = slot_of(w, mask);
-  while (atomicCAS(table + h, -1, w) != -1) h = (h + 1) & mask;
-  tbin[h] = (uint8_t)bw;
+// Bin of a rank: ranks ascend by degree, so every bin is a range of them,
+// lo[b] to lo[b + 1] (lo[nb] = n).
+__device__ __forceinline__ uint32_t rank_bin(const uint32_t* lo, uint32_t nb, uint32_t r) {
+  uint32_t b = 0, e = nb;  // last bin with lo <= r
+  while (e - b > 1) {
+    const uint32_t mid = (b + e) >> 1;
+    if (lo[mid] <= r) b = mid; else e = mid;
+  }
+  return b;
 }
 
-// Slot of key w, or -1.
-__device__ __forceinline__ int find_key(const int32_t* table, uint32_t mask, int32_t w) {
-  uint32_t h = slot_of(w, mask);
-  while (true) {
-    const int32_t x = table[h];
-    if (x == w) return (int)h;
-    if (x == -1) return -1;
-    h = (h + 1) & mask;
+// Which w are in N+(v), and the counter each has.
+struct HashRow {  // a hash table; the counter is the slot
+  const uint32_t* table;
+  uint32_t mask;
+  __device__ __forceinline__ bool find(uint32_t w, uint32_t& slot) const {
+    uint32_t h = slot_of(w, mask);
+    while (true) {
+      const uint32_t x = table[h];
+      slot = h;
+      if (x == w) return true;
+      if (x == ~0u) return false;
+      h = (h + 1) & mask;
+    }
+  }
+};
+struct BitRow {  // one bit per rank above v; the counter is w's place in the row
+  const uint32_t* bits;
+  const uint16_t* before;  // row entries before the word's first
+  uint32_t above;          // v + 1
+  __device__ __forceinline__ bool find(uint32_t w, uint32_t& slot) const {
+    const uint32_t i = w - above, word = bits[i >> 5], rest = word >> (i & 31u);
+    if (!(rest & 1u)) return false;
+    slot = before[i >> 5] + __popc(word) - __popc(rest);
+    return true;
+  }
+};
+struct MemoryRow {  // a search of the row in memory; no counters
+  const uint32_t* row;
+  uint32_t d;
+  __device__ __forceinline__ bool find(uint32_t w, uint32_t&) const {
+    uint32_t lo = 0, hi = d;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi) >> 1, x = __ldg(row + mid);
+      if (x == w) return true;
+      if (x < w) lo = mid + 1; else hi = mid;
+    }
+    return false;
+  }
+};
+
+// The tails of up to 32 in-edges of v (one per lane; length 0: none) against
+// N+(v). A found w closes the triangle u < v < w, one closed wedge centred at
+// each vertex, of class 1 + (endpoints in the centre's bin): w's are added to
+// its counter (low half: bin(u) != bin(w), high half: equal; at most one per
+// in-edge, so the halves do not overflow) or, where there is none, to the
+// histogram; u's and v's are summed per tail, kept by the lane whose in-edge it
+// is, and added at the end by all lanes at once (cv: v's, by number of
+// endpoints in v's bin). w > v > u, so w is in u's bin iff it lies below that
+// bin's end.
+// Long tails are streamed one after the other by the whole warp. Tails shorter
+// than FLAT entries on average are taken as one list of their entries (a search
+// by shuffles finds an entry's tail): a warp per tail left most lanes idle
+// (uniform graph, 16 M edges, tails of 7: 1.7 ms, 0.9 so).
+constexpr uint32_t FLAT = 24;
+
+template <bool COUNTERS, typename Row>
+__device__ __forceinline__ void count_tails(const CountArgs& a, const Row& nv, const uint32_t* s_lo,
+                                            unsigned long long* hist, uint2 r, uint32_t bv, uint32_t* hits,
+                                            uint32_t* seg, uint32_t (&cv)[3], int lane) {
+  if (r.x >= a.n) r.y = 0;  // (here and below: only if the graph is not symmetric)
+  const uint32_t my_bin = r.y ? rank_bin(s_lo, a.nb, r.x) : 0u, my_end_u = s_lo[my_bin + 1];
+  const int64_t my_row_end = r.y ? __ldg(a.row_off + r.x + 1) : 0;
+  if (my_row_end > a.m || my_row_end < (int64_t)r.y) r.y = 0;
+  const uint64_t my_tail = (uint64_t)(my_row_end - r.y);
+  const uint32_t end_v = s_lo[bv + 1];
+  uint32_t found = 0, with_u = 0, with_v = 0;  // this lane's in-edge
+  // w of a tail of a u whose bin ends at end_u: what it adds to found (low 10
+  // bits), with_u (next 10) and with_v (the rest)
+  auto look = [&](uint32_t w, uint32_t end_u) {
+    uint32_t slot;
+    if (!nv.find(w, slot)) return 0u;
+    const bool in_u = w < end_u;
+    if (COUNTERS) {
+      atomicAdd(hits + slot, in_u ? 0x10000u : 1u);
+    } else {
+      const uint32_t bu = rank_bin(s_lo, a.nb, end_u - 1u), bw = rank_bin(s_lo, a.nb, w);
+      atomicAdd(&hist[bw * 4 + 1 + (bu == bw) + (bv == bw)], 1ULL);
+      if (a.t_i) atomicAdd(a.t_i + a.order[w], 1ULL);
+    }
+    return (in_u ? 1025u : 1u) + (w < end_v ? 1u << 20 : 0u);
+  };
+  uint32_t todo = __ballot_sync(FULL_MASK, r.y != 0);
+  const uint32_t total = __reduce_add_sync(FULL_MASK, min(r.y, 2 * 32 * FLAT));
+  if (total < FLAT * __popc(todo)) {
+    uint32_t incl = r.y;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(FULL_MASK, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const uint64_t my_first = my_tail - (incl - r.y);  // entry t of the list is a.rows[my_first + t]
+    seg[lane] = 0;
+    __syncwarp();
+    for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+      const uint32_t t = min(t0 + lane, total - 1u);
+      int l = 0;  // the first lane whose tails end after t
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1)
+        if (__shfl_sync(FULL_MASK, incl, l + step - 1) <= t) l += step;
+      const uint64_t first = __shfl_sync(FULL_MASK, my_first, l);
+      const uint32_t end_u = __shfl_sync(FULL_MASK, my_end_u, l);
+      if (t0 + lane < total) {
+        const uint32_t add = look(__ldg(a.rows + first + t), end_u);
+        if (add) atomicAdd(seg + l, add);
+      }
+    }
+    __syncwarp();
+    found = seg[lane] & 1023u;
+    with_u = (seg[lane] >> 10) & 1023u;
+    with_v = seg[lane] >> 20;
+    __syncwarp();
+  } else {
+    for (; todo; todo &= todo - 1) {
+      const int l = __ffs(todo) - 1;
+      const uint32_t len = __shfl_sync(FULL_MASK, r.y, l), end_u = __shfl_sync(FULL_MASK, my_end_u, l);
+      const uint32_t* tail = a.rows + __shfl_sync(FULL_MASK, my_tail, l);
+      for (uint32_t k0 = 0; k0 < len; k0 += 30 * 32) {  // (sums of 30 x 32 fit their 10 bits)
+        uint32_t mine = 0;
+        const uint32_t k1 = min(len, k0 + 30 * 32);
+        for (uint32_t k = k0 + lane; k < k1; k += 64) {  // two loads in flight
+          const bool two = k + 32 < k1;
+          const uint32_t w0 = __ldg(tail + k), w1 = two ? __ldg(tail + k + 32) : 0u;
+          mine += look(w0, end_u);
+          if (two) mine += look(w1, end_u);
+        }
+        mine = __reduce_add_sync(FULL_MASK, mine);
+        if (lane == l) {
+          found += mine & 1023u;
+          with_u += (mine >> 10) & 1023u;
+          with_v += mine >> 20;
+        }
+      }
+    }
+  }
+  if (found) {
+    unsigned long long* hu = hist + my_bin * 4 + 1 + (bv == my_bin);
+    if (found > with_u) atomicAdd(hu, (unsigned long long)(found - with_u));
+    if (with_u) atomicAdd(hu + 1, (unsigned long long)with_u);
+    if (a.t_i) atomicAdd(a.t_i + a.order[r.x], (unsigned long long)found);
+    const uint32_t diff = found - with_v;
+    if (my_bin == bv) {
+      cv[1] += diff;
+      cv[2] += with_v;
+    } else {
+      cv[0] += diff;
+      cv[1] += with_v;
+    }
   }
 }
 
-// Closed wedges counted in registers for one centre (u, or the current v of
-// a walker), by class 1..3.
-struct Tally {
-  int32_t vertex;
-  uint32_t bin;
-  uint32_t c1, c2, c3;
-};
-
-__device__ __forceinline__ void tally_add(Tally& t, uint32_t same) {
-  t.c1 += same == 0u;
-  t.c2 += same == 1u;
-  t.c3 += same == 2u;
+// v's closed wedges, summed over the warp.
+__device__ __forceinline__ void flush_centre(const CountArgs& a, unsigned long long* hist, uint32_t v, uint32_t bv,
+                                             uint32_t (&cv)[3], int lane) {
+  for (int q = 0; q < 3; ++q) cv[q] = __reduce_add_sync(FULL_MASK, cv[q]);
+  if (lane != 0) return;
+  for (int q = 0; q < 3; ++q)
+    if (cv[q]) atomicAdd(&hist[bv * 4 + 1 + q], (unsigned long long)cv[q]);
+  const uint32_t all = cv[0] + cv[1] + cv[2];
+  if (a.t_i && all) atomicAdd(a.t_i + a.order[v], (unsigned long long)all);
 }
 
-__device__ __forceinline__ void tally_flush(unsigned long long* hist, Tally& t, unsigned long long* t_i) {
-  if (t.c1) atomicAdd(&hist[t.bin * 4 + 1], (unsigned long long)t.c1);
-  if (t.c2) atomicAdd(&hist[t.bin * 4 + 2], (unsigned long long)t.c2);
-  if (t.c3) atomicAdd(&hist[t.bin * 4 + 3], (unsigned long long)t.c3);
-  const uint32_t tot = t.c1 + t.c2 + t.c3;
-  if (t_i && tot) atomicAdd(t_i + t.vertex, (unsigned long long)tot);
-  t.c1 = t.c2 = t.c3 = 0;
+// Adds a counter (closed wedges centred at w) to the histogram and clears it.
+__device__ __forceinline__ void fold_hit(const CountArgs& a, const uint32_t* s_lo, unsigned long long* hist,
+                                         uint32_t* hit, uint32_t w, uint32_t bv) {
+  const uint32_t x = *hit, same = x >> 16, diff = x & 0xffffu;
+  *hit = 0;
+  const uint32_t bw = rank_bin(s_lo, a.nb, w);
+  unsigned long long* hw = hist + bw * 4 + 1 + (bv == bw);
+  if (diff) atomicAdd(hw, (unsigned long long)diff);
+  if (same) atomicAdd(hw + 1, (unsigned long long)same);
+  if (a.t_i) atomicAdd(a.t_i + a.order[w], (unsigned long long)(same + diff));
 }
 
-// Triangle u < v < w (degree order), w found in table slot h. One closed
-// wedge centred at each vertex, class 1 + (endpoints in the centre's bin):
-// u and v are tallied in registers; w in the slot's hit counter (low half:
-// bin(v) != bin(w), high half: bin(v) == bin(w); at most d+(u) <= 2^12 hits
-// a slot per vertex u, so the halves cannot overflow).
-__device__ __forceinline__ void count_triangle(Tally& tu, Tally& tv, uint32_t* hits, int h, uint32_t bw) {
-  const uint32_t bu = tu.bin, bv = tv.bin;
-  tally_add(tu, (bv == bu) + (bw == bu));
-  tally_add(tv, (bu == bv) + (bw == bv));
-  atomicAdd(hits + h, bv == bw ? 0x10000u : 1u);
-}
-
-// Fold the slots' hit counters (closed wedges centred at the table's
-// vertices w) into the histogram; reset them.
-__device__ __forceinline__ void fold_hits(unsigned long long* hist, const int32_t* table, const uint8_t* tbin,
-                                          uint32_t* hits, uint32_t slots, uint32_t bu, unsigned long long* t_i,
-                                          int first, int stride) {
-  for (uint32_t h = first; h < slots; h += stride) {
-    const uint32_t x = hits[h];
-    if (x == 0) continue;
-    hits[h] = 0;
-    const uint32_t bw = tbin[h];
-    const uint32_t base = bw * 4 + 1 + (bu == bw);
-    const uint32_t same = x >> 16, diff = x & 0xffffu;
-    if (diff) atomicAdd(&hist[base], (unsigned long long)diff);
-    if (same) atomicAdd(&hist[base + 1], (unsigned long long)same);
-    if (t_i) atomicAdd(t_i + table[h], (unsigned long long)(same + diff));
-  }
-}
-
-struct WarpSmem {
-  uint64_t lo[WEDGE_MAX_BINS];
-  unsigned long long hist[WEDGE_MAX_BINS * 4];
-  int32_t table[TC_THREADS / 32][WARP_SLOTS];
-  uint32_t hits[TC_THREADS / 32][WARP_SLOTS];
-  uint8_t tbin[TC_THREADS / 32][WARP_SLOTS];
-  uint32_t pre[TC_THREADS / 32][WARP_DEG + 1];  // work prefix over the row's entries
-  int64_t voff[TC_THREADS / 32][WARP_DEG];      // row start of each out-neighbour v
-  int32_t vid[TC_THREADS / 32][WARP_DEG];
-  uint8_t vbin[TC_THREADS / 32][WARP_DEG];
-};
-
-// Triangles whose smallest vertex u (in degree order) has 2 <= d+(u) <= WARP_DEG:
-// one warp per u. N+(u) goes into a shared-memory hash table (with each
-// entry's bin); the rows N+(v) of all v in N+(u) are streamed as one
-// flattened work list split across the lanes, each entry w probed in the
-// table. Longer rows are queued.
-__global__ __launch_bounds__(TC_THREADS) void k_tri_hash_warp(CountArgs a) {
-  __shared__ WarpSmem sm;
-  for (int i = threadIdx.x; i < (int)a.nb; i += TC_THREADS) sm.lo[i] = a.lo[i];
-  for (int i = threadIdx.x; i < (int)a.nb * 4; i += TC_THREADS) sm.hist[i] = 0;
+// One warp per vertex v with a short row and a short in-list, highest ranks
+// (the most work) first; the others are queued as units of UNIT_IN in-edges.
+__global__ __launch_bounds__(EX_THREADS) void k_tri_hash_warp(CountArgs a) {
+  __shared__ uint32_t s_lo[WEDGE_MAX_BINS + 1];
+  __shared__ unsigned long long s_hist[WEDGE_MAX_BINS * 4];
+  __shared__ uint32_t s_table[EX_WARPS][WARP_SLOTS];
+  __shared__ uint32_t s_hits[EX_WARPS][WARP_SLOTS];
+  __shared__ uint32_t s_seg[EX_WARPS][32];
+  for (int i = threadIdx.x; i <= (int)a.nb; i += EX_THREADS) s_lo[i] = a.bin_lo[i];
+  for (int i = threadIdx.x; i < (int)a.nb * 4; i += EX_THREADS) s_hist[i] = 0;
+  for (int i = threadIdx.x; i < EX_WARPS * WARP_SLOTS; i += EX_THREADS) (&s_hits[0][0])[i] = 0;
   __syncthreads();
-  const BinTable bt{sm.lo, a.nb, a.pow2};
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int32_t* table = sm.table[wid];
-  uint8_t* tbin = sm.tbin[wid];
-  uint32_t* hits = sm.hits[wid];
-  uint32_t* pre = sm.pre[wid];
-  for (int i = lane; i < WARP_SLOTS; i += 32) hits[i] = 0;
+  uint32_t* table = s_table[wid];
+  uint32_t* hits = s_hits[wid];
+  const int64_t in0 = __ldg(a.in_off + a.r0);
+  const uint32_t count = (uint32_t)(a.r1 - a.r0);
   while (true) {
     unsigned int first = 0;
-    if (lane == 0) first = atomicAdd(a.next, (unsigned int)GRAB);
+    if (lane == 0) first = atomicAdd(a.next, a.grab);
     first = __shfl_sync(FULL_MASK, first, 0);
-    if (first >= (unsigned int)a.n) break;
-    const int32_t last = (int32_t)min((unsigned int)a.n, first + (unsigned int)GRAB);
-    for (int32_t u = (int32_t)first; u < last; ++u) {
-      const int64_t u_lo = __ldg(a.offp + u);
-      const int32_t d = (int32_t)(__ldg(a.offp + u + 1) - u_lo);
-      if (d < 2) continue;
-      if (d > WARP_DEG) {  // medium rows fill the list from the front, long ones from the back
-        if (lane == 0) {
-          if (d <= MID_ROW) a.big[atomicAdd(a.big_n, 1u)] = u;
-          else a.big[a.n - 1 - (int32_t)atomicAdd(a.big_n + 1, 1u)] = u;
-        }
+    if (first >= count) break;
+    const uint32_t last = min(count, first + a.grab);
+    for (uint32_t i = first; i < last; ++i) {
+      const uint32_t v = (uint32_t)a.r1 - 1u - i;
+      const int64_t row = __ldg(a.row_off + v), in = __ldg(a.in_off + v);
+      // (the bounds hold by themselves unless the graph is not symmetric)
+      const int64_t d = min(a.m, __ldg(a.row_off + v + 1)) - row;
+      const int64_t k = min(in0 + a.edges, __ldg(a.in_off + v + 1)) - in;
+      if (d <= 0 || k <= 0) continue;
+      if (d > WARP_ROW || k > WARP_IN) {
+        const uint32_t parts = (uint32_t)((k + UNIT_IN - 1) / UNIT_IN);
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(a.n_units + (d > MID_ROW), parts);
+        at = __shfl_sync(FULL_MASK, at, 0);
+        for (uint32_t p = lane; p < parts; p += 32)
+          if (at + p < a.max_units) a.units[d > MID_ROW ? a.max_units - 1 - (at + p) : at + p] = make_uint2(v, p);
         continue;
       }
-      for (int i = lane; i < WARP_SLOTS; i += 32) table[i] = -1;
+      const uint32_t bv = rank_bin(s_lo, a.nb, v);
+      uint32_t cv[3] = {0, 0, 0};
+      auto tails = [&](int64_t j) {
+        return j + lane < k ? __ldcs(a.rec + (in - in0) + j + lane) : make_uint2(0, 0);
+      };
+      if (d <= MEMORY_ROW) {  // a few entries are found faster than they are entered into a table
+        for (int64_t j = 0; j < k; j += 32)
+          count_tails<false>(a, MemoryRow{a.rows + row, (uint32_t)d}, s_lo, s_hist, tails(j), bv, hits, s_seg[wid], cv,
+                             lane);
+        flush_centre(a, s_hist, v, bv, cv, lane);
+        continue;
+      }
+      uint32_t slots = 32;
+      while (slots < 4u * (uint32_t)d) slots <<= 1;  // at most WARP_SLOTS
+      for (uint32_t j = lane; j < slots; j += 32) table[j] = ~0u;
       __syncwarp();
-      // N+(u) into the table; per-entry work lengths d+(v)
-      uint32_t len[WARP_DEG / 32];
-      uint32_t mine = 0;
-#pragma unroll
-      for (int j = 0; j < WARP_DEG / 32; ++j) {
-        const int i = lane * (WARP_DEG / 32) + j;  // blocked: lane owns 4 consecutive entries
-        len[j] = 0;
-        if (i < d) {
-          const int32_t v = __ldg(a.adjp + u_lo + i);
-          const uint32_t bv = bin_of(bt, (uint64_t)__ldg(a.deg + v));
-          insert_key(table, tbin, WARP_SLOTS - 1, v, bv);
-          const int64_t v_lo = __ldg(a.offp + v);
-          len[j] = (uint32_t)(__ldg(a.offp + v + 1) - v_lo);
-          sm.voff[wid][i] = v_lo;
-          sm.vid[wid][i] = v;
-          sm.vbin[wid][i] = (uint8_t)bv;
-        }
-        mine += len[j];
-      }
-      uint32_t incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL_MASK, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t total = __shfl_sync(FULL_MASK, incl, 31);
-      uint32_t run = incl - mine;
-#pragma unroll
-      for (int j = 0; j < WARP_DEG / 32; ++j) {
-        const int i = lane * (WARP_DEG / 32) + j;
-        if (i < d) pre[i] = run;
-        run += len[j];
-      }
-      if (lane == 0) pre[d] = total;
+      for (uint32_t j = lane; j < (uint32_t)d; j += 32) insert_key(table, slots - 1, __ldg(a.rows + row + j));
       __syncwarp();
-      if (total == 0) continue;
-      Tally tu{u, bin_of(bt, (uint64_t)__ldg(a.deg + u)), 0, 0, 0};
-      Tally tv{0, 0, 0, 0, 0};
-      int i = 0, cur = -1;  // pre[i] <= t < pre[i+1], walked forward as t grows
-      for (uint32_t t = lane; t < total; t += 32) {
-        while (pre[i + 1] <= t) ++i;
-        if (i != cur) {
-          tally_flush(sm.hist, tv, a.t_i);
-          tv.vertex = sm.vid[wid][i];
-          tv.bin = sm.vbin[wid][i];
-          cur = i;
-        }
-        const int32_t w = __ldg(a.adjp + sm.voff[wid][i] + (t - pre[i]));
-        const int h = find_key(table, WARP_SLOTS - 1, w);
-        if (h >= 0) count_triangle(tu, tv, hits, h, tbin[h]);
-      }
-      tally_flush(sm.hist, tv, a.t_i);
-      tally_flush(sm.hist, tu, a.t_i);
+      for (int64_t j = 0; j < k; j += 32)
+        count_tails<true>(a, HashRow{table, slots - 1}, s_lo, s_hist, tails(j), bv, hits, s_seg[wid], cv, lane);
+      flush_centre(a, s_hist, v, bv, cv, lane);
       __syncwarp();
-      fold_hits(sm.hist, table, tbin, hits, WARP_SLOTS, tu.bin, a.t_i, lane, 32);
+      for (uint32_t h = lane; h < slots; h += 32)
+        if (hits[h]) fold_hit(a, s_lo, s_hist, hits + h, table[h], bv);
       __syncwarp();
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < (int)a.nb * 4; i += TC_THREADS)
-    if (sm.hist[i]) atomicAdd(a.pbq + i, sm.hist[i]);
+  for (int i = threadIdx.x; i < (int)a.nb * 4; i += EX_THREADS)
+    if (s_hist[i]) atomicAdd(a.pbq + i, s_hist[i]);
 }
 
-// One CTA per queued vertex u with d+(u) > WARP_DEG, taken by ticket. N+(u)
-// (with each entry's bin) goes into a table of SLOTS slots in dynamic shared
-// memory when d+(u) <= SLOTS / 2; a longer row searches N+(u) in global
-// memory instead (degree order bounds d+ by about sqrt(2m), so this is rare).
-// The rows N+(v), v in N+(u), are streamed in chunks of SLOTS / 2
-// out-neighbours as one flattened work list. (The walker code allows several
-// items in flight per thread; one measured fastest: fewer registers, more
-// resident warps.)
-template <int THREADS, int SLOTS>
-__global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const int32_t* __restrict__ list,
-                                                          int32_t n_list, unsigned int* ticket) {
-  constexpr int ILP = 1;
-  constexpr int CHUNK = SLOTS / 2;
+// One CTA per unit (by ticket); its warps take the unit's in-edges 32 at a
+// time. N+(v) is a bit map in shared memory where v is among the MAP_BITS
+// highest ranks (most of the work is: they have the long in-lists; six
+// instructions and no loop per look), a hash table where SLOTS is at least
+// twice the row, and else searched in memory (degree order bounds rows by about
+// sqrt(2m), so this is rare).
+template <int THREADS, int SLOTS, int MAP_BITS>
+struct CtaSmem {
+  union {
+    uint32_t table[SLOTS];
+    struct {
+      uint32_t bits[MAP_BITS / 32];
+      uint16_t before[MAP_BITS / 32];
+    } map;
+  };
+  uint32_t hits[SLOTS];
+};
+
+template <int THREADS, int SLOTS, int MAP_BITS>
+__global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uint2* __restrict__ list, int dir,
+                                                          const unsigned int* __restrict__ n_units,
+                                                          unsigned int* ticket) {
   extern __shared__ __align__(16) unsigned char dyn[];
-  int32_t* table = reinterpret_cast<int32_t*>(dyn);
-  uint32_t* hits = reinterpret_cast<uint32_t*>(dyn + SLOTS * sizeof(int32_t));                 // SLOTS entries
-  uint32_t* pre = reinterpret_cast<uint32_t*>(dyn + 2 * SLOTS * sizeof(int32_t));              // CHUNK + 1 entries
-  uint8_t* tbin = dyn + 2 * SLOTS * sizeof(int32_t) + (CHUNK + 1) * sizeof(uint32_t);         // SLOTS entries
-  __shared__ uint64_t s_lo[WEDGE_MAX_BINS];
+  CtaSmem<THREADS, SLOTS, MAP_BITS>& sm = *reinterpret_cast<CtaSmem<THREADS, SLOTS, MAP_BITS>*>(dyn);
+  __shared__ uint32_t s_lo[WEDGE_MAX_BINS + 1];
   __shared__ unsigned long long s_hist[WEDGE_MAX_BINS * 4];
-  __shared__ uint32_t s_wsum[THREADS / 32];
-  __shared__ int32_t s_q;
-  for (int i = threadIdx.x; i < (int)a.nb; i += THREADS) s_lo[i] = a.lo[i];
+  __shared__ uint32_t s_seg[THREADS / 32][32];
+  __shared__ uint32_t s_q, s_batch;
+  for (int i = threadIdx.x; i <= (int)a.nb; i += THREADS) s_lo[i] = a.bin_lo[i];
   for (int i = threadIdx.x; i < (int)a.nb * 4; i += THREADS) s_hist[i] = 0;
-  for (int i = threadIdx.x; i < SLOTS; i += THREADS) hits[i] = 0;
-  const BinTable bt{s_lo, a.nb, a.pow2};
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  while (true) {
-    __syncthreads();  // previous vertex finished with table and pre
-    if (tid == 0) s_q = (int32_t)atomicAdd(ticket, 1u);
+  for (int i = threadIdx.x; i < SLOTS; i += THREADS) sm.hits[i] = 0;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t in0 = __ldg(a.in_off + a.r0);
+  const uint32_t n_list = min(*n_units, a.max_units);
+  while (n_list > 0) {
+    __syncthreads();  // the previous unit is done with the table
+    if (tid == 0) {
+      s_q = atomicAdd(ticket, 1u);
+      s_batch = 0;
+    }
     __syncthreads();
-    const int32_t q = s_q;
+    const uint32_t q = s_q;
     if (q >= n_list) break;
-    const int32_t u = list[q];
-    const int64_t u_lo = __ldg(a.offp + u);
-    const int32_t d = (int32_t)(__ldg(a.offp + u + 1) - u_lo);
-    const bool in_smem = d <= CHUNK;
+    const uint2 unit = list[(int64_t)dir * q];
+    const uint32_t v = unit.x;
+    const int64_t row_at = __ldg(a.row_off + v);
+    const uint32_t* row = a.rows + row_at;
+    const uint32_t d = (uint32_t)(min(a.m, __ldg(a.row_off + v + 1)) - row_at);
+    const int64_t in = __ldg(a.in_off + v) + (int64_t)unit.y * UNIT_IN;
+    const uint32_t k = (uint32_t)min((int64_t)UNIT_IN, min(in0 + a.edges, __ldg(a.in_off + v + 1)) - in);
+    const uint32_t range = a.n - 1u - v;  // ranks above v
+    const bool in_map = range <= (uint32_t)MAP_BITS && d <= (uint32_t)SLOTS;
+    const bool in_table = !in_map && 2u * d <= (uint32_t)SLOTS;
     uint32_t slots = 64;
-    while (slots < 2u * (uint32_t)d && slots < (uint32_t)SLOTS) slots <<= 1;
-    const uint32_t mask = slots - 1;
-    if (in_smem) {
-      for (uint32_t i = tid; i < slots; i += THREADS) table[i] = -1;
+    while (slots < 4u * d && slots < (uint32_t)SLOTS) slots <<= 1;
+    if (in_map) {
+      for (uint32_t i = tid; i < (range + 31u) / 32u; i += THREADS) sm.map.bits[i] = 0;
       __syncthreads();
-      for (int i = tid; i < d; i += THREADS) {
-        const int32_t w = __ldg(a.adjp + u_lo + i);
-        insert_key(table, tbin, mask, w, bin_of(bt, (uint64_t)__ldg(a.deg + w)));
+      for (uint32_t i = tid; i < d; i += THREADS) {
+        const uint32_t x = __ldg(row + i) - (v + 1u), y = i ? __ldg(row + i - 1) - (v + 1u) : ~0u;
+        atomicOr(&sm.map.bits[x >> 5], 1u << (x & 31u));
+        if ((x >> 5) != (y >> 5)) sm.map.before[x >> 5] = (uint16_t)i;
       }
+      __syncthreads();
+    } else if (in_table) {
+      for (uint32_t i = tid; i < slots; i += THREADS) sm.table[i] = ~0u;
+      __syncthreads();
+      for (uint32_t i = tid; i < d; i += THREADS) insert_key(sm.table, slots - 1, __ldg(row + i));
+      __syncthreads();
     }
-    Tally tu{u, bin_of(bt, (uint64_t)__ldg(a.deg + u)), 0, 0, 0};
-    for (int c0 = 0; c0 < d; c0 += CHUNK) {
-      const int cn = min(d - c0, CHUNK);
-      const int per = (cn + THREADS - 1) / THREADS;  // blocked: thread owns `per` consecutive entries
-      uint32_t mine = 0;
-      for (int j = 0; j < per; ++j) {
-        const int i = tid * per + j;
-        if (i < cn) {
-          const int32_t v = __ldg(a.adjp + u_lo + c0 + i);
-          mine += (uint32_t)(__ldg(a.offp + v + 1) - __ldg(a.offp + v));
-        }
-      }
-      uint32_t incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL_MASK, incl, o);
-        if (lane >= o) incl += y;
-      }
-      __syncthreads();  // table inserts done; the previous chunk's readers are done with pre
-      if (lane == 31) s_wsum[warp] = incl;
-      __syncthreads();
-      uint32_t wpre = 0, total = 0;
-      for (int w = 0; w < THREADS / 32; ++w) {
-        if (w < warp) wpre += s_wsum[w];
-        total += s_wsum[w];
-      }
-      uint32_t run = wpre + incl - mine;
-      for (int j = 0; j < per; ++j) {
-        const int i = tid * per + j;
-        if (i < cn) {
-          pre[i] = run;
-          const int32_t v = __ldg(a.adjp + u_lo + c0 + i);
-          run += (uint32_t)(__ldg(a.offp + v + 1) - __ldg(a.offp + v));
-        }
-      }
-      if (tid == 0) pre[cn] = total;
-      __syncthreads();
-      // ILP independent walkers: item r of an iteration is t0 + r * THREADS
-      int wi[ILP], cur[ILP];
-      int32_t wv[ILP];
-      int64_t wlo[ILP];
-      Tally tv[ILP];
-#pragma unroll
-      for (int r = 0; r < ILP; ++r) {
-        wi[r] = 0;
-        cur[r] = -1;
-        wv[r] = 0;
-        wlo[r] = 0;
-        tv[r] = Tally{0, 0, 0, 0, 0};
-      }
-      for (uint32_t t0 = tid; t0 < total; t0 += ILP * THREADS) {
-        int32_t w[ILP];
-#pragma unroll
-        for (int r = 0; r < ILP; ++r) {
-          const uint32_t t = t0 + (uint32_t)r * THREADS;
-          w[r] = -1;
-          if (t < total) {
-            while (pre[wi[r] + 1] <= t) ++wi[r];
-            if (wi[r] != cur[r]) {
-              tally_flush(s_hist, tv[r], a.t_i);
-              cur[r] = wi[r];
-              wv[r] = __ldg(a.adjp + u_lo + c0 + wi[r]);
-              wlo[r] = __ldg(a.offp + wv[r]);
-              tv[r].vertex = wv[r];
-              tv[r].bin = bin_of(bt, (uint64_t)__ldg(a.deg + wv[r]));
-            }
-            w[r] = __ldg(a.adjp + wlo[r] + (t - pre[wi[r]]));
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < ILP; ++r) {
-          if (w[r] < 0) continue;
-          if (in_smem) {
-            const int h = find_key(table, mask, w[r]);
-            if (h >= 0) count_triangle(tu, tv[r], hits, h, tbin[h]);
-          } else {
-            int64_t lo = u_lo, hi = u_lo + d;
-            while (lo < hi) {
-              const int64_t mid = lo + ((hi - lo) >> 1);
-              if (__ldg(a.adjp + mid) < w[r]) lo = mid + 1; else hi = mid;
-            }
-            if (lo < u_lo + d && __ldg(a.adjp + lo) == w[r]) {
-              // no table: the closed wedge at w goes straight to the histogram
-              const uint32_t bw = bin_of(bt, (uint64_t)__ldg(a.deg + w[r]));
-              const uint32_t bu = tu.bin, bv = tv[r].bin;
-              tally_add(tu, (bv == bu) + (bw == bu));
-              tally_add(tv[r], (bu == bv) + (bw == bv));
-              atomicAdd(&s_hist[bw * 4 + 1 + (bu == bw) + (bv == bw)], 1ULL);
-              if (a.t_i) atomicAdd(a.t_i + w[r], 1ULL);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < ILP; ++r) tally_flush(s_hist, tv[r], a.t_i);
+    const uint32_t bv = rank_bin(s_lo, a.nb, v);
+    uint32_t cv[3] = {0, 0, 0};
+    while (true) {
+      uint32_t j = 0;
+      if (lane == 0) j = atomicAdd(&s_batch, 32u);
+      j = __shfl_sync(FULL_MASK, j, 0);
+      if (j >= k) break;
+      const uint2 r = j + lane < k ? __ldcs(a.rec + (in - in0) + j + lane) : make_uint2(0, 0);
+      if (in_map)
+        count_tails<true>(a, BitRow{sm.map.bits, sm.map.before, v + 1u}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
+      else if (in_table)
+        count_tails<true>(a, HashRow{sm.table, slots - 1}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
+      else count_tails<false>(a, MemoryRow{row, d}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
     }
-    tally_flush(s_hist, tu, a.t_i);
-    if (in_smem) {
-      __syncthreads();  // all hits counted
-      fold_hits(s_hist, table, tbin, hits, slots, tu.bin, a.t_i, tid, THREADS);
+    flush_centre(a, s_hist, v, bv, cv, lane);
+    __syncthreads();  // all hits counted
+    if (in_map) {
+      for (uint32_t i = tid; i < d; i += THREADS)
+        if (sm.hits[i]) fold_hit(a, s_lo, s_hist, sm.hits + i, __ldg(row + i), bv);
+    } else if (in_table) {
+      for (uint32_t i = tid; i < slots; i += THREADS)
+        if (sm.hits[i]) fold_hit(a, s_lo, s_hist, sm.hits + i, sm.table[i], bv);
     }
   }
   __syncthreads();
@@ -525,13 +623,20 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const int
     if (s_hist[i]) atomicAdd(a.pbq + i, s_hist[i]);
 }
 
-constexpr int MID_THREADS = 256, MID_SLOTS = 2048;    // 128 < d+ <= 1024
-constexpr int BIG_THREADS = 512, BIG_SLOTS = 8192;    // d+ > 1024 (table for d+ <= 4096)
+constexpr int MID_THREADS = 256, MID_SLOTS = 2048, MID_BITS = 1 << 16;    // rows up to 1024
+constexpr int BIG_THREADS = 512, BIG_SLOTS = 16384, BIG_BITS = 1 << 19;   // rows beyond (table up to 8192)
 
-template <int THREADS, int SLOTS>
-constexpr size_t cta_smem() {
-  return 2 * (size_t)SLOTS * sizeof(int32_t) + ((size_t)SLOTS / 2 + 1) * sizeof(uint32_t) + (size_t)SLOTS;
+template <typename F>
+int ctas_per_sm(F* f, int threads, size_t smem) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  return std::max(n, 1);
 }
+
+unsigned blocks_for(int64_t items) { return (unsigned)((items + EX_THREADS - 1) / EX_THREADS); }
 
 }  // namespace
 }  // namespace wedge
@@ -551,125 +656,238 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
   for (uint32_t k = 0; k < inf.n_bins; ++k) out->p_b[k] = inf.p_b[k];
   const int32_t n = g->n;
   const int64_t n_adj = g->n_adj;
-  const int64_t m = n_adj / 2;
   if (t_i) WEDGE_CUDA_TRY(cudaMemsetAsync(t_i, 0, (size_t)n * sizeof(uint64_t), s), "wedge_exact");
-  if (m == 0) {
+  if (n_adj == 0) {
     for (uint32_t k = 0; k < inf.n_bins; ++k) out->pbq[k][0] = inf.p_b[k];
     return WEDGE_OK;
   }
+  const int64_t m = n_adj / 2;
+  if (n_adj / (EX_WARPS * 32 * OR_STEPS) >= (int64_t)INT32_MAX) return fail(WEDGE_EINVAL, "wedge_exact: graph too large");
 
-  int32_t* dplus = nullptr;
-  int64_t* offp = nullptr;
-  int32_t* adjp = nullptr;
-  uint64_t* status = nullptr;
+  uint64_t* keys = nullptr;
+  uint64_t* alt = nullptr;
   void* scratch = nullptr;
-  uint32_t* derr = nullptr;  // [0] error bits, [1] tile counter, [2] warp ticket, [3..4] queued, [5..6] CTA tickets
-  unsigned long long* cnt = nullptr;  // pbq [nb*4]
-  int32_t* big = nullptr;
+  int32_t* rank = nullptr;     // ranks, then vertices by rank (2n)
+  int32_t* counts = nullptr;   // per rank: lower and higher neighbours, entries taken, row entries, run ends (5n)
+  int64_t* offs = nullptr;     // in-list, then row offsets by rank (2(n + 1))
+  uint32_t* rows = nullptr;
+  uint32_t* v_of = nullptr;
+  uint2* rec = nullptr;
+  uint2* units = nullptr;
+  // control words (error bits, warp ticket, 2 unit counts, 2 CTA tickets), pbq [nb*4], the bins' first ranks
+  unsigned long long* cnt = nullptr;
   auto done = [&](wedge_status st) {
-    dfree(dplus, s);
-    dfree(offp, s);
-    dfree(adjp, s);
-    dfree(status, s);
+    dfree(keys, s);
+    dfree(alt, s);
     dfree(scratch, s);
-    dfree(derr, s);
+    dfree(rank, s);
+    dfree(counts, s);
+    dfree(offs, s);
+    dfree(rows, s);
+    dfree(v_of, s);
+    dfree(rec, s);
+    dfree(units, s);
     dfree(cnt, s);
-    dfree(big, s);
     return st;
   };
-  const int64_t tiles = (n_adj + OR_TILE - 1) / OR_TILE;
-  if (tiles > (int64_t)UINT32_MAX) return fail(WEDGE_EINVAL, "wedge_exact: graph too large");
-  const size_t n_cnt = (size_t)inf.n_bins * 4;
-  wedge_status st;
-  if ((st = dalloc_n(&dplus, (size_t)n, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc_n(&offp, (size_t)n + 1, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc_n(&adjp, (size_t)m, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc_n(&status, (size_t)tiles, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc(&scratch, scan_scratch_bytes(n), s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc_n(&derr, 8, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc_n(&cnt, n_cnt, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  if ((st = dalloc_n(&big, (size_t)n, s, "wedge_exact")) != WEDGE_OK) return done(st);
-  cudaError_t e = cudaMemsetAsync(dplus, 0, (size_t)n * sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, (size_t)tiles * sizeof(uint64_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(derr, 0, 8 * sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, n_cnt * sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return done(cuda_fail(e, "wedge_exact"));
+#define EXACT_TRY(expr)                                                        \
+  do {                                                                         \
+    const cudaError_t e__ = (expr);                                            \
+    if (e__ != cudaSuccess) return done(cuda_fail(e__, "wedge_exact"));        \
+  } while (0)
+#define EXACT_DO(expr)                                     \
+  do {                                                     \
+    const wedge_status st__ = (expr);                      \
+    if (st__ != WEDGE_OK) return done(st__);               \
+  } while (0)
 
-  OrientArgs oa;
+  // control words and histogram, then the bins as ranges of ranks (bin_lo, n)
+  const uint32_t nb = inf.n_bins;
+  const size_t n_cnt = (size_t)nb * 4;
+  EXACT_DO(dalloc_n(&cnt, 4 + n_cnt + nb / 2 + 1, s, "wedge_exact"));
+  EXACT_TRY(cudaMemsetAsync(cnt, 0, (4 + n_cnt) * sizeof(unsigned long long), s));
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(cnt);
+  unsigned long long* pbq = cnt + 4;
+  std::vector<uint32_t> bin_lo(nb + 1, 0);  // bin 0: degree 0
+  uint64_t below = (uint64_t)n;
+  for (uint32_t k = 0; k < nb; ++k) below -= inf.n_b[k];
+  for (uint32_t k = 1; k < nb; ++k) {
+    bin_lo[k] = (uint32_t)below;
+    below += inf.n_b[k];
+  }
+  bin_lo[nb] = (uint32_t)n;
+  uint32_t* d_bin_lo = reinterpret_cast<uint32_t*>(pbq + n_cnt);
+  EXACT_TRY(cudaMemcpyAsync(d_bin_lo, bin_lo.data(), (nb + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
+
+  // 1. ranks
+  EXACT_DO(dalloc_n(&rank, 2 * (size_t)n, s, "wedge_exact: ranks"));
+  int32_t* order = rank + n;
+  uint64_t* sorted = nullptr;
+  if (n <= FEW_VERTICES) {
+    EXACT_DO(launch("exact_ranks", s, [&] {
+      k_ranks_few<<<(unsigned)((n + 31) / 32), EX_THREADS, 0, s>>>(g->deg, n, order, rank);
+    }));
+  } else {
+    int deg_bits = 1;
+    while (deg_bits < 31 && (g->max_degree >> deg_bits) != 0) ++deg_bits;
+    EXACT_DO(dalloc_n(&keys, (size_t)n, s, "wedge_exact: ranks"));
+    EXACT_DO(dalloc_n(&alt, (size_t)n, s, "wedge_exact: ranks"));
+    EXACT_DO(dalloc(&scratch, sort_scratch_bytes(n, deg_bits), s, "wedge_exact: ranks"));
+    EXACT_DO(launch("exact_ranks", s, [&] { k_degree_keys<<<blocks_for(n), EX_THREADS, 0, s>>>(g->deg, n, keys); }));
+    EXACT_DO(radix_sort_u64(keys, alt, n, deg_bits, scratch, ctl, s, &sorted, false, 32));
+    EXACT_DO(launch("exact_ranks", s, [&] { k_ranks<<<blocks_for(n), EX_THREADS, 0, s>>>(sorted, n, order, rank); }));
+    dfree(keys, s);
+    dfree(alt, s);
+    dfree(scratch, s);
+    keys = alt = nullptr;
+    scratch = nullptr;
+  }
+
+  // 2. neighbours of lower and higher rank, in-list and row offsets
+  EXACT_DO(dalloc_n(&counts, 5 * (size_t)n, s, "wedge_exact: counts"));
+  EXACT_DO(dalloc_n(&offs, 2 * ((size_t)n + 1), s, "wedge_exact: offsets"));
+  EXACT_DO(dalloc(&scratch, scan_scratch_bytes(n), s, "wedge_exact"));
+  int32_t* lower = counts;
+  int32_t* higher = counts + n;
+  int32_t* taken = counts + 2 * (size_t)n;  // of a vertex's in-list
+  uint32_t* fill = reinterpret_cast<uint32_t*>(counts + 3 * (size_t)n);  // entries per row so far
+  uint32_t* run_end = reinterpret_cast<uint32_t*>(counts + 4 * (size_t)n);
+  int64_t* in_off = offs;
+  int64_t* row_off = offs + (n + 1);
+  EXACT_TRY(cudaMemsetAsync(counts, 0, 4 * (size_t)n * sizeof(int32_t), s));
+  // a warp takes fewer entries where there are too few for all warps
+  const int steps = (int)std::max<int64_t>(1, std::min<int64_t>(OR_STEPS, n_adj / ((int64_t)sm_count() * 64 * 32)));
+  const int64_t tile = (int64_t)EX_WARPS * 32 * steps;
+  const unsigned tiles = (unsigned)((n_adj + tile - 1) / tile);
+  OrientArgs oa{};
   oa.off = g->off;
   oa.adj = g->adj;
-  oa.deg = g->deg;
+  oa.rank = rank;
   oa.n = n;
   oa.n_adj = n_adj;
-  oa.status = status;
-  oa.tile_ctr = derr + 1;
-  oa.err = derr;
-  oa.adjp = adjp;
-  oa.dplus = dplus;
-  st = launch("exact_orient", s, [&] { k_orient<<<(unsigned)tiles, OR_THREADS, 0, s>>>(oa); });
-  if (st != WEDGE_OK) return done(st);
-  if ((st = scan_i32_to_i64(dplus, offp, n, offp + n, nullptr, scratch, derr, s)) != WEDGE_OK) return done(st);
+  oa.steps = steps;
+  oa.lower = lower;
+  oa.higher = higher;
+  EXACT_DO(launch("exact_orient", s, [&] { k_orient<false><<<tiles, EX_THREADS, 0, s>>>(oa); }));
+  EXACT_DO(scan_i32_to_i64(higher, row_off, n, row_off + n, nullptr, scratch, ctl, s));
+  EXACT_DO(scan_counts_to_i64(lower, in_off, n, in_off + n, scratch, ctl, s, "scan_in_counts"));
+  dfree(scratch, s);
+  scratch = nullptr;
+  oa.lower = taken;
 
-  CountArgs ca;
-  ca.offp = offp;
-  ca.adjp = adjp;
-  ca.deg = g->deg;
-  ca.n = n;
-  ca.lo = b->lo_dev;
-  ca.nb = inf.n_bins;
-  ca.pow2 = b->pow2;
-  ca.pbq = cnt;
-  ca.t_i = reinterpret_cast<unsigned long long*>(t_i);
-  ca.next = derr + 2;
-  ca.big = big;
-  ca.big_n = derr + 3;
-  int per_sm = 0;
-  WEDGE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tri_hash_warp, TC_THREADS, 0), "wedge_exact");
-  const unsigned wblocks = (unsigned)(sm_count() * std::max(per_sm, 1));
-  st = launch("exact_hash_warp", s, [&] { k_tri_hash_warp<<<wblocks, TC_THREADS, 0, s>>>(ca); });
-  if (st != WEDGE_OK) return done(st);
-  uint32_t n_big[2] = {0, 0};
-  e = cudaMemcpyAsync(n_big, ca.big_n, sizeof(n_big), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return done(cuda_fail(e, "wedge_exact"));
-  static bool attr_set = false;
-  if (!attr_set) {
-    WEDGE_CUDA_TRY(cudaFuncSetAttribute(k_tri_hash_cta<BIG_THREADS, BIG_SLOTS>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)cta_smem<BIG_THREADS, BIG_SLOTS>()),
-                   "wedge_exact: shared memory");
-    attr_set = true;
-  }
-  if (n_big[0] > 0) {
-    int per = 0;
-    WEDGE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_tri_hash_cta<MID_THREADS, MID_SLOTS>,
-                                                                 MID_THREADS, cta_smem<MID_THREADS, MID_SLOTS>()),
-                   "wedge_exact");
-    const unsigned blocks = (unsigned)std::min<int64_t>((int64_t)n_big[0], (int64_t)sm_count() * std::max(per, 1));
-    st = launch("exact_hash_cta", s, [&] {
-      k_tri_hash_cta<MID_THREADS, MID_SLOTS><<<blocks, MID_THREADS, cta_smem<MID_THREADS, MID_SLOTS>(), s>>>(
-          ca, big, (int32_t)n_big[0], derr + 5);
-    });
-    if (st != WEDGE_OK) return done(st);
-  }
-  if (n_big[1] > 0) {
-    int per = 0;
-    WEDGE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_tri_hash_cta<BIG_THREADS, BIG_SLOTS>,
-                                                                 BIG_THREADS, cta_smem<BIG_THREADS, BIG_SLOTS>()),
-                   "wedge_exact");
-    const unsigned blocks = (unsigned)std::min<int64_t>((int64_t)n_big[1], (int64_t)sm_count() * std::max(per, 1));
-    st = launch("exact_hash_cta_long", s, [&] {
-      k_tri_hash_cta<BIG_THREADS, BIG_SLOTS><<<blocks, BIG_THREADS, cta_smem<BIG_THREADS, BIG_SLOTS>(), s>>>(
-          ca, big + (n - (int32_t)n_big[1]), (int32_t)n_big[1], derr + 6);
-    });
-    if (st != WEDGE_OK) return done(st);
+  // 3-4. groups of ranks, highest first
+  {
+    auto in_at = [&](int32_t r, int64_t* x) {  // in_off[r]
+      cudaError_t e = cudaMemcpyAsync(x, in_off + r, sizeof(*x), cudaMemcpyDeviceToHost, s);
+      return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    };
+    std::vector<std::pair<int32_t, int64_t>> cut{{n, m}};  // ends of the groups, from the top: rank, in_off there
+    const int64_t cap = std::max<int64_t>(GROUP_EDGES, g->max_degree);
+    int64_t largest = m;
+    if (m > cap) {
+      largest = 0;
+      while (cut.back().second > 0) {
+        const int64_t top = cut.back().second;
+        int32_t lo = 0, hi = cut.back().first - 1;  // least rank whose group [rank, end) is at most cap
+        int64_t at = 0;
+        while (lo < hi) {
+          const int32_t mid = lo + (hi - lo) / 2;
+          EXACT_TRY(in_at(mid, &at));
+          if (top - at <= cap) hi = mid; else lo = mid + 1;
+        }
+        EXACT_TRY(in_at(lo, &at));
+        largest = std::max(largest, top - at);
+        cut.push_back({lo, at});
+      }
+    } else {
+      cut.push_back({0, 0});
+    }
+    const uint64_t max_units = (uint64_t)largest / UNIT_IN + (uint64_t)largest / WARP_IN + (uint64_t)m / WARP_ROW + 64;
+    if (largest > (int64_t)UINT32_MAX || max_units > UINT32_MAX)
+      return done(fail(WEDGE_EINVAL, "wedge_exact: graph too large"));
+    const int key_bits = (int)g->id_bits;
+    EXACT_DO(dalloc_n(&keys, (size_t)largest, s, "wedge_exact: edges"));
+    EXACT_DO(dalloc_n(&alt, (size_t)largest, s, "wedge_exact: edges"));
+    EXACT_DO(dalloc(&scratch, sort_scratch_bytes(largest, key_bits), s, "wedge_exact: edges"));
+    EXACT_DO(dalloc_n(&rows, (size_t)m, s, "wedge_exact: rows"));
+    EXACT_DO(dalloc_n(&v_of, (size_t)largest, s, "wedge_exact: edges"));
+    EXACT_DO(dalloc_n(&units, (size_t)max_units, s, "wedge_exact: units"));
+    constexpr auto mid_kernel = k_tri_hash_cta<MID_THREADS, MID_SLOTS, MID_BITS>;
+    constexpr auto big_kernel = k_tri_hash_cta<BIG_THREADS, BIG_SLOTS, BIG_BITS>;
+    constexpr size_t mid_smem = sizeof(CtaSmem<MID_THREADS, MID_SLOTS, MID_BITS>);
+    constexpr size_t big_smem = sizeof(CtaSmem<BIG_THREADS, BIG_SLOTS, BIG_BITS>);
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem);
+    EXACT_TRY(attr);
+    static const int warp_ctas = ctas_per_sm(k_tri_hash_warp, EX_THREADS, 0);
+    static const int mid_ctas = ctas_per_sm(mid_kernel, MID_THREADS, mid_smem);
+    static const int big_ctas = ctas_per_sm(big_kernel, BIG_THREADS, big_smem);
+    const int sms = sm_count();
+    for (size_t gi = 0; gi + 1 < cut.size(); ++gi) {
+      const int32_t r1 = cut[gi].first, r0 = cut[gi + 1].first;
+      const int64_t edges = cut[gi].second - cut[gi + 1].second;
+      if (edges == 0) continue;
+      oa.in_off = in_off;
+      oa.r0 = r0;
+      oa.r1 = r1;
+      oa.keys = keys;
+      oa.v_of = v_of;
+      oa.edges = (uint64_t)edges;
+      EXACT_DO(launch("exact_edges", s, [&] { k_orient<true><<<tiles, EX_THREADS, 0, s>>>(oa); }));
+      EXACT_DO(radix_sort_u64(keys, alt, edges, key_bits, scratch, ctl, s, &sorted, false, 32));
+      rec = reinterpret_cast<uint2*>(sorted == keys ? alt : keys);  // the sort's other buffer
+      EXACT_DO(launch("exact_rows", s, [&] {
+        const unsigned blocks = blocks_for(edges);
+        if (edges == m) {
+          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, v_of, row_off, run_end, fill, rows, m, rec);
+        } else {
+          k_run_ends<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, run_end);
+          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, v_of, row_off, run_end, fill, rows, m, rec);
+          k_run_add<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, run_end, fill);
+        }
+      }));
+      CountArgs ca{};
+      ca.row_off = row_off;
+      ca.rows = rows;
+      ca.in_off = in_off;
+      ca.rec = rec;
+      ca.order = order;
+      ca.bin_lo = d_bin_lo;
+      ca.nb = nb;
+      ca.n = (uint32_t)n;
+      ca.m = m;
+      ca.edges = edges;
+      ca.r0 = r0;
+      ca.r1 = r1;
+      ca.pbq = pbq;
+      ca.t_i = reinterpret_cast<unsigned long long*>(t_i);
+      ca.next = ctl + 1;
+      ca.units = units;
+      ca.max_units = (uint32_t)max_units;
+      ca.n_units = ctl + 2;
+      rec = nullptr;
+      // few vertices to a ticket where there are few for each warp
+      const int64_t warps = (int64_t)sms * warp_ctas * EX_WARPS;
+      ca.grab = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(GRAB, (r1 - r0) / (4 * warps)));
+      if (gi > 0) EXACT_TRY(cudaMemsetAsync(ctl + 1, 0, 5 * sizeof(uint32_t), s));
+      EXACT_DO(launch("exact_hash_warp", s, [&] { k_tri_hash_warp<<<sms * warp_ctas, EX_THREADS, 0, s>>>(ca); }));
+      // (their work lists are on the device; a kernel without work ends at once)
+      EXACT_DO(launch("exact_hash_cta", s, [&] {
+        mid_kernel<<<sms * mid_ctas, MID_THREADS, mid_smem, s>>>(ca, units, 1, ctl + 2, ctl + 4);
+      }));
+      if (g->max_degree > MID_ROW)
+        EXACT_DO(launch("exact_hash_cta_long", s, [&] {
+          big_kernel<<<sms * big_ctas, BIG_THREADS, big_smem, s>>>(ca, units + (max_units - 1), -1, ctl + 3, ctl + 5);
+        }));
+    }
   }
   std::vector<unsigned long long> h(n_cnt);
   uint32_t herr = 0;
-  e = cudaMemcpyAsync(h.data(), cnt, n_cnt * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return done(cuda_fail(e, "wedge_exact"));
+  EXACT_TRY(cudaMemcpyAsync(h.data(), pbq, n_cnt * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  EXACT_TRY(cudaMemcpyAsync(&herr, ctl, sizeof(herr), cudaMemcpyDeviceToHost, s));
+  EXACT_TRY(cudaStreamSynchronize(s));
+#undef EXACT_TRY
+#undef EXACT_DO
   if (herr & DERR_TIMEOUT) return done(fail(WEDGE_ETIMEOUT, "wedge_exact: a look-back wait gave up"));
   uint64_t closed = 0;
   for (uint32_t k = 0; k < inf.n_bins; ++k) {

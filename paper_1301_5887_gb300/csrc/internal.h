@@ -106,6 +106,9 @@ size_t scan_scratch_bytes(int64_t n);
 // If maxv != nullptr, atomicMax(maxv, max input) (inputs interpreted as int32).
 wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, int32_t* maxv, void* scratch,
                              uint32_t* derr, cudaStream_t s);
+// The same under a name of its own.
+wedge_status scan_counts_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch,
+                                uint32_t* derr, cudaStream_t s, const char* name);
 // out[i] = sum in[0..i) for i < n and out[n] = the total (out holds n + 1).
 wedge_status scan_u32_with_total(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s);

@@ -161,6 +161,11 @@ wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t
   return run_scan<int32_t, int64_t>(in, out, n, total, maxv, scratch, derr, s, "scan_degrees");
 }
 
+wedge_status scan_counts_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch,
+                                uint32_t* derr, cudaStream_t s, const char* name) {
+  return run_scan<int32_t, int64_t>(in, out, n, total, nullptr, scratch, derr, s, name);
+}
+
 wedge_status scan_u32_with_total(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s) {
   return run_scan<uint32_t, int64_t>(in, out, n, out + n, nullptr, scratch, derr, s, "scan_bin_counts");
