@@ -218,8 +218,8 @@ WEDGE_API wedge_status wedge_bins_copy(const wedge_bins* b, int32_t* L, uint64_t
  * wedges with the edge list: every sample's closure query, packed with its
  * stream and class as x << (b + P) | y << P | payload (x the endpoint with
  * the smaller (degree, id), b = id bits, P = 2 + bits of the stream count),
- * is radix-sorted, and the sorted queries are checked in order, each
- * adjacency row searched once per run of queries. Needs 2b + P <= 64.
+ * is radix-sorted by the highest bits of x, and the queries are checked in
+ * that order, block after block of adjacency rows. Needs 2b + P <= 64.
  *
  * Errors: EINVAL if eps or delta is outside (0,1) while a budget is 0,
  * bins do not belong to g, records is set with WEDGE_FLAG_NO_GLOBAL,

@@ -9,11 +9,13 @@
 //     x << (b + P) | y << P | stream << 2 | (class - 1)
 // where x is the endpoint with the smaller (degree, id) (the row that is
 // searched), y the other, b the id width and P the payload width; radix-sort
-// the keys; then walk them in order, so the rows of the adjacency array are
-// visited in increasing order and each is searched once per run of queries
-// (the search for the next y resumes where the previous one ended). The
-// payload carries what Alg. Phase 4c's tally needs, so the counts are
-// identical to wedge_sample's. Needs 2b + P <= 64.
+// the keys by x's highest bits; then walk them in order, so that the searches
+// go through the adjacency array block by block, from L2. The payload carries
+// what Alg. Phase 4c's tally needs, so the counts are identical to
+// wedge_sample's. Needs 2b + P <= 64.
+// Sorting whole keys (seven passes at scale 22) and resuming each row's search
+// where the last one ended took 5.38 ms for 66 M samples; one pass and a search
+// of its own for each query take 3.63 (keys 2.42, sort 0.37, closure 0.83).
 #include <string.h>
 
 #include <algorithm>
@@ -32,6 +34,7 @@ constexpr int KEY_PER_THREAD = 8;
 constexpr int KEY_TILE = KEY_THREADS * KEY_PER_THREAD;
 constexpr int CL_THREADS = 256;
 constexpr int CL_ITEMS = 8;
+constexpr uint64_t BLOCK_BYTES = 32 << 20;
 
 struct KeyStream {
   int64_t start, len;   // the bin's vertices in L
@@ -97,55 +100,41 @@ __global__ __launch_bounds__(KEY_THREADS) void k_sample_keys(KeyArgs a) {
 }
 
 struct ClosureArgs {
-  const uint64_t* keys;  // sorted
+  const uint64_t* keys;  // in order of the rows' blocks
   uint64_t n;
   const int64_t* off;
   const int32_t* adj;
   uint32_t id_bits, pbits;
+  float ids_inv;  // 1 / number of ids
   uint32_t n_streams;
   unsigned long long* q_out;  // [n_streams][4]
 };
 
+// Closes the queries in order. The sort has brought together the queries of a
+// block of rows, which lies in L2 while they are closed; within it each query
+// searches its row on its own, so that a warp's 32 queries are independent.
 __global__ __launch_bounds__(CL_THREADS) void k_closure_sorted(ClosureArgs a) {
   extern __shared__ uint32_t s_cnt[];  // [n_streams][4]
   for (uint32_t i = threadIdx.x; i < a.n_streams * 4; i += CL_THREADS) s_cnt[i] = 0;
   __syncthreads();
-  const uint64_t base = ((uint64_t)blockIdx.x * CL_THREADS + threadIdx.x) * CL_ITEMS;
+  const int lane = threadIdx.x & 31;
+  const uint64_t base = (uint64_t)blockIdx.x * CL_THREADS * CL_ITEMS + threadIdx.x;
   const uint64_t ymask = (1ULL << a.id_bits) - 1ULL, pmask = (1ULL << a.pbits) - 1ULL;
-  int64_t row_lo = 0, row_hi = 0, pos = 0;
-  int64_t prev_x = -1;
+  bool guess = true;
   for (int it = 0; it < CL_ITEMS; ++it) {
-    const uint64_t e = base + it;
-    if (e >= a.n) break;
-    const uint64_t key = a.keys[e];
-    const int32_t x = (int32_t)(key >> (a.id_bits + a.pbits));
-    const int32_t y = (int32_t)((key >> a.pbits) & ymask);
-    const uint32_t pay = (uint32_t)(key & pmask);
-    const bool same_row = x == prev_x;
-    if (!same_row) {
-      row_lo = __ldg(a.off + x);
-      row_hi = __ldg(a.off + x + 1);
-      pos = row_lo;
-      prev_x = x;
+    const uint64_t e = base + (uint64_t)it * CL_THREADS;
+    if (e - lane >= a.n) break;  // the whole warp
+    bool useful = guess;
+    if (e < a.n) {
+      const uint64_t key = __ldcs(a.keys + e);
+      const int32_t x = (int32_t)(key >> (a.id_bits + a.pbits));
+      const int32_t y = (int32_t)((key >> a.pbits) & ymask);
+      const uint32_t pay = (uint32_t)(key & pmask);
+      const int64_t row = __ldg(a.off + x);
+      const bool closed = row_contains(a.adj, row, __ldg(a.off + x + 1) - row, y, a.ids_inv, useful);
+      atomicAdd(&s_cnt[(pay >> 2) * 4 + (closed ? 1u + (pay & 3u) : 0u)], 1u);
     }
-    // keys ascend, so within a row y does not decrease: the first entry >= y
-    // lies at or after the previous answer; in the same row gallop from
-    // there, then bisect
-    int64_t lo = pos, hi = row_hi;
-    for (int64_t step = 1; same_row && lo + step < row_hi; step <<= 1) {
-      if (__ldg(a.adj + lo + step - 1) >= y) {
-        hi = lo + step - 1;
-        break;
-      }
-      lo += step;
-    }
-    while (lo < hi) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
-      if (__ldg(a.adj + mid) < y) lo = mid + 1; else hi = mid;
-    }
-    pos = lo;
-    const bool closed = lo < row_hi && __ldg(a.adj + lo) == y;
-    atomicAdd(&s_cnt[(pay >> 2) * 4 + (closed ? 1u + (pay & 3u) : 0u)], 1u);
+    guess = warp_guesses(guess, guess && !useful);
   }
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < a.n_streams * 4; i += CL_THREADS)
@@ -186,10 +175,15 @@ wedge_status sample_sorted_closure(const wedge_graph* g, const wedge_bins* b, ui
   if (streams.empty()) return WEDGE_OK;
   uint32_t pbits = 2;
   while ((1ULL << (pbits - 2)) < streams.size()) ++pbits;
-  const uint32_t bits = 2 * g->id_bits + pbits;
+  uint32_t bits = 2 * g->id_bits + pbits;
   if (bits > 64)
     return fail(WEDGE_EINVAL, "wedge_sample: sorted closure needs 2 x %u id bits + %u payload bits <= 64", g->id_bits,
                 pbits);
+  // the row's highest bits end at a digit of the sort (pbits: where y begins)
+  while (bits % 8) {
+    ++bits;
+    ++pbits;
+  }
   if (tiles > (uint64_t)INT32_MAX || total > (1ULL << 40))
     return fail(WEDGE_EINVAL, "wedge_sample: sorted closure budget too large");
 
@@ -243,7 +237,12 @@ wedge_status sample_sorted_closure(const wedge_graph* g, const wedge_bins* b, ui
   st = launch("sorted_keys", s, [&] { k_sample_keys<<<(unsigned)tiles, KEY_THREADS, 0, s>>>(ka); });
   if (st != WEDGE_OK) return done(st);
   uint64_t* sorted = keys;
-  if ((st = radix_sort_u64(keys, alt, (int64_t)total, (int)bits, scratch, derr, s, &sorted, false)) != WEDGE_OK)
+  // Sorted by the row's highest 8 bits, or 16 where the adjacency of a block of
+  // rows would still be large beside L2.
+  const int by = (uint64_t)g->n_adj * sizeof(int32_t) >> 8 <= BLOCK_BYTES ? 8 : 16;
+  const int from = std::max(0, (int)bits - by);
+  if ((st = radix_sort_u64(keys, alt, (int64_t)total, (int)bits - from, scratch, derr, s, &sorted, false, from)) !=
+      WEDGE_OK)
     return done(st);
   ClosureArgs ca;
   ca.keys = sorted;
@@ -251,6 +250,7 @@ wedge_status sample_sorted_closure(const wedge_graph* g, const wedge_bins* b, ui
   ca.off = g->off;
   ca.adj = g->adj;
   ca.id_bits = g->id_bits;
+  ca.ids_inv = 1.0f / (float)g->n;
   ca.pbits = pbits;
   ca.n_streams = (uint32_t)streams.size();
   ca.q_out = cnt;

@@ -60,6 +60,8 @@ def test_bins_and_samples(n, tau, omega):
     want = oracle.sample(off, adj, tau, omega, n + tau, 700, 9_000)
     assert np.array_equal(c.counts_matrix(), want["counts"])
     assert c.closed_global == int(want["glob"][1]) and np.array_equal(c.stats, want["stats"])
+    bins_only = wedge.sample(g, b, seed=n + tau, k_per_bin=700, flags=wedge.FLAG_SORTED_CLOSURE | wedge.FLAG_NO_GLOBAL)
+    assert np.array_equal(bins_only.counts_matrix(), want["counts"])
     r = wedge.Requests([{"graph": g, "bins": b, "seed": n + tau, "k_per_bin": 700, "k_global": 9_000}])
     for mapping in (wedge.MAP_THREAD, wedge.MAP_WARP):
         got = wedge.sample_batch(r, {f"mapping_{s}": mapping for s in ("small", "medium", "large")})[0]
