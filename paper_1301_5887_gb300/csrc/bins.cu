@@ -22,6 +22,7 @@ namespace {
 
 constexpr int BIN_THREADS = 256;
 constexpr int BIN_WARPS = BIN_THREADS / 32;
+constexpr int64_t SMALL_MATRIX = 4096;  // (bin, tile) counts
 constexpr int BIN_ITEMS = 16;
 constexpr int BIN_TILE = BIN_THREADS * BIN_ITEMS;
 
@@ -78,12 +79,14 @@ __host__ __device__ inline uint32_t mat_row(uint32_t b, uint32_t nb) { return b 
 // degrees takes 10).
 __global__ __launch_bounds__(BIN_THREADS) void k_bin_count(const int32_t* __restrict__ deg, int32_t n,
                                                            const uint64_t* __restrict__ lo_g, uint32_t nb,
-                                                           int64_t n_tiles, uint32_t* __restrict__ mat_cnt) {
+                                                           int64_t n_tiles, uint32_t* __restrict__ mat_cnt,
+                                                           uint32_t* err) {
   __shared__ DegreeBins s_bins;
   extern __shared__ uint32_t s_n[];  // [bin][lane]
   const int tid = threadIdx.x;
   const int64_t tile = blockIdx.x;
   const int64_t tbase = tile * BIN_TILE;
+  if (tile == 0 && tid == 0) *err = 0u;  // first in the stream: nothing has been reported yet
   int4 d[BIN_ITEMS / 4];
 #pragma unroll
   for (int i = 0; i < BIN_ITEMS / 4; ++i) d[i] = load_degrees(deg, n, tbase + 4 * (i * BIN_THREADS + tid));
@@ -397,22 +400,18 @@ extern "C" wedge_status wedge_bin(const wedge_graph* g, const wedge_bin_params* 
   uint32_t* mat_cnt = nullptr;
   int64_t* pos_base = nullptr;
   int32_t* ldeg = nullptr;  // degree per entry of L; its C(d,2) are scanned into W
-  unsigned long long* sums = nullptr;  // W at the nb + 1 bin boundaries, then the nb + 1 bin starts
+  // (pos_base is followed by, in 8-byte words: the error word, W at the nb + 1
+  // bin boundaries, the nb + 1 bin starts; what the host reads lies together)
   void* scratch = nullptr;
-  uint32_t* derr = nullptr;
   auto release_tmp = [&]() {
     dfree(mat_cnt, s);
     dfree(pos_base, s);
     dfree(ldeg, s);
-    dfree(sums, s);
     dfree(scratch, s);
-    dfree(derr, s);
     mat_cnt = nullptr;
     pos_base = nullptr;
     ldeg = nullptr;
-    sums = nullptr;
     scratch = nullptr;
-    derr = nullptr;
   };
   auto bail = [&](wedge_status e) {
     release_tmp();
@@ -426,29 +425,36 @@ extern "C" wedge_status wedge_bin(const wedge_graph* g, const wedge_bin_params* 
   wedge_status st;
   if ((st = dalloc_n(&b->lo_dev, nb, s, "wedge_bin")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&mat_cnt, (size_t)mat, s, "wedge_bin")) != WEDGE_OK) return bail(st);
-  if ((st = dalloc_n(&pos_base, (size_t)mat + 1, s, "wedge_bin")) != WEDGE_OK) return bail(st);
-  if ((st = dalloc_n(&sums, 2 * (size_t)nb + 2, s, "wedge_bin")) != WEDGE_OK) return bail(st);
+  if ((st = dalloc_n(&pos_base, (size_t)mat + 2 * (size_t)nb + 4, s, "wedge_bin")) != WEDGE_OK) return bail(st);
   if ((st = dalloc(&scratch, scan_scratch_bytes(mat), s, "wedge_bin")) != WEDGE_OK) return bail(st);
-  if ((st = dalloc_n(&derr, 64, s, "wedge_bin")) != WEDGE_OK) return bail(st);
+  uint32_t* derr = reinterpret_cast<uint32_t*>(pos_base + mat + 1);
+  unsigned long long* sums = reinterpret_cast<unsigned long long*>(pos_base + mat + 2);
   BIN_TRY(cudaMemcpyAsync(b->lo_dev, lo.data(), nb * sizeof(uint64_t), cudaMemcpyHostToDevice, s), "wedge_bin");
-  BIN_TRY(cudaMemsetAsync(derr, 0, 64 * sizeof(uint32_t), s), "wedge_bin");
 
   st = launch("bin_count", s, [&] {
-    k_bin_count<<<(unsigned)n_tiles, BIN_THREADS, nb * 32 * sizeof(uint32_t), s>>>(g->deg, n, b->lo_dev, nb, n_tiles, mat_cnt);
+    k_bin_count<<<(unsigned)n_tiles, BIN_THREADS, nb * 32 * sizeof(uint32_t), s>>>(g->deg, n, b->lo_dev, nb, n_tiles, mat_cnt,
+                                                                                     derr);
   });
   if (st != WEDGE_OK) return bail(st);
   if ((st = scan_u32_with_total(mat_cnt, pos_base, mat, scratch, derr, s)) != WEDGE_OK) return bail(st);
 
   // the matrix rows' starts (one entry a row), and the total
-  std::vector<int64_t> rows(nb);
-  std::vector<unsigned long long> bound(nb + 1, 0);
-  uint32_t herr = 0;
-  BIN_TRY(cudaMemcpy2DAsync(rows.data(), sizeof(int64_t), pos_base, (size_t)n_tiles * sizeof(int64_t), sizeof(int64_t),
-                            nb - 1, cudaMemcpyDeviceToHost, s),
-          "wedge_bin");
-  BIN_TRY(cudaMemcpyAsync(&rows[nb - 1], pos_base + mat, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "wedge_bin");
-  BIN_TRY(cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost, s), "wedge_bin");
-  BIN_TRY(cudaStreamSynchronize(s), "wedge_bin");
+  std::vector<int64_t> rows(nb + 1);
+  std::vector<unsigned long long> bound(nb + 2, 0);  // the error word, W at the bin boundaries
+  if (mat <= SMALL_MATRIX) {  // one copy of all of it is shorter than two of parts
+    std::vector<int64_t> all((size_t)mat + 2);
+    BIN_TRY(cudaMemcpyAsync(all.data(), pos_base, all.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s), "wedge_bin");
+    BIN_TRY(cudaStreamSynchronize(s), "wedge_bin");
+    for (uint32_t r = 0; r < nb; ++r) rows[r] = all[(size_t)r * n_tiles];  // (nb - 1 rows, and the total)
+    rows[nb] = all[(size_t)mat + 1];
+  } else {
+    BIN_TRY(cudaMemcpy2DAsync(rows.data(), sizeof(int64_t), pos_base, (size_t)n_tiles * sizeof(int64_t),
+                              sizeof(int64_t), nb - 1, cudaMemcpyDeviceToHost, s),
+            "wedge_bin");
+    BIN_TRY(cudaMemcpyAsync(&rows[nb - 1], pos_base + mat, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s), "wedge_bin");
+    BIN_TRY(cudaStreamSynchronize(s), "wedge_bin");
+  }
+  uint32_t herr = (uint32_t)rows[nb];
   if (herr & DERR_TIMEOUT) return bail(fail(WEDGE_ETIMEOUT, "wedge_bin: a look-back wait gave up"));
 
   wedge_bins_info& inf = b->info;
@@ -500,17 +506,17 @@ extern "C" wedge_status wedge_bin(const wedge_graph* g, const wedge_bin_params* 
       k_bin_guide<<<(unsigned)gblocks, BIN_THREADS, 0, s>>>(b->W, n2, starts, b->gtab, nb, b->guide, guide_len, derr);
     });
     if (st != WEDGE_OK) return bail(st);
-    BIN_TRY(cudaMemcpyAsync(bound.data(), sums, (nb + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, s), "wedge_bin");
-    BIN_TRY(cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost, s), "wedge_bin");
+    BIN_TRY(cudaMemcpyAsync(bound.data(), derr, (nb + 2) * sizeof(uint64_t), cudaMemcpyDeviceToHost, s), "wedge_bin");
   } else {
     BIN_TRY(cudaMemsetAsync(b->W, 0, sizeof(uint64_t), s), "wedge_bin");
   }
   BIN_TRY(cudaStreamSynchronize(s), "wedge_bin");
+  herr = (uint32_t)bound[0];
   if (herr & DERR_TIMEOUT) return bail(fail(WEDGE_ETIMEOUT, "wedge_bin: a look-back wait gave up"));
   if (herr & DERR_BOUNDS) return bail(fail(WEDGE_ECUDA, "wedge_bin: an index outside its buffer (bounds-checked build)"));
   // p_b: the wedge prefix across bin b's stretch of L
-  for (uint32_t k = 0; k < nb; ++k) inf.p_b[k] = bound[k + 1] - bound[k];
-  inf.p_total = bound[nb];
+  for (uint32_t k = 0; k < nb; ++k) inf.p_b[k] = bound[k + 2] - bound[k + 1];
+  inf.p_total = bound[nb + 1];
   release_tmp();
   inf.L = b->L;
   inf.W = b->W;

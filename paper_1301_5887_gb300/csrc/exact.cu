@@ -734,7 +734,7 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
     EXACT_DO(dalloc_n(&alt, (size_t)n, s, "wedge_exact: ranks"));
     EXACT_DO(dalloc(&scratch, sort_scratch_bytes(n, deg_bits), s, "wedge_exact: ranks"));
     EXACT_DO(launch("exact_ranks", s, [&] { k_degree_keys<<<blocks_for(n), EX_THREADS, 0, s>>>(g->deg, n, keys); }));
-    EXACT_DO(radix_sort_u64(keys, alt, n, deg_bits, scratch, ctl, s, &sorted, false, 32));
+    EXACT_DO(radix_sort_u64(keys, alt, n, deg_bits, scratch, ctl, s, &sorted, SortScratch::unused, 32));
     EXACT_DO(launch("exact_ranks", s, [&] { k_ranks<<<blocks_for(n), EX_THREADS, 0, s>>>(sorted, n, order, rank); }));
     dfree(keys, s);
     dfree(alt, s);
@@ -834,7 +834,7 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
       oa.v_of = v_of;
       oa.edges = (uint64_t)edges;
       EXACT_DO(launch("exact_edges", s, [&] { k_orient<true><<<tiles, EX_THREADS, 0, s>>>(oa); }));
-      EXACT_DO(radix_sort_u64(keys, alt, edges, key_bits, scratch, ctl, s, &sorted, false, 32));
+      EXACT_DO(radix_sort_u64(keys, alt, edges, key_bits, scratch, ctl, s, &sorted, SortScratch::unused, 32));
       rec = reinterpret_cast<uint2*>(sorted == keys ? alt : keys);  // the sort's other buffer
       EXACT_DO(launch("exact_rows", s, [&] {
         const unsigned blocks = blocks_for(edges);

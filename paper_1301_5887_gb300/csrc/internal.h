@@ -49,12 +49,14 @@ namespace wedge {
 
 // Sort-scratch size and sort (sort.cu). The scratch starts with the digit
 // histograms (8 passes x 256 unsigned long long); a caller that produces the
-// keys may accumulate them there itself (sort_clear_hist first) and pass
-// hist_ready = true.
+// keys may accumulate them there itself: after sort_clear for that many keys
+// (cleared), or after clearing the histograms alone (histograms), which leaves
+// the rest of the scratch free for other uses until the sort.
+enum class SortScratch { unused, histograms, cleared };
 constexpr int SORT_MAX_PASSES = 8;
 size_t sort_scratch_bytes(int64_t n, int bits);
 unsigned long long* sort_hist_area(void* scratch);
-wedge_status sort_clear_hist(void* scratch, cudaStream_t s);
+wedge_status sort_clear(void* scratch, int64_t n, cudaStream_t s);
 // Placement by the last pass of a sort of transposed keys (w << 32) | u: the
 // key at sorted position j writes u to adj[j + row_start[w]] and counts one
 // for w in count[w] (instead of being written out).
@@ -83,11 +85,12 @@ struct SortEdges {
 // first_pass_unstable: every nonzero bit of every key lies in the sorted range
 // (keys equal in it are identical) and the lowest digit is evenly spread, so
 // the first pass may rank by one shared atomic per key without stability.
-// edges (shift0 = 0, first_pass_unstable, hist_ready): the first pass computes
+// edges (shift0 = 0, first_pass_unstable, cleared): the first pass computes
 // the keys from the edge list; keys is not read (it is written by later
 // passes, as without edges).
 wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, void* scratch, uint32_t* derr,
-                            cudaStream_t s, uint64_t** sorted, bool hist_ready, int shift0 = 0,
+                            cudaStream_t s, uint64_t** sorted, SortScratch ready = SortScratch::unused,
+                            int shift0 = 0,
                             const SortEmit* emit = nullptr, bool first_pass_unstable = false,
                             const SortEdges* edges = nullptr);
 

@@ -26,7 +26,11 @@ namespace {
 
 constexpr int SAMPLE_THREADS = 256;
 constexpr int SAMPLE_PER_THREAD = 8;
-constexpr int SAMPLE_TILE = SAMPLE_THREADS * SAMPLE_PER_THREAD;
+// A budget too small to give every SM this many CTAs takes fewer samples a
+// thread: each sample is a chain of dependent loads, so a thread's samples one
+// after the other are the kernel's time (210,000 samples of a scale-12 graph:
+// 33 us at 8 a thread, 19 at 1).
+constexpr int SAMPLE_MIN_CTAS = 4;
 
 struct StreamDesc {
   int64_t start;        // first index of the stream's vertices in L
@@ -53,6 +57,7 @@ struct SampleArgs {
   uint32_t nb;
   uint32_t pow2;
   uint32_t seed_lo, seed_hi;
+  int per_thread;              // samples of a thread: a CTA's tile is per_thread * SAMPLE_THREADS
   unsigned long long* q_out;   // [n_streams][4]
   unsigned long long* stats;   // [WEDGE_STAT_BINS][WEDGE_STAT_BINS]
   wedge_record* records;       // global stream records or nullptr
@@ -88,10 +93,10 @@ __global__ __launch_bounds__(SAMPLE_THREADS) void k_sample(SampleArgs a) {
   const GraphView gv{a.off, a.adj, a.L, a.W, a.guide, 1.0f / (float)a.n, a.n, a.n_adj, a.n_L, a.err};
   const bool global = desc.tag != 0;
   const GuideRange gr{s_gtab, global ? 2u : desc.bin, global ? a.nb : desc.bin + 1u};
-  const uint64_t first = ((uint64_t)blockIdx.x - desc.tile_begin) * SAMPLE_TILE;
+  const uint64_t first = ((uint64_t)blockIdx.x - desc.tile_begin) * (uint32_t)(SAMPLE_THREADS * a.per_thread);
   uint32_t q0 = 0, q1 = 0, q2 = 0, q3 = 0;
   bool guess = true;
-  for (int j = 0; j < SAMPLE_PER_THREAD; ++j) {
+  for (int j = 0; j < a.per_thread; ++j) {
     const uint64_t local = first + (uint64_t)j * SAMPLE_THREADS + tid;
     if (local - lane >= desc.k) break;  // the whole warp
     bool lost = false;
@@ -230,10 +235,8 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
     d.wbase = wbase;
     d.k = k;
     d.first = sp->first_sample;
-    d.tile_begin = tiles;
     d.bin = bin;
     d.tag = tag;
-    tiles += (k + SAMPLE_TILE - 1) / SAMPLE_TILE;
     streams.push_back(d);
     stream_bin.push_back(tag == 0 ? (int)bin : -1);
   };
@@ -245,6 +248,15 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
     wacc += inf.p_b[k];
   }
   add(0, inf.n_wedge_vertices, inf.p_total, k_glob, 0u, 1u, 0ULL);
+  double budget = 0;
+  for (const StreamDesc& d : streams) budget += (double)d.k;
+  const double fills = budget / ((double)SAMPLE_THREADS * SAMPLE_MIN_CTAS * sm_count());
+  const int per_thread = fills >= SAMPLE_PER_THREAD ? SAMPLE_PER_THREAD : std::max(1, (int)fills);
+  const uint64_t tile_samples = (uint64_t)SAMPLE_THREADS * per_thread;
+  for (StreamDesc& d : streams) {
+    d.tile_begin = tiles;
+    tiles += (d.k + tile_samples - 1) / tile_samples;
+  }
   if (tiles > (uint64_t)INT32_MAX) return fail(WEDGE_EINVAL, "wedge_sample: sample budget too large");
 
   memset(out, 0, sizeof(*out));
@@ -291,6 +303,7 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
   a.pow2 = b->pow2;
   a.seed_lo = (uint32_t)sp->seed;
   a.seed_hi = (uint32_t)(sp->seed >> 32);
+  a.per_thread = per_thread;
   a.q_out = d_cnt;
   a.stats = d_cnt + streams.size() * 4;
   a.records = static_cast<wedge_record*>(sp->records);

@@ -42,7 +42,7 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restric
   __shared__ uint32_t s_tile;
   __shared__ Tout s_excl;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
+  if (tid == 0) s_tile = tile_ctr ? atomicAdd(tile_ctr, 1u) : 0u;  // nullptr: the only tile
   __syncthreads();
   const int64_t tile = s_tile;
   const int64_t tbase = tile * SCAN_TILE;
@@ -138,9 +138,10 @@ wedge_status run_scan(const Tin* in, Tout* out, int64_t n, Tout* total, int32_t*
   }
   const int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (tiles > (int64_t)UINT32_MAX) return fail(WEDGE_EINVAL, "%s: too many items (%lld)", name, (long long)n);
-  uint32_t* ctr = static_cast<uint32_t*>(scratch);
+  // a single tile waits for none and needs no cleared words
+  uint32_t* ctr = tiles > 1 ? static_cast<uint32_t*>(scratch) : nullptr;
   uint64_t* status = reinterpret_cast<uint64_t*>(static_cast<char*>(scratch) + 256);
-  WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, 256 + (size_t)tiles * sizeof(uint64_t), s), name);
+  if (tiles > 1) WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, 256 + (size_t)tiles * sizeof(uint64_t), s), name);
   // L2 prefetch about one wave of CTAs ahead (six 34 KB tile buffers fit an SM)
   const int64_t prefetch = (reinterpret_cast<uintptr_t>(in) & 15) == 0 ? 6 * (int64_t)sm_count() : 0;
   return launch(name, s, [&] {

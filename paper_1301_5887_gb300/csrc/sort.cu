@@ -10,6 +10,7 @@
 // equal digits contiguously. Each CTA also asks the L2 to prefetch the tile
 // that will be claimed one wave of CTAs later (a bulk prefetch), so a tile's
 // loads mostly hit L2 instead of waiting on HBM.
+// A sort of at most one 1536-key tile per SM takes those small tiles instead.
 //
 // Only `bits` bits from bit `shift0` up are sorted (shift0 a multiple of 8),
 // 8 bits per pass; stable, so the result is sorted by that bit range and keeps
@@ -18,6 +19,8 @@
 // and whose lowest digit is evenly spread may let the first pass, whose input
 // order carries no meaning, rank without stability (one shared atomic per key,
 // which slows down where many keys of a warp share a digit).
+#include <algorithm>
+
 #include "device.cuh"
 #include "internal.h"
 #include "runtime.h"
@@ -32,6 +35,8 @@ constexpr int SORT_WARPS = SORT_THREADS / 32;
 constexpr int SORT_ITEMS = 16;
 constexpr int SORT_MIN_BLOCKS = 3;  // resident CTAs per SM the register budget must allow
 constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;  // 6144 keys
+constexpr int SMALL_ITEMS = 4;
+constexpr int SMALL_TILE = SORT_THREADS * SMALL_ITEMS;  // 1536 keys
 constexpr int MAX_PASSES = SORT_MAX_PASSES;
 constexpr int HIST_THREADS = 256;
 
@@ -60,31 +65,13 @@ __global__ __launch_bounds__(HIST_THREADS) void k_sort_hist(const uint64_t* __re
     if (sh[i]) atomicAdd(&hist[i], (unsigned long long)sh[i]);
 }
 
-// Exclusive scan of each pass's 256-bin histogram: the global start of each digit.
-__global__ __launch_bounds__(RADIX) void k_sort_base(const unsigned long long* __restrict__ hist,
-                                                     uint64_t* __restrict__ base) {
-  __shared__ uint64_t s_w[RADIX / 32];
-  const int p = blockIdx.x, d = threadIdx.x, lane = d & 31, warp = d >> 5;
-  const uint64_t v = hist[p * RADIX + d];
-  uint64_t incl = v;
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t y = __shfl_up_sync(FULL_MASK, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) s_w[warp] = incl;
-  __syncthreads();
-  uint64_t pre = 0;
-  for (int w = 0; w < warp; ++w) pre += s_w[w];
-  base[p * RADIX + d] = pre + incl - v;
-}
-
 struct PassArgs {
   const uint64_t* in;
   uint64_t* out;
   int64_t n;
   uint32_t shift;
   uint32_t epoch;
-  const uint64_t* base;  // RADIX digit starts for this pass
+  const unsigned long long* hist;  // RADIX digit counts for this pass
   uint64_t* status;      // tiles * RADIX look-back words
   uint32_t* tile_ctr;
   uint32_t* err;
@@ -94,15 +81,15 @@ struct PassArgs {
   uint32_t edge_prefetch;  // bit 0: src, bit 1: dst 16-byte aligned (L2 prefetch allowed)
 };
 
+template <int ITEMS>
 struct PassSmem {
-  uint64_t keys[SORT_TILE];           // tile in digit order
+  uint64_t keys[SORT_THREADS * ITEMS];  // tile in digit order
   uint64_t goff[RADIX];               // global index - local position, per digit
   uint32_t whist[SORT_WARPS][RADIX];  // per-warp digit counts, then running positions
   uint32_t dstart[RADIX];             // tile-local start of each digit
   uint32_t wsum[SORT_WARPS];
   uint32_t tile;
 };
-constexpr size_t PASS_SMEM = sizeof(PassSmem);
 
 // Digit of a key: byte `sel` of its high (HI) or low 32-bit half (digits are
 // byte-aligned, so one never straddles the halves).
@@ -141,13 +128,13 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d) {
 // the tile position of this warp's next key of digit d: every peer reads it,
 // the lowest peer advances it past the group, and each key lands at that
 // position plus the number of its peers in lower lanes.
-template <bool HI, bool FULL, int RB>
-__device__ __forceinline__ void rank_stable(PassSmem& sm, const uint64_t (&k)[SORT_ITEMS], uint32_t sel, int nvalid,
+template <bool HI, bool FULL, int RB, int ITEMS>
+__device__ __forceinline__ void rank_stable(PassSmem<ITEMS>& sm, const uint64_t (&k)[ITEMS], uint32_t sel, int nvalid,
                                             int warp, int lane, uint32_t* err) {
   const uint32_t lt = lanemask_lt();
 #pragma unroll
-  for (int i = 0; i < SORT_ITEMS; ++i) {
-    const int li = warp * (32 * SORT_ITEMS) + i * 32 + lane;
+  for (int i = 0; i < ITEMS; ++i) {
+    const int li = warp * (32 * ITEMS) + i * 32 + lane;
     const bool has = FULL || li < nvalid;
     const uint32_t d = has ? digit_of<HI>(k[i], sel) : (uint32_t)RADIX;
     const uint32_t peers = digit_peers<FULL, RB>(d);
@@ -157,7 +144,7 @@ __device__ __forceinline__ void rank_stable(PassSmem& sm, const uint64_t (&k)[SO
     if (has) {
       if (below == 0) sm.whist[warp][d] = next + __popc(peers);
       const uint32_t pos = next + __popc(below);
-      if (in_bounds(pos, SORT_TILE, err)) sm.keys[pos] = k[i];
+      if (in_bounds(pos, SORT_THREADS * ITEMS, err)) sm.keys[pos] = k[i];
     }
     __syncwarp();
   }
@@ -165,22 +152,22 @@ __device__ __forceinline__ void rank_stable(PassSmem& sm, const uint64_t (&k)[SO
 
 // Unstable rank: each key takes the next position of its digit in its warp's
 // range by a shared atomic (the order among equal digits is arbitrary).
-template <bool HI>
-__device__ __forceinline__ void rank_unstable(PassSmem& sm, const uint64_t (&k)[SORT_ITEMS], uint32_t sel, int nvalid,
+template <bool HI, int ITEMS>
+__device__ __forceinline__ void rank_unstable(PassSmem<ITEMS>& sm, const uint64_t (&k)[ITEMS], uint32_t sel, int nvalid,
                                               int warp, int lane, uint32_t* err) {
 #pragma unroll
-  for (int i = 0; i < SORT_ITEMS; ++i) {
-    const int li = warp * (32 * SORT_ITEMS) + i * 32 + lane;
+  for (int i = 0; i < ITEMS; ++i) {
+    const int li = warp * (32 * ITEMS) + i * 32 + lane;
     if (li < nvalid) {
       const uint32_t pos = atomicAdd(&sm.whist[warp][digit_of<HI>(k[i], sel)], 1u);
-      if (in_bounds(pos, SORT_TILE, err)) sm.keys[pos] = k[i];
+      if (in_bounds(pos, SORT_THREADS * ITEMS, err)) sm.keys[pos] = k[i];
     }
   }
 }
 
-// One LSD pass over a 6144-key tile (three CTAs per SM; the 256 digit owners
-// are threads 0..255):
-//  1. claim a tile, ask L2 to prefetch the tile one wave ahead, load 16 keys
+// One LSD pass over a 6144-key tile (three CTAs per SM; ITEMS = 4: a 1536-key
+// tile; the 256 digit owners are threads 0..255):
+//  1. claim a tile, ask L2 to prefetch the tile one wave ahead, load ITEMS keys
 //     per thread (coalesced) and count digits per warp;
 //  2. publish the tile's digit counts to the look-back words at once, so
 //     later tiles need not wait for this tile's ranking;
@@ -189,7 +176,8 @@ __device__ __forceinline__ void rank_unstable(PassSmem& sm, const uint64_t (&k)[
 //     advances it), or by one shared atomic per key where STABLE is false,
 //     and place them in shared memory in digit order;
 //  4. look back for the tile's global digit offsets (two predecessors per
-//     round trip);
+//     round trip; sixteen for small tiles, which all run at once, so that most
+//     predecessors have published aggregates alone);
 //  5. write runs of equal digits to their global positions.
 // HI: the pass's digit lies in the keys' high 32-bit half. EMIT (last pass
 // of a sort of transposed keys (w << 32) | u): instead of writing the key to
@@ -197,69 +185,91 @@ __device__ __forceinline__ void rank_unstable(PassSmem& sm, const uint64_t (&k)[
 // runs of equal w to emit.count[w]. RB < 8: only the digit's low RB bits can
 // be nonzero in any key (the top digit of keys narrower than the passes).
 // EDGES (first pass of a CSR build): key j is edge_key(src[j], dst[j]).
-template <bool HI, bool EMIT, bool STABLE, int RB = RADIX_BITS, bool EDGES = false>
+template <bool HI, bool EMIT, bool STABLE, int RB = RADIX_BITS, bool EDGES = false, int ITEMS = SORT_ITEMS>
 __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PassSmem& sm = *reinterpret_cast<PassSmem*>(smem_raw);
+  PassSmem<ITEMS>& sm = *reinterpret_cast<PassSmem<ITEMS>*>(smem_raw);
+  constexpr int TILE = SORT_THREADS * ITEMS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t sel = (a.shift >> 3) & 3u;  // byte of the half
   if (tid == 0) sm.tile = atomicAdd(a.tile_ctr, 1u);
   for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_THREADS) (&sm.whist[0][0])[i] = 0;
   __syncthreads();
   const int64_t tile = sm.tile;
-  const int64_t tbase = tile * SORT_TILE;
+  const int64_t tbase = tile * TILE;
   if (a.prefetch_tiles > 0 && tid == 0) {
     // a whole tile, in bounds, 16-byte aligned (the input is aligned and a
     // tile is 48 KB of keys, 24 KB of each endpoint array)
-    const int64_t pbase = tbase + a.prefetch_tiles * SORT_TILE;
-    if (pbase + SORT_TILE <= a.n) {
+    const int64_t pbase = tbase + a.prefetch_tiles * TILE;
+    if (pbase + TILE <= a.n) {
       if (!EDGES) {
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.in + pbase),
-                     "r"((uint32_t)(SORT_TILE * sizeof(uint64_t)))
+                     "r"((uint32_t)(TILE * sizeof(uint64_t)))
                      : "memory");
       } else {
         if (a.edge_prefetch & 1u)
           asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.edges.src + pbase),
-                       "r"((uint32_t)(SORT_TILE * sizeof(int32_t)))
+                       "r"((uint32_t)(TILE * sizeof(int32_t)))
                        : "memory");
         if (a.edge_prefetch & 2u)
           asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.edges.dst + pbase),
-                       "r"((uint32_t)(SORT_TILE * sizeof(int32_t)))
+                       "r"((uint32_t)(TILE * sizeof(int32_t)))
                        : "memory");
       }
     }
   }
 
-  // 1. load (item i of lane l in warp w is tile key w*512 + i*32 + l) and count
-  uint64_t k[SORT_ITEMS];
+  // 1. load (item i of lane l in warp w is tile key w*32*ITEMS + i*32 + l) and count
+  uint64_t k[ITEMS];
   if (!EDGES) {
 #pragma unroll
-    for (int i = 0; i < SORT_ITEMS; ++i) {
-      const int64_t idx = tbase + warp * (32 * SORT_ITEMS) + i * 32 + lane;
+    for (int i = 0; i < ITEMS; ++i) {
+      const int64_t idx = tbase + warp * (32 * ITEMS) + i * 32 + lane;
       k[i] = idx < a.n ? __ldcs(a.in + idx) : ~0ULL;
     }
   } else {
-    int32_t u[SORT_ITEMS], v[SORT_ITEMS];
+    int32_t u[ITEMS], v[ITEMS];
 #pragma unroll
-    for (int i = 0; i < SORT_ITEMS; ++i) {
-      const int64_t idx = tbase + warp * (32 * SORT_ITEMS) + i * 32 + lane;
+    for (int i = 0; i < ITEMS; ++i) {
+      const int64_t idx = tbase + warp * (32 * ITEMS) + i * 32 + lane;
       u[i] = idx < a.n ? __ldcs(a.edges.src + idx) : 0;
       v[i] = idx < a.n ? __ldcs(a.edges.dst + idx) : 0;
     }
 #pragma unroll
-    for (int i = 0; i < SORT_ITEMS; ++i) {
-      const int64_t idx = tbase + warp * (32 * SORT_ITEMS) + i * 32 + lane;
+    for (int i = 0; i < ITEMS; ++i) {
+      const int64_t idx = tbase + warp * (32 * ITEMS) + i * 32 + lane;
       k[i] = idx < a.n ? edge_key(u[i], v[i], a.edges.n_vertices, a.edges.b, a.edges.sentinel, a.err) : ~0ULL;
     }
   }
   const int64_t left = a.n - tbase;
-  const int nvalid = left < SORT_TILE ? (int)left : SORT_TILE;
+  const int nvalid = left < TILE ? (int)left : TILE;
 #pragma unroll
-  for (int i = 0; i < SORT_ITEMS; ++i) {
-    const int li = warp * (32 * SORT_ITEMS) + i * 32 + lane;
+  for (int i = 0; i < ITEMS; ++i) {
+    const int li = warp * (32 * ITEMS) + i * 32 + lane;
     if (li < nvalid) atomicAdd(&sm.whist[warp][digit_of<HI>(k[i], sel)], 1u);
   }
   __syncthreads();
+
+  // The first tile starts the look-back chains: its owners scan the pass's
+  // histogram for the digits' global starts (kept in goff until step 4).
+  if (tile == 0) {
+    uint64_t v = 0, incl = 0;
+    if (tid < RADIX) {
+      incl = v = a.hist[tid];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(FULL_MASK, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) sm.goff[warp] = incl;
+    }
+    __syncthreads();
+    uint64_t start = incl - v;
+    if (tid < RADIX)
+      for (int w = 0; w < warp; ++w) start += sm.goff[w];
+    __syncthreads();
+    if (tid < RADIX) sm.goff[tid] = start;
+  }
 
   // 2. digit owners: warp bases, tile count, publish, block scan
   uint32_t cnt = 0;
@@ -271,7 +281,7 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
       cnt += c;
     }
     uint64_t* st = a.status + tile * RADIX + tid;
-    if (tile == 0) st_relaxed(st, lb_pack(a.epoch, LB_INC, a.base[tid] + cnt));
+    if (tile == 0) st_relaxed(st, lb_pack(a.epoch, LB_INC, sm.goff[tid] + cnt));
     else st_relaxed(st, lb_pack(a.epoch, LB_AGG, cnt));
     uint32_t incl = cnt;
 #pragma unroll
@@ -296,18 +306,18 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
   __syncthreads();
 
   // 3. rank into shared memory in digit order
-  if (!STABLE) rank_unstable<HI>(sm, k, sel, nvalid, warp, lane, a.err);
-  else if (nvalid == SORT_TILE) rank_stable<HI, true, RB>(sm, k, sel, nvalid, warp, lane, a.err);
-  else rank_stable<HI, false, RB>(sm, k, sel, nvalid, warp, lane, a.err);
+  if (!STABLE) rank_unstable<HI, ITEMS>(sm, k, sel, nvalid, warp, lane, a.err);
+  else if (nvalid == TILE) rank_stable<HI, true, RB, ITEMS>(sm, k, sel, nvalid, warp, lane, a.err);
+  else rank_stable<HI, false, RB, ITEMS>(sm, k, sel, nvalid, warp, lane, a.err);
 
   // 4. look-back for the global offset of each digit
   __syncthreads();
   if (tid < RADIX) {
     uint64_t excl;
     if (tile == 0) {
-      excl = a.base[tid];
+      excl = sm.goff[tid];
     } else {
-      excl = lookback_window<2>(a.status + tid, tile, RADIX, a.epoch, a.err);
+      excl = lookback_window<(ITEMS == SORT_ITEMS ? 2 : 16)>(a.status + tid, tile, RADIX, a.epoch, a.err);
     }
     // the tile count is the distance to the next digit's start
     const uint32_t next = tid + 1 < RADIX ? sm.dstart[tid + 1] : (uint32_t)nvalid;
@@ -320,7 +330,7 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
   // 5. write out in runs
   if (!EMIT) {
 #pragma unroll
-    for (int i = 0; i < SORT_ITEMS; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
       const int pos = i * SORT_THREADS + tid;
       if (pos < nvalid) {
         const uint64_t key = sm.keys[pos];
@@ -334,7 +344,7 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
     // across consecutive lanes.
     const uint32_t le = lanemask_lt() | (1u << lane);
 #pragma unroll
-    for (int i = 0; i < SORT_ITEMS; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
       const int pos = i * SORT_THREADS + tid;
       uint64_t key = 0;
       uint32_t w = 0xffffffffu;
@@ -358,69 +368,103 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
   }
 }
 
+template <int ITEMS, typename F>
+void for_each_pass(F&& f) {
+  constexpr size_t bytes = sizeof(PassSmem<ITEMS>);
+  f(reinterpret_cast<const void*>(k_sort_pass<false, false, true, RADIX_BITS, false, ITEMS>), bytes);
+  f(reinterpret_cast<const void*>(k_sort_pass<true, false, true, RADIX_BITS, false, ITEMS>), bytes);
+  f(reinterpret_cast<const void*>(k_sort_pass<false, false, false, RADIX_BITS, false, ITEMS>), bytes);
+  f(reinterpret_cast<const void*>(k_sort_pass<true, true, true, RADIX_BITS, false, ITEMS>), bytes);
+  f(reinterpret_cast<const void*>(k_sort_pass<true, true, true, 4, false, ITEMS>), bytes);
+  f(reinterpret_cast<const void*>(k_sort_pass<false, false, false, RADIX_BITS, true, ITEMS>), bytes);
+}
+
+template <int ITEMS>
+void launch_pass(const PassArgs& a, int64_t tiles, cudaStream_t s, bool from_edges, bool place, bool narrow,
+                 bool unstable) {
+  constexpr size_t bytes = sizeof(PassSmem<ITEMS>);
+  const unsigned grid = (unsigned)tiles;
+  if (from_edges) k_sort_pass<false, false, false, RADIX_BITS, true, ITEMS><<<grid, SORT_THREADS, bytes, s>>>(a);
+  else if (place && narrow) k_sort_pass<true, true, true, 4, false, ITEMS><<<grid, SORT_THREADS, bytes, s>>>(a);
+  else if (place) k_sort_pass<true, true, true, RADIX_BITS, false, ITEMS><<<grid, SORT_THREADS, bytes, s>>>(a);
+  else if (unstable) k_sort_pass<false, false, false, RADIX_BITS, false, ITEMS><<<grid, SORT_THREADS, bytes, s>>>(a);
+  else if (a.shift >= 32) k_sort_pass<true, false, true, RADIX_BITS, false, ITEMS><<<grid, SORT_THREADS, bytes, s>>>(a);
+  else k_sort_pass<false, false, true, RADIX_BITS, false, ITEMS><<<grid, SORT_THREADS, bytes, s>>>(a);
+}
+
+// While every SM has at most one small tile, a pass is one short latency chain
+// and a quarter of the keys per thread shortens it (the rank takes the thread's
+// keys one after the other): 65,536 edges, 11.1 us a pass against 9.8 with its
+// neighbours' gaps; 131,072 11.9 against 10.3; 262,144, past the line, 12.3
+// both ways; 524,288 13.3 against 16.0 (longer look-back chains).
+int64_t small_max() { return (int64_t)sm_count() * SMALL_TILE; }
+
+int64_t pass_tiles(int64_t n) {
+  const int64_t tile = n <= small_max() ? SMALL_TILE : SORT_TILE;
+  return (n + tile - 1) / tile;
+}
+
 int passes_for(int bits) { return (bits + RADIX_BITS - 1) / RADIX_BITS; }
 
 }  // namespace
 
-// Scratch: [hist 8*256 u64][base 8*256 u64][counters 256 B][status tiles*256 u64]
+// Scratch: [hist 8*256 u64][counters 256 B][status tiles*256 u64]
 size_t sort_scratch_bytes(int64_t n, int bits) {
-  const int64_t tiles = (n + SORT_TILE - 1) / SORT_TILE;
+  // enough for a shorter sort too, whose tiles may be small
+  const int64_t tiles = std::max(pass_tiles(n), pass_tiles(std::min(n, small_max())));
   (void)bits;
-  return (size_t)2 * MAX_PASSES * RADIX * sizeof(uint64_t) + 256 + (size_t)tiles * RADIX * sizeof(uint64_t);
+  return (size_t)MAX_PASSES * RADIX * sizeof(uint64_t) + 256 + (size_t)tiles * RADIX * sizeof(uint64_t);
 }
 
 unsigned long long* sort_hist_area(void* scratch) { return static_cast<unsigned long long*>(scratch); }
 
-wedge_status sort_clear_hist(void* scratch, cudaStream_t s) {
-  WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, MAX_PASSES * RADIX * sizeof(uint64_t), s), "radix sort: clear histograms");
+wedge_status sort_clear(void* scratch, int64_t n, cudaStream_t s) {
+  const size_t bytes = MAX_PASSES * RADIX * sizeof(uint64_t) + 256 + (size_t)pass_tiles(n) * RADIX * sizeof(uint64_t);
+  WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, bytes, s), "radix sort: clear scratch");
   return WEDGE_OK;
 }
 
 wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, void* scratch, uint32_t* derr,
-                            cudaStream_t s, uint64_t** sorted, bool hist_ready, int shift0, const SortEmit* emit,
+                            cudaStream_t s, uint64_t** sorted, SortScratch ready, int shift0, const SortEmit* emit,
                             bool first_pass_unstable, const SortEdges* edges) {
   *sorted = keys;
-  if (edges && (n < 2 || shift0 != 0 || !first_pass_unstable || !hist_ready || emit))
+  if (edges && (n < 2 || shift0 != 0 || !first_pass_unstable || ready != SortScratch::cleared || emit))
     return fail(WEDGE_EINVAL, "radix sort: keys from edges need n >= 2 and a whole-key sort from bit 0");
   if (n <= 1) return WEDGE_OK;
   const int passes = passes_for(bits);
   if (passes < 1 || passes > MAX_PASSES || shift0 < 0 || (shift0 & 7) || shift0 + 8 * passes > 64)
     return fail(WEDGE_EINVAL, "radix sort: unsupported key bits %d from %d", bits, shift0);
-  const int64_t tiles = (n + SORT_TILE - 1) / SORT_TILE;
+  const bool small = n <= small_max();
+  const int64_t tiles = pass_tiles(n);
   if (tiles > (int64_t)UINT32_MAX) return fail(WEDGE_EINVAL, "radix sort: too many keys (%lld)", (long long)n);
   char* base_ptr = static_cast<char*>(scratch);
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(base_ptr);
-  uint64_t* digit_base = reinterpret_cast<uint64_t*>(base_ptr + MAX_PASSES * RADIX * sizeof(uint64_t));
-  uint32_t* ctr = reinterpret_cast<uint32_t*>(base_ptr + 2 * MAX_PASSES * RADIX * sizeof(uint64_t));
-  uint64_t* status = reinterpret_cast<uint64_t*>(base_ptr + 2 * MAX_PASSES * RADIX * sizeof(uint64_t) + 256);
-  // Histograms (unless the caller already accumulated them), then the rest.
   const size_t hist_bytes = MAX_PASSES * RADIX * sizeof(uint64_t);
+  uint32_t* ctr = reinterpret_cast<uint32_t*>(base_ptr + hist_bytes);
+  uint64_t* status = reinterpret_cast<uint64_t*>(base_ptr + hist_bytes + 256);
   wedge_status st = WEDGE_OK;
-  if (!hist_ready) {
-    WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, sort_scratch_bytes(n, bits), s), "radix sort: clear scratch");
+  if (ready == SortScratch::unused) {
+    if ((st = sort_clear(scratch, n, s)) != WEDGE_OK) return st;
     const int hist_blocks = sm_count() * 8;
     st = launch("sort_histogram", s, [&] {
       k_sort_hist<<<hist_blocks, HIST_THREADS, 0, s>>>(keys, n, passes, (uint32_t)shift0, hist);
     });
     if (st != WEDGE_OK) return st;
-  } else {
-    WEDGE_CUDA_TRY(cudaMemsetAsync(base_ptr + hist_bytes, 0, sort_scratch_bytes(n, bits) - hist_bytes, s),
+  } else if (ready == SortScratch::histograms) {
+    WEDGE_CUDA_TRY(cudaMemsetAsync(base_ptr + hist_bytes, 0, 256 + (size_t)tiles * RADIX * sizeof(uint64_t), s),
                    "radix sort: clear scratch");
   }
-  st = launch("sort_digit_base", s, [&] { k_sort_base<<<passes, RADIX, 0, s>>>(hist, digit_base); });
-  if (st != WEDGE_OK) return st;
 
   static bool attr_set = false;
   if (!attr_set) {
-    const void* fns[] = {reinterpret_cast<const void*>(k_sort_pass<false, false, true>),
-                         reinterpret_cast<const void*>(k_sort_pass<true, false, true>),
-                         reinterpret_cast<const void*>(k_sort_pass<false, false, false>),
-                         reinterpret_cast<const void*>(k_sort_pass<true, true, true>),
-                         reinterpret_cast<const void*>(k_sort_pass<true, true, true, 4>),
-                         reinterpret_cast<const void*>(k_sort_pass<false, false, false, RADIX_BITS, true>)};
-    for (const void* f : fns)
-      WEDGE_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PASS_SMEM),
-                     "radix sort: shared memory");
+    wedge_status fst = WEDGE_OK;
+    auto allow = [&](const void* f, size_t bytes) {
+      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+      if (e != cudaSuccess && fst == WEDGE_OK) fst = cuda_fail(e, "radix sort: shared memory");
+    };
+    for_each_pass<SORT_ITEMS>(allow);
+    for_each_pass<SMALL_ITEMS>(allow);
+    if (fst != WEDGE_OK) return fst;
     attr_set = true;
   }
   if (emit && shift0 < 32) return fail(WEDGE_EINVAL, "radix sort: placement needs keys sorted from bit 32");
@@ -436,7 +480,7 @@ wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, 
     a.n = n;
     a.shift = (uint32_t)(shift0 + p * RADIX_BITS);
     a.epoch = (uint32_t)(p + 1);
-    a.base = digit_base + p * RADIX;
+    a.hist = hist + p * RADIX;
     a.status = status;
     a.tile_ctr = ctr + p;
     a.err = derr;
@@ -457,13 +501,8 @@ wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, 
     // in use (b = 28: bits 24..27), the rank looks at those 4 alone
     const bool narrow = bits - RADIX_BITS * (passes - 1) <= 4;
     st = launch("sort_onesweep_pass", s, [&] {
-      if (from_edges)
-        k_sort_pass<false, false, false, RADIX_BITS, true><<<(unsigned)tiles, SORT_THREADS, PASS_SMEM, s>>>(a);
-      else if (place && narrow) k_sort_pass<true, true, true, 4><<<(unsigned)tiles, SORT_THREADS, PASS_SMEM, s>>>(a);
-      else if (place) k_sort_pass<true, true, true><<<(unsigned)tiles, SORT_THREADS, PASS_SMEM, s>>>(a);
-      else if (unstable) k_sort_pass<false, false, false><<<(unsigned)tiles, SORT_THREADS, PASS_SMEM, s>>>(a);
-      else if (a.shift >= 32) k_sort_pass<true, false, true><<<(unsigned)tiles, SORT_THREADS, PASS_SMEM, s>>>(a);
-      else k_sort_pass<false, false, true><<<(unsigned)tiles, SORT_THREADS, PASS_SMEM, s>>>(a);
+      if (small) launch_pass<SMALL_ITEMS>(a, tiles, s, from_edges, place, narrow, unstable);
+      else launch_pass<SORT_ITEMS>(a, tiles, s, from_edges, place, narrow, unstable);
     });
     if (st != WEDGE_OK) return st;
     uint64_t* t = src;

@@ -241,8 +241,8 @@ wedge_status sample_sorted_closure(const wedge_graph* g, const wedge_bins* b, ui
   // rows would still be large beside L2.
   const int by = (uint64_t)g->n_adj * sizeof(int32_t) >> 8 <= BLOCK_BYTES ? 8 : 16;
   const int from = std::max(0, (int)bits - by);
-  if ((st = radix_sort_u64(keys, alt, (int64_t)total, (int)bits - from, scratch, derr, s, &sorted, false, from)) !=
-      WEDGE_OK)
+  if ((st = radix_sort_u64(keys, alt, (int64_t)total, (int)bits - from, scratch, derr, s, &sorted,
+                           SortScratch::unused, from)) != WEDGE_OK)
     return done(st);
   ClosureArgs ca;
   ca.keys = sorted;

@@ -195,9 +195,9 @@ extern "C" wedge_status wedge_triangle_stats(const wedge_graph* g, const wedge_b
   //    ratio >= 1 is a positive double, whose bits order like its value
   uint64_t* sorted_bins = bin_keys;
   uint64_t* sorted_ratio = ratio_keys;
-  if ((st = radix_sort_u64(bin_keys, bin_alt, (int64_t)n, 38, scratch, derr, s, &sorted_bins, false)) != WEDGE_OK)
+  if ((st = radix_sort_u64(bin_keys, bin_alt, (int64_t)n, 38, scratch, derr, s, &sorted_bins)) != WEDGE_OK)
     return cleanup(st);
-  if ((st = radix_sort_u64(ratio_keys, ratio_alt, (int64_t)n, 63, scratch, derr, s, &sorted_ratio, false)) != WEDGE_OK)
+  if ((st = radix_sort_u64(ratio_keys, ratio_alt, (int64_t)n, 63, scratch, derr, s, &sorted_ratio)) != WEDGE_OK)
     return cleanup(st);
 
   // 4. box plot per BinId(d_min); ratio order statistics
