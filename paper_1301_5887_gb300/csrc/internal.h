@@ -56,6 +56,7 @@ enum class SortScratch { unused, histograms, cleared };
 constexpr int SORT_MAX_PASSES = 8;
 size_t sort_scratch_bytes(int64_t n, int bits);
 unsigned long long* sort_hist_area(void* scratch);
+bool sort_is_small(int64_t n);
 wedge_status sort_clear(void* scratch, int64_t n, cudaStream_t s);
 // Placement by the last pass of a sort of transposed keys (w << 32) | u: the
 // key at sorted position j writes u to adj[j + row_start[w]] and counts one
@@ -66,6 +67,7 @@ struct SortEmit {
   int32_t* count;
   int64_t adj_len;  // entries of adj (checked by the debug build)
   int64_t rows;     // entries of row_start and count
+  const int64_t* n_keys;  // device: number of keys, the sort's n being the most there can be (sort_is_small(n)), or nullptr
 };
 
 // Keys of the first pass computed from an edge list instead of read (CSR

@@ -197,11 +197,13 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
   __syncthreads();
   const int64_t tile = sm.tile;
   const int64_t tbase = tile * TILE;
+  const int64_t n = ITEMS == SMALL_ITEMS && a.emit.n_keys ? *a.emit.n_keys : a.n;
+  if (ITEMS == SMALL_ITEMS && tbase >= n) return;  // (later tiles have none either, so no one waits for this one)
   if (a.prefetch_tiles > 0 && tid == 0) {
     // a whole tile, in bounds, 16-byte aligned (the input is aligned and a
     // tile is 48 KB of keys, 24 KB of each endpoint array)
     const int64_t pbase = tbase + a.prefetch_tiles * TILE;
-    if (pbase + TILE <= a.n) {
+    if (pbase + TILE <= n) {
       if (!EDGES) {
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.in + pbase),
                      "r"((uint32_t)(TILE * sizeof(uint64_t)))
@@ -225,23 +227,23 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       const int64_t idx = tbase + warp * (32 * ITEMS) + i * 32 + lane;
-      k[i] = idx < a.n ? __ldcs(a.in + idx) : ~0ULL;
+      k[i] = idx < n ? __ldcs(a.in + idx) : ~0ULL;
     }
   } else {
     int32_t u[ITEMS], v[ITEMS];
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       const int64_t idx = tbase + warp * (32 * ITEMS) + i * 32 + lane;
-      u[i] = idx < a.n ? __ldcs(a.edges.src + idx) : 0;
-      v[i] = idx < a.n ? __ldcs(a.edges.dst + idx) : 0;
+      u[i] = idx < n ? __ldcs(a.edges.src + idx) : 0;
+      v[i] = idx < n ? __ldcs(a.edges.dst + idx) : 0;
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       const int64_t idx = tbase + warp * (32 * ITEMS) + i * 32 + lane;
-      k[i] = idx < a.n ? edge_key(u[i], v[i], a.edges.n_vertices, a.edges.b, a.edges.sentinel, a.err) : ~0ULL;
+      k[i] = idx < n ? edge_key(u[i], v[i], a.edges.n_vertices, a.edges.b, a.edges.sentinel, a.err) : ~0ULL;
     }
   }
-  const int64_t left = a.n - tbase;
+  const int64_t left = n - tbase;
   const int nvalid = left < TILE ? (int)left : TILE;
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
@@ -335,7 +337,7 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
       if (pos < nvalid) {
         const uint64_t key = sm.keys[pos];
         const uint64_t j = sm.goff[digit_of<HI>(key, sel)] + (uint64_t)pos;
-        if (in_bounds(j, (uint64_t)a.n, a.err)) __stcs(a.out + j, key);
+        if (in_bounds(j, (uint64_t)n, a.err)) __stcs(a.out + j, key);
       }
     }
   } else {
@@ -416,6 +418,8 @@ size_t sort_scratch_bytes(int64_t n, int bits) {
   return (size_t)MAX_PASSES * RADIX * sizeof(uint64_t) + 256 + (size_t)tiles * RADIX * sizeof(uint64_t);
 }
 
+bool sort_is_small(int64_t n) { return n <= small_max(); }
+
 unsigned long long* sort_hist_area(void* scratch) { return static_cast<unsigned long long*>(scratch); }
 
 wedge_status sort_clear(void* scratch, int64_t n, cudaStream_t s) {
@@ -467,6 +471,8 @@ wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, 
     if (fst != WEDGE_OK) return fst;
     attr_set = true;
   }
+  if (emit && emit->n_keys && !small)
+    return fail(WEDGE_EINVAL, "radix sort: a number of keys on the device needs a small sort");
   if (emit && shift0 < 32) return fail(WEDGE_EINVAL, "radix sort: placement needs keys sorted from bit 32");
   // L2 prefetch one SM count of tiles ahead (tiles are claimed in order, so
   // that tile is claimed about one wave of CTAs later)

@@ -1,5 +1,6 @@
-"""Small inputs: sorts of at most one 1536-key tile per SM, scans of one tile
-and sample budgets of less than a full chip take kernels' short forms. Sizes on
+"""Small inputs: sorts of at most one 1536-key tile per SM (whose number of
+keys may be known to the device alone), scans of one tile and sample budgets of
+less than a full chip take kernels' short forms. Sizes on
 either side of each line, against plain sorting by torch (integers: equal) and
 against the same samples drawn in one long call.
 """
@@ -54,6 +55,15 @@ def _lines():
 def test_builds_about_the_small_sort(where, delta, n):
     m = _lines()[where == "chip"] + delta
     _check(*_edges(m, n), n)[0].free()
+
+
+@pytest.mark.parametrize("m", [1, 2, 3, 1537, 20_000])
+@pytest.mark.parametrize("left", [0, 1, 2])
+def test_few_edges_left(m, left):
+    """Loops, or one or two edges again and again: the transposed sort has `left` keys (its host does not know)."""
+    src = torch.arange(m, device="cuda", dtype=torch.int32) % max(left, 1)
+    dst = src + 5 if left else src.clone()
+    _check(src, dst, 9)[0].free()
 
 
 @pytest.mark.parametrize("n", [3000, 300_000])
