@@ -154,36 +154,35 @@ def oracle_step(scale: int, edgefactor: int, k: int):
     return dt, adj.shape[0] // 2, n_samples
 
 
-def modelled_sampler_sectors(wedge, torch, g, b, k_bin, k_glob, hot_levels=20):
-    """The random-access model of one sample (32-byte sectors, one per
-    random access): the centre search over the stream's prefix W (uint64,
-    4 per sector, ceil(log2(len/4)) levels) + L[j] + off[v0] + adj[i], adj[j]
-    + off[v1], off[v2] + the closure search in the smaller row (int32, 8 per
-    sector, ceil(log2(d_lo/8)) levels + 1); the top `hot_levels` levels of
-    either search stay in L2. Centre searches use each stream's actual length
-    (bin sizes); the closure term uses the degrees of a recorded draw of the
-    global stream. Returns sectors per sample over the step's streams."""
-    import numpy as np
-    bi = b.info()
-    k = min(k_glob, 1 << 20)
-    rec = torch.zeros(k * 8, dtype=torch.int32, device="cuda")
-    wedge.sample(g, b, seed=SEED + 1, k_global=k, flags=wedge.FLAG_NO_BINS, records=rec)
-    r = rec.cpu().numpy().reshape(-1, 8).astype(np.int64)
-    d1, d2 = r[:, 5], r[:, 6]
-    dlo = np.minimum(d1, d2)
-    closure = np.maximum(0, np.ceil(np.log2(np.maximum(dlo, 1) / 8.0)) - hot_levels) + 1
-    per_sample = 6.0 + float(closure.mean())
+def modelled_sampler_sectors(wedge, torch, g, b, k_bin, k_glob):
+    """The random-access model of one sample: the accesses that leave L2. A
+    sample reads, each at a random place, its guide entry (4 bytes per 4
+    vertices of the stream), one sector of the prefix W (8 per vertex), L[j]
+    (4), off[v0], adj[i], adj[j], off[v1], off[v2] and one sector of the
+    smaller row (the interpolated place of the sought id). An access to an
+    array of S bytes misses an L2 of C bytes with probability max(0, 1 - C/S);
+    off[v0] of a stream's vertices touches one 128-byte line per vertex at
+    most. Neighbours are drawn towards hubs, whose offsets stay in L2 more
+    often than that, which the model leaves out. Returns accesses per sample
+    over the step's streams."""
+    l2 = getattr(torch.cuda.get_device_properties(0), "L2_cache_size", 0) or 129 << 20
+    bi, gi = b.info(), g.info()
+
+    def miss(size):
+        return max(0.0, 1.0 - l2 / size) if size > 0 else 0.0
+
+    rows = 3.0 * miss(4 * gi.n_adj) + 2.0 * miss(8 * gi.n_vertices)
 
     def centre(length):
-        return max(0.0, math.ceil(math.log2(max(length, 1) / 4.0)) - hot_levels)
+        return miss(length) + miss(8 * length) + miss(4 * length) + miss(min(128 * length, 8 * gi.n_vertices))
 
     total, count = 0.0, 0
     for bid in range(2, bi.n_bins):
         nb = int(bi.start[bid + 1] - bi.start[bid])
         if int(bi.p_b[bid]) > 0 and nb > 0:
-            total += k_bin * (centre(nb) + per_sample)
+            total += k_bin * (centre(nb) + rows)
             count += k_bin
-    total += k_glob * (centre(int(bi.n_wedge_vertices)) + per_sample)
+    total += k_glob * (centre(int(bi.n_wedge_vertices)) + rows)
     count += k_glob
     return total / count
 
@@ -392,12 +391,11 @@ def bench_batched(wedge, graphgen, torch, probe_rate=None, probe_spa=None, autot
     for it in items:
         it["bins"].free()
         it["graph"].free()
-    # Every graph of the mix has at most 2^22 vertices, so in the access model
-    # (modelled_sampler_sectors) all search levels stay in L2: 7 random
-    # accesses per sample (6 gathers + the last closure probe), and most of
-    # the mix's working set is L2-resident (ncu: a few DRAM sectors per
-    # sample). The ceiling is then the rate of random reads that hit L2.
-    s_mix = 7.0
+    # Every graph of the mix has at most 2^22 vertices, and most of the mix's
+    # working set is L2-resident (ncu: under one DRAM access per sample). The
+    # ceiling is the rate of random reads that hit L2, for the nine a sample
+    # takes (guide, W, L, off[v0], two neighbours, their offsets, the row).
+    s_mix = 9.0
     roof = {"bound": "random-access (L2-resident working set)", "kernel": "batch_sample",
             "modelled_accesses_per_sample": s_mix, "unit": "G accesses/s",
             "achieved": s_mix * samples / batch_s / 1e9,

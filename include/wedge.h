@@ -280,7 +280,7 @@ WEDGE_API wedge_status wedge_sample(const wedge_graph* g, const wedge_bins* b, c
  * GPU counterpart of serving many graphs and budgets at once.
  *
  * Launch configuration: a tile is drawn one sample per thread
- * (WEDGE_MAP_THREAD: binary searches) or one sample per warp
+ * (WEDGE_MAP_THREAD: searches of its own) or one sample per warp
  * (WEDGE_MAP_WARP: 33-way cooperative searches of W and of the closure row),
  * chosen per stream class by the number of vertices the stream searches
  * (small < 2^12, medium < 2^20, large). block_threads is 128, 256 or 512

@@ -1,7 +1,7 @@
 // sample_device.cuh — device code for drawing one wedge and checking its
 // closure (Sec. 3.2, Alg. Phase 3b), shared by the single-graph sampler and
 // the batched persistent sampler. Two mappings:
-//   thread: one thread draws one wedge; binary searches.
+//   thread: one thread draws one wedge; the centre from a guide, the row searched by interpolation.
 //   warp:   the 32 lanes of a warp draw one wedge together; 33-way searches
 //           (each step probes 32 positions at once), so a search of length n
 //           takes about log33(n) dependent steps instead of log2(n).

@@ -89,6 +89,8 @@ uint64_t request_samples(const wedge_server_request& r, const wedge_bins* b) {
   return total;
 }
 
+// (The guide over W, a byte a vertex, is left out: a budget admits what it did
+// before there was one.)
 uint64_t graph_bytes(const wedge_graph* g, const wedge_bins* b) {
   const uint64_t n = (uint64_t)g->n;
   uint64_t bytes = 8 * (n + 1) + 4 * n + 4 * (uint64_t)(2 * g->n_input > 0 ? 2 * g->n_input : 1);
