@@ -67,9 +67,20 @@ struct SampleArgs {
   unsigned long long* q_out;   // [n_streams][4]
   unsigned long long* stats;   // [WEDGE_STAT_BINS][WEDGE_STAT_BINS]
   wedge_record* records;       // global stream records or nullptr
+  bool whole_records;          // records are aligned to their size
   int64_t n, n_adj, n_L;       // sizes for the bounds-checked debug build
   uint32_t* err;
 };
+
+// A 32-byte aligned record as one store: eight words one by one write each
+// sector eight times (scale 24, 5 M records: 544 and 564 us on two machines, 528
+// and 556 so; without records 502).
+static_assert(sizeof(wedge_record) == 32, "a record is a sector");
+__device__ __forceinline__ void store_record(wedge_record* p, const wedge_record& r) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(r.v0), "r"(r.v1), "r"(r.v2),
+               "r"(r.closed), "r"(r.d0), "r"(r.d1), "r"(r.d2), "r"(r.reserved)
+               : "memory");
+}
 
 __global__ __launch_bounds__(SAMPLE_THREADS) void k_sample(SampleArgs a) {
   __shared__ StreamDesc s_desc;
@@ -142,7 +153,11 @@ __global__ __launch_bounds__(SAMPLE_THREADS) void k_sample(SampleArgs a) {
           rec.d1 = (int32_t)d1;
           rec.d2 = (int32_t)d2;
           rec.reserved = 0;
-          a.records[local] = rec;
+          if (a.whole_records) {
+            store_record(a.records + local, rec);
+          } else {
+            a.records[local] = rec;
+          }
         }
       }
     }
@@ -313,6 +328,7 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
   a.q_out = d_cnt;
   a.stats = d_cnt + streams.size() * 4;
   a.records = static_cast<wedge_record*>(sp->records);
+  a.whole_records = reinterpret_cast<uintptr_t>(sp->records) % sizeof(wedge_record) == 0;
   a.n = g->n;
   a.n_adj = g->n_adj;
   a.n_L = inf.n_wedge_vertices;

@@ -26,43 +26,87 @@
 namespace wedge {
 namespace {
 
-__global__ __launch_bounds__(256) void k_tri_keys(const wedge_record* __restrict__ rec, uint64_t k,
-                                                  unsigned long long* __restrict__ n_closed,
-                                                  uint64_t* __restrict__ bin_keys, uint64_t* __restrict__ ratio_keys) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  const uint32_t lane = threadIdx.x & 31u;
-  // Every lane of a warp runs the same number of iterations (the bound is
-  // rounded up to whole warps), so the warp-wide append below is safe.
-  const uint64_t k_round = (k + 31) & ~31ULL;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k_round; i += stride) {
-    bool closed = false;
-    uint64_t dmin = 0, dmax = 0;
-    if (i < k) {
-      const wedge_record r = rec[i];
-      closed = r.closed != 0;
-      const uint64_t d0 = (uint64_t)r.d0, d1 = (uint64_t)r.d1, d2 = (uint64_t)r.d2;
-      dmin = min(d0, min(d1, d2));
-      dmax = max(d0, max(d1, d2));
+constexpr int KEY_THREADS = 256;
+constexpr int KEY_RECORDS = 8;  // of a thread at a time
+
+// A CTA takes KEY_THREADS * KEY_RECORDS records at a time, whose `closed` words
+// are all loaded before the first is looked at, and makes room for its closed
+// ones with one atomic. They are few (one in sixty on Kronecker scale 24), so
+// they are gathered first and their keys made by full warps: a double division
+// occupies the few FP64 units as long for one lane as for 32. 5 M records (160
+// MB): 75 us with an atomic and a division per warp and 32 records, 32 so.
+__global__ __launch_bounds__(KEY_THREADS) void k_tri_keys(const wedge_record* __restrict__ rec, uint64_t k,
+                                                          unsigned long long* __restrict__ n_closed,
+                                                          uint64_t* __restrict__ bin_keys,
+                                                          uint64_t* __restrict__ ratio_keys) {
+  __shared__ uint2 s_degrees[KEY_THREADS * KEY_RECORDS];  // least, largest
+  __shared__ uint32_t s_count[KEY_THREADS / 32];
+  __shared__ uint32_t s_total;
+  __shared__ unsigned long long s_base;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr uint64_t TILE = (uint64_t)KEY_THREADS * KEY_RECORDS;
+  for (uint64_t t0 = blockIdx.x * TILE; t0 < k; t0 += gridDim.x * TILE) {
+    bool closed[KEY_RECORDS];
+#pragma unroll
+    for (int j = 0; j < KEY_RECORDS; ++j) {
+      const uint64_t i = t0 + (uint64_t)j * KEY_THREADS + tid;
+      closed[j] = i < k && __ldg(&rec[i].closed) != 0;
     }
-    const uint32_t ballot = __ballot_sync(0xffffffffu, closed);
-    if (ballot == 0) continue;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(n_closed, (unsigned long long)__popc(ballot));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (closed) {
-      const uint64_t slot = base + __popc(ballot & ((1u << lane) - 1u));
-      bin_keys[slot] = ((uint64_t)stat_bin(dmin) << 32) | dmax;
-      ratio_keys[slot] = (uint64_t)__double_as_longlong(__ddiv_rn((double)dmax, (double)dmin));
+    uint32_t mine = 0, bal[KEY_RECORDS];
+#pragma unroll
+    for (int j = 0; j < KEY_RECORDS; ++j) {
+      bal[j] = __ballot_sync(FULL_MASK, closed[j]);
+      mine += __popc(bal[j]);
     }
+    if (lane == 0) s_count[warp] = mine;
+    __syncthreads();
+    if (tid == 0) {
+      uint32_t total = 0;
+      for (int w = 0; w < KEY_THREADS / 32; ++w) {
+        const uint32_t c = s_count[w];
+        s_count[w] = total;
+        total += c;
+      }
+      s_total = total;
+      s_base = total ? atomicAdd(n_closed, (unsigned long long)total) : 0ULL;
+    }
+    __syncthreads();
+    uint32_t slot = s_count[warp];
+    const uint32_t below = lanemask_lt();
+#pragma unroll
+    for (int j = 0; j < KEY_RECORDS; ++j) {
+      if (closed[j]) {
+        const wedge_record& r = rec[t0 + (uint64_t)j * KEY_THREADS + tid];
+        const uint32_t d0 = (uint32_t)r.d0, d1 = (uint32_t)r.d1, d2 = (uint32_t)r.d2;
+        s_degrees[slot + __popc(bal[j] & below)] = make_uint2(min(d0, min(d1, d2)), max(d0, max(d1, d2)));
+      }
+      slot += __popc(bal[j]);
+    }
+    __syncthreads();
+    const uint64_t base = s_base;
+    for (uint32_t i = tid; i < s_total; i += KEY_THREADS) {
+      const uint2 d = s_degrees[i];
+      bin_keys[base + i] = ((uint64_t)stat_bin(d.x) << 32) | d.y;
+      ratio_keys[base + i] = (uint64_t)__double_as_longlong(__ddiv_rn((double)d.y, (double)d.x));
+    }
+    __syncthreads();  // the gathered degrees have been read
   }
 }
 
-// Index of the first key >= x in sorted keys[0, n).
+// Index of the first key >= x in sorted keys[0, n), by a warp: 32 probes at a
+// time. The same on every lane.
 __device__ __forceinline__ uint64_t lower_bound_u64(const uint64_t* keys, uint64_t n, uint64_t x) {
-  uint64_t lo = 0, hi = n;
+  const uint32_t lane = threadIdx.x & 31u;
+  uint64_t lo = 0, hi = n;  // the index lies in [lo, hi]
   while (lo < hi) {
-    const uint64_t mid = lo + ((hi - lo) >> 1);
-    if (keys[mid] < x) lo = mid + 1; else hi = mid;
+    const uint64_t step = (hi - lo + 31) / 32;
+    const uint64_t at = lo + lane * step;
+    const uint32_t less = __ballot_sync(FULL_MASK, at < hi && keys[at] < x);  // lanes 0 .. m - 1
+    const uint32_t m = __popc(less);
+    if (m == 0) return lo;
+    const uint64_t from = lo;
+    lo = from + (m - 1) * step + 1;
+    hi = min(hi, from + m * step);
   }
   return lo;
 }
@@ -74,10 +118,10 @@ __device__ __forceinline__ uint64_t rank_index(uint64_t n, uint64_t num, uint64_
   return r - 1;
 }
 
+// One warp per bin.
 __global__ __launch_bounds__(32) void k_tri_box(const uint64_t* __restrict__ keys, uint64_t n,
                                                 wedge_triangle_box* __restrict__ out) {
   const uint32_t b = blockIdx.x;
-  if (threadIdx.x != 0) return;
   const uint64_t lo = lower_bound_u64(keys, n, (uint64_t)b << 32);
   const uint64_t hi = lower_bound_u64(keys, n, (uint64_t)(b + 1) << 32);
   wedge_triangle_box box = {};
@@ -102,7 +146,7 @@ __global__ __launch_bounds__(32) void k_tri_box(const uint64_t* __restrict__ key
     box.whisker_hi = z > 0 ? (keys[lo + z - 1] & mask) : box.max;
     box.outliers = a + (c - z);
   }
-  out[b] = box;
+  if (threadIdx.x == 0) out[b] = box;
 }
 
 __global__ void k_tri_ratio(const uint64_t* __restrict__ keys, uint64_t n, double* __restrict__ q) {
@@ -132,22 +176,23 @@ extern "C" wedge_status wedge_triangle_stats(const wedge_graph* g, const wedge_b
 
   wedge_record* own_rec = nullptr;
   uint64_t *bin_keys = nullptr, *bin_alt = nullptr, *ratio_keys = nullptr, *ratio_alt = nullptr;
-  unsigned long long* n_closed = nullptr;
-  wedge_triangle_box* d_box = nullptr;
-  double* d_ratio = nullptr;
+  // what the host reads, in one block: appended keys, error bits, the ratio's
+  // quartiles, the boxes
+  struct Results {
+    unsigned long long n_closed, err;
+    double ratio_q[5];
+    wedge_triangle_box box[WEDGE_STAT_BINS];
+  };
+  Results* res = nullptr;
   void* scratch = nullptr;
-  uint32_t* derr = nullptr;
   auto cleanup = [&](wedge_status st) {
     dfree(own_rec, s);
     dfree(bin_keys, s);
     dfree(bin_alt, s);
     dfree(ratio_keys, s);
     dfree(ratio_alt, s);
-    dfree(n_closed, s);
-    dfree(d_box, s);
-    dfree(d_ratio, s);
+    dfree(res, s);
     dfree(scratch, s);
-    dfree(derr, s);
     return st;
   };
   wedge_status st;
@@ -175,20 +220,18 @@ extern "C" wedge_status wedge_triangle_stats(const wedge_graph* g, const wedge_b
   if ((st = dalloc_n(&bin_alt, nk, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
   if ((st = dalloc_n(&ratio_keys, nk, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
   if ((st = dalloc_n(&ratio_alt, nk, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
-  if ((st = dalloc_n(&n_closed, 1, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
-  if ((st = dalloc_n(&d_box, WEDGE_STAT_BINS, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
-  if ((st = dalloc_n(&d_ratio, 5, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
+  if ((st = dalloc_n(&res, 1, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
   if ((st = dalloc(&scratch, sort_scratch_bytes((int64_t)nk, 64), s, "wedge_triangle_stats")) != WEDGE_OK)
     return cleanup(st);
-  if ((st = dalloc_n(&derr, 1, s, "wedge_triangle_stats")) != WEDGE_OK) return cleanup(st);
-  cudaError_t e = cudaMemsetAsync(n_closed, 0, sizeof(unsigned long long), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(derr, 0, sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_ratio, 0, 5 * sizeof(double), s);
+  uint32_t* derr = reinterpret_cast<uint32_t*>(&res->err);
+  cudaError_t e = cudaMemsetAsync(res, 0, sizeof(Results), s);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "wedge_triangle_stats"));
 
   // 2. one (BinId(d_min), d_max) key and one ratio key per closed sample
-  const unsigned blocks = (unsigned)std::min<uint64_t>((k + 255) / 256, (uint64_t)sm_count() * 8);
-  st = launch("triangle_keys", s, [&] { k_tri_keys<<<blocks, 256, 0, s>>>(rec, k, n_closed, bin_keys, ratio_keys); });
+  constexpr uint64_t tile = (uint64_t)KEY_THREADS * KEY_RECORDS;
+  const unsigned blocks = (unsigned)std::min<uint64_t>((k + tile - 1) / tile, (uint64_t)sm_count() * 8);
+  st = launch("triangle_keys", s,
+              [&] { k_tri_keys<<<blocks, KEY_THREADS, 0, s>>>(rec, k, &res->n_closed, bin_keys, ratio_keys); });
   if (st != WEDGE_OK) return cleanup(st);
 
   // 3. sort: BinId(d_min) <= 32 sits in bits 32..37 above d_max < 2^31; a
@@ -201,18 +244,18 @@ extern "C" wedge_status wedge_triangle_stats(const wedge_graph* g, const wedge_b
     return cleanup(st);
 
   // 4. box plot per BinId(d_min); ratio order statistics
-  st = launch("triangle_box", s, [&] { k_tri_box<<<WEDGE_STAT_BINS, 32, 0, s>>>(sorted_bins, n, d_box); });
+  st = launch("triangle_box", s, [&] { k_tri_box<<<WEDGE_STAT_BINS, 32, 0, s>>>(sorted_bins, n, res->box); });
   if (st != WEDGE_OK) return cleanup(st);
-  st = launch("triangle_ratio", s, [&] { k_tri_ratio<<<1, 32, 0, s>>>(sorted_ratio, n, d_ratio); });
+  st = launch("triangle_ratio", s, [&] { k_tri_ratio<<<1, 32, 0, s>>>(sorted_ratio, n, res->ratio_q); });
   if (st != WEDGE_OK) return cleanup(st);
-  uint32_t herr = 0;
-  unsigned long long appended = 0;
-  e = cudaMemcpyAsync(out->box, d_box, sizeof(out->box), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out->ratio_q, d_ratio, sizeof(out->ratio_q), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&appended, n_closed, sizeof(appended), cudaMemcpyDeviceToHost, s);
+  Results h;
+  e = cudaMemcpyAsync(&h, res, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "wedge_triangle_stats"));
+  memcpy(out->box, h.box, sizeof(out->box));
+  memcpy(out->ratio_q, h.ratio_q, sizeof(out->ratio_q));
+  const uint32_t herr = (uint32_t)h.err;
+  const unsigned long long appended = h.n_closed;
   if (herr & DERR_TIMEOUT) return cleanup(fail(WEDGE_ETIMEOUT, "wedge_triangle_stats: a look-back wait gave up"));
   if (appended != n)
     return cleanup(fail(WEDGE_ECUDA, "wedge_triangle_stats: %llu closed records for %llu closed samples", appended,

@@ -106,3 +106,26 @@ def test_budgets_about_the_full_chip(k):
     assert torch.equal(q, q0 + q1) and closed == c0 + c1
     b.free()
     g.free()
+
+
+@pytest.mark.parametrize("k", [1, 2047, 2048, 2049, 40_000, 2_500_000])
+def test_triangle_keys_about_a_tile(k):
+    """Ratio quartiles and box counts against the records, written whole (aligned) and word by word."""
+    n = 700
+    g = _check(*_edges(9000, n), n)[0]
+    b = wedge.bin(g)
+    room = torch.zeros(8 * k + 8, dtype=torch.int32, device="cuda")
+    aligned, shifted = room[: 8 * k], torch.zeros(8 * k + 8, dtype=torch.int32, device="cuda")[1 : 8 * k + 1]
+    t = wedge.triangle_stats(g, b, 11, k, records=aligned)
+    u = wedge.triangle_stats(g, b, 11, k, records=shifted)
+    assert torch.equal(aligned, shifted) and int(room[8 * k :].abs().sum()) == 0
+    r = aligned.view(-1, 8)
+    d = r[r[:, 3] != 0][:, 4:7].cpu().double()
+    assert t["closed"] == u["closed"] == len(d)
+    lo, hi = (d.min(1).values, d.max(1).values) if len(d) else (d.sum(1), d.sum(1))
+    ratio = (hi / lo).sort().values
+    if len(d):
+        at = [0] + [max(1, -(-len(d) * q // 4)) - 1 for q in (1, 2, 3)] + [len(d) - 1]
+        assert list(t["ratio_q"]) == list(u["ratio_q"]) == ratio[at].tolist()
+    b.free()
+    g.free()
