@@ -312,26 +312,6 @@ __global__ __launch_bounds__(256) void k_count_back(const uint64_t* __restrict__
   }
 }
 
-// Degrees, offsets (forward and backward exclusive scans added), largest degree.
-__global__ __launch_bounds__(256) void k_rows(const int32_t* __restrict__ fdeg, const int32_t* __restrict__ bdeg,
-                                              const int64_t* __restrict__ foff, const int64_t* __restrict__ boff,
-                                              int32_t n, int32_t* __restrict__ deg, int64_t* __restrict__ off,
-                                              int32_t* maxdeg) {
-  int32_t mx = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += stride) {
-    off[x] = foff[x] + boff[x];
-    if (x < n) {
-      const int32_t d = fdeg[x] + bdeg[x];
-      deg[x] = d;
-      mx = max(mx, d);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(FULL_MASK, mx, o));
-  if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(maxdeg, mx);
-}
-
 // Forward entry i (the i-th unique sorted forward key (u << b) | w) goes to
 // i + boff[u + 1]: row u starts at foff[u] + boff[u] and holds its
 // boff[u + 1] - boff[u] backward entries first. The sorted keys are read
@@ -760,13 +740,8 @@ extern "C" wedge_status wedge_graph_build(const int32_t* src, const int32_t* dst
     }
 
     // 5. backward offsets, degrees, forward placement
-    st = scan_i32_to_i64(bdeg, boff, n_vertices, boff + n_vertices, nullptr, bb.scratch, bb.derr, s);
-    if (st != WEDGE_OK) return bail(st);
     int32_t* maxdeg = reinterpret_cast<int32_t*>(bb.scalars + 1);
-    st = launch("row_offsets", s, [&] {
-      k_rows<<<grid_stride_blocks((int64_t)n_vertices + 1, 256), 256, 0, s>>>(bb.fdeg, bdeg, bb.foff, boff, n_vertices,
-                                                                          g->deg, g->off, maxdeg);
-    });
+    st = scan_rows(bb.fdeg, bdeg, bb.foff, boff, n_vertices, g->off, g->deg, maxdeg, bb.scratch, bb.derr, s);
     if (st != WEDGE_OK) return bail(st);
     if (m_unique > 0) {
       st = launch("place_rows", s, [&] {

@@ -114,6 +114,10 @@ wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t
 // The same under a name of its own.
 wedge_status scan_counts_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch,
                                 uint32_t* derr, cudaStream_t s, const char* name);
+// boff: exclusive scan of bdeg (n + 1); off = foff + boff (n + 1), deg = fdeg +
+// bdeg, *maxdeg raised to the largest; n >= 1.
+wedge_status scan_rows(const int32_t* fdeg, const int32_t* bdeg, const int64_t* foff, int64_t* boff, int64_t n,
+                       int64_t* off, int32_t* deg, int32_t* maxdeg, void* scratch, uint32_t* derr, cudaStream_t s);
 // out[i] = sum in[0..i) for i < n and out[n] = the total (out holds n + 1).
 wedge_status scan_u32_with_total(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s);
