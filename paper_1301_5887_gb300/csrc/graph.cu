@@ -116,6 +116,7 @@ __global__ __launch_bounds__(EXPAND_THREADS) void k_expand(const int32_t* __rest
     if (WRITE) __stcs(keys + e, key);
     count_digits<NP>(sh, key, passes, copy);
   }
+  asm volatile("griddepcontrol.launch_dependents;");  // the sort's first pass may start up
   __syncthreads();
   for (int i = threadIdx.x; i < passes * 256; i += blockDim.x) {
     uint32_t v = 0;
