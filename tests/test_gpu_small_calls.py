@@ -72,10 +72,11 @@ def test_long_list_of_few_edges(n):
     _check(*_edges(_lines()[1] * 3, n, repeat=12), n)[0].free()
 
 
-@pytest.mark.parametrize("n,m", [(4096, 30_000), (4097, 30_000), (20_000, 3000), (300_000, 900_000), (3_000_000, 9_000_000)])
-def test_bins_read_back(n, m):
+@pytest.mark.parametrize("n,m,tau", [(4096, 30_000, 2), (4097, 30_000, 2), (20_000, 3000, 2), (300_000, 900_000, 2),
+                                     (3_000_000, 9_000_000, 2), (9_000_000, 20_000_000, 60)])
+def test_bins_read_back(n, m, tau):
     g, deg = _check(*_edges(m, n), n)
-    b = wedge.bin(g, tau=2, omega=2)
+    b = wedge.bin(g, tau=tau, omega=2)
     info = b.info()
     lo = torch.tensor(list(info.lo_deg)[: info.n_bins])
     which = torch.searchsorted(lo, deg.cpu(), right=True) - 1
