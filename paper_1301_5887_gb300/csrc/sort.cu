@@ -37,11 +37,6 @@ constexpr int SORT_MIN_BLOCKS = 3;  // resident CTAs per SM the register budget 
 constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;  // 6144 keys
 constexpr int SMALL_ITEMS = 4;
 constexpr int SMALL_TILE = SORT_THREADS * SMALL_ITEMS;  // 1536 keys
-// Passes of at most this many tiles are chained: a CTA may start before the pass
-// before has ended. Over more tiles the last wave is nothing, and the two
-// instructions a tile cost more (builds of 2^28 edges 14.26 -> 14.24 ms chained, of
-// 2^29 33.07 -> 33.30).
-constexpr int64_t CHAIN_TILES = 1 << 16;
 constexpr int MAX_PASSES = SORT_MAX_PASSES;
 constexpr int HIST_THREADS = 256;
 
@@ -75,7 +70,7 @@ struct PassArgs {
   const uint64_t* in;
   uint64_t* out;
   int64_t n;
-  bool chained;          // launched before the kernel before it has ended (CHAIN_TILES)
+  bool chained;          // launched before the kernel before it has ended (sort_pass_chained)
   uint32_t shift;
   uint32_t epoch;
   const unsigned long long* hist;  // RADIX digit counts for this pass
@@ -204,7 +199,8 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
   __syncthreads();
   // A CTA may start while the kernel before (the pass that writes its input, or
   // the histogram) still runs; what it wrote is there from here on. Every load
-  // of it takes its address from sm.tile, so none is moved up before this.
+  // of it takes its address from sm.tile, so none is moved up before this. (The
+  // ticket was cleared before that kernel started: sort_pass_chained.)
   if (a.chained) asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t tile = sm.tile;
   const int64_t tbase = tile * TILE;
@@ -402,7 +398,7 @@ template <int ITEMS>
 void launch_pass(const PassArgs& a, int64_t tiles, cudaStream_t s, bool from_edges, bool place, bool narrow,
                  bool unstable) {
   constexpr size_t bytes = sizeof(PassSmem<ITEMS>);
-  cudaLaunchAttribute attr;  // (without effect after anything but a kernel)
+  cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
@@ -511,7 +507,7 @@ wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, 
     a.in = src;
     a.out = dst;
     a.n = n;
-    a.chained = tiles <= CHAIN_TILES;
+    a.chained = sort_pass_chained(ready, p, tiles);
     a.shift = (uint32_t)(shift0 + p * RADIX_BITS);
     a.epoch = (uint32_t)(p + 1);
     a.hist = hist + p * RADIX;
