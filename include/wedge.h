@@ -489,8 +489,11 @@ WEDGE_API wedge_status wedge_classify(const wedge_graph* g, const wedge_bins* b,
  *   Synchronises s. Needs about 4m + 44n bytes of device memory beyond the
  *   graph (m undirected edges), and about 22 bytes for each of m, but at most
  *   2^27 (or the largest degree, if that is more), edges.
- *   Errors: EINVAL for NULL handles or bins of another graph; ENOMEM;
- *   ECUDA; ETIMEOUT (a bounded look-back wait gave up).
+ *   Errors: EINVAL for NULL handles or bins of another graph, or if other
+ *   than half of the CSR's entries go to a larger (degree, id), which an
+ *   imported CSR that is not symmetric may have (t_i is then zeros; one
+ *   that has half is counted, and means nothing); ENOMEM; ECUDA; ETIMEOUT (a
+ *   bounded look-back wait gave up).
  * ------------------------------------------------------------------------ */
 typedef struct {
   uint64_t triangles;

@@ -26,6 +26,13 @@
 // Vertices are taken in groups of at most GROUP_EDGES in-edges, highest ranks
 // first, so that the edges' scratch is bounded; rows fill from their ends, and
 // the tails that a group reads are there when it is counted.
+//
+// Symmetry of an imported CSR is its owner's promise. What the kernels rely on
+// is less: that m entries go to a lower rank (one_way). Every buffer of edges
+// holds m, and the second look at the entries gives each the place that the
+// first counted for it, so with m of them all places of in-lists and rows are
+// filled, with ranks in order, in any CSR of strictly ascending rows. With
+// another number nothing after the scans runs, and the call fails.
 #include <string.h>
 
 #include <algorithm>
@@ -69,6 +76,11 @@ __device__ __forceinline__ int32_t next_row(const int64_t* __restrict__ off, int
     if (__ldg(off + mid) <= e) lo = mid; else hi = mid;
   }
   return lo;
+}
+
+// Whether m entries go to a lower rank (in_off[n] is their number).
+__device__ __forceinline__ bool one_way(const int64_t* __restrict__ in_off, uint32_t n, int64_t m) {
+  return __ldg(in_off + n) == m;
 }
 
 __global__ __launch_bounds__(EX_THREADS) void k_degree_keys(const int32_t* __restrict__ deg, int32_t n,
@@ -132,7 +144,7 @@ struct OrientArgs {
   int32_t r0, r1;         // EMIT: the group's ranks
   uint64_t* keys;         // EMIT: u << 32 | place in the group's in-lists
   uint32_t* v_of;         // EMIT: v by place
-  uint64_t edges;         // EMIT: places
+  int64_t m;              // EMIT: places in all in-lists
 };
 
 // Every adjacency entry (v, u) with rank(u) < rank(v): counted for both ends,
@@ -143,7 +155,7 @@ __global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
   const int lane = threadIdx.x & 31;
   const uint32_t le = lanemask_lt() | (1u << lane);
   const int64_t base = ((int64_t)blockIdx.x * EX_WARPS + (threadIdx.x >> 5)) * (32 * a.steps);
-  if (base >= a.n_adj) return;
+  if (base >= a.n_adj || (EMIT && !one_way(a.in_off, (uint32_t)a.n, a.m))) return;
   int32_t x = row_of(a.off, a.n, min(base + lane, a.n_adj - 1)), rx = __ldg(a.rank + x);
   for (int i = 0; i < a.steps; ++i) {
     const int64_t e = base + i * 32 + lane;
@@ -175,58 +187,52 @@ __global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
       if (keep) {
         const uint64_t pos = (uint64_t)(__ldg(a.in_off + rx) - __ldg(a.in_off + a.r0)) + (uint32_t)at +
                              __popc(mine & lanemask_lt());
-        if (pos < a.edges) {  // (always, unless the graph is not symmetric)
-          a.keys[pos] = ((uint64_t)(uint32_t)ry << 32) | pos;
-          a.v_of[pos] = (uint32_t)rx;
-        }
+        a.keys[pos] = ((uint64_t)(uint32_t)ry << 32) | pos;
+        a.v_of[pos] = (uint32_t)rx;
       }
     }
   }
 }
 
 // Last place of each u's run in the group's edges sorted by u.
-// (u < n here and below: always, unless the graph is not symmetric and places
-// were left empty.)
-__global__ __launch_bounds__(EX_THREADS) void k_run_ends(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
+__global__ __launch_bounds__(EX_THREADS) void k_run_ends(const uint64_t* __restrict__ keys, int64_t m,
                                                          uint32_t* __restrict__ run_end) {
   const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
   if (i >= m) return;
   const uint32_t u = (uint32_t)(keys[i] >> 32);
-  if (u >= n) return;
   if (i + 1 == m || (uint32_t)(keys[i + 1] >> 32) != u) run_end[u] = (uint32_t)(i + 1);
 }
 
 // After a group: how many entries each row holds now.
-__global__ __launch_bounds__(EX_THREADS) void k_run_add(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
+__global__ __launch_bounds__(EX_THREADS) void k_run_add(const uint64_t* __restrict__ keys, int64_t m,
                                                         const uint32_t* __restrict__ run_end,
                                                         uint32_t* __restrict__ filled) {
   const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
   if (i >= m) return;
   const uint32_t u = (uint32_t)(keys[i] >> 32);
-  if (u >= n) return;
   if (i == 0 || (uint32_t)(keys[i - 1] >> 32) != u) filled[u] += run_end[u] - (uint32_t)i;
 }
 
 // Rows N+(u), from their ends: sorted edge i (u, and by its place the v) goes
 // before the entries of higher rank, and its in-list place learns how many
-// these are. WHOLE: the group is all there is, so i is the place in the rows.
+// these are. WHOLE: the group is all there is, so i is the place in the rows,
+// and whether all of it was filled is not known to the host.
 template <bool WHOLE>
 __global__ __launch_bounds__(EX_THREADS) void k_rows(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
+                                                     const int64_t* __restrict__ in_off,
                                                      const uint32_t* __restrict__ v_of,
                                                      const int64_t* __restrict__ row_off,
                                                      const uint32_t* __restrict__ run_end,
                                                      const uint32_t* __restrict__ filled, uint32_t* __restrict__ rows,
-                                                     int64_t n_rows, uint2* __restrict__ rec) {
+                                                     uint2* __restrict__ rec) {
   const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
-  if (i >= m) return;
+  if (i >= m || (WHOLE && !one_way(in_off, n, m))) return;
   const uint64_t key = __ldcs(keys + i);
   const uint32_t u = (uint32_t)(key >> 32), pos = (uint32_t)key;
-  if (u >= n || pos >= m) return;
   const int64_t row_end = __ldg(row_off + u + 1);
   const uint32_t after = WHOLE ? (uint32_t)(row_end - 1 - i)
                                : __ldg(filled + u) + (__ldg(run_end + u) - 1u - (uint32_t)i);
-  const int64_t at = row_end - 1 - (int64_t)after;
-  if (at < n_rows) rows[at] = __ldg(v_of + pos);  // (always, unless the graph is not symmetric)
+  rows[row_end - 1 - (int64_t)after] = __ldg(v_of + pos);
   rec[pos] = make_uint2(u, after);
 }
 
@@ -242,11 +248,11 @@ struct CountArgs {
   uint32_t nb;
   uint32_t n;
   int64_t m;               // entries of rows
-  int64_t edges;           // entries of rec
   uint32_t grab;           // vertices a warp takes per ticket
   int32_t r0, r1;          // the group's ranks
   unsigned long long* pbq; // [nb][4] (class 1..3 used)
   unsigned long long* t_i; // per-vertex closed wedges or nullptr
+  uint32_t* err;           // DERR_BAD_ID: not one_way
   unsigned int* next;      // work counter of the warp kernel
   uint2* units;            // (v, part of its in-list) for the CTA kernels: medium rows from the front, long from the back
   uint32_t max_units;
@@ -339,10 +345,8 @@ template <bool COUNTERS, typename Row>
 __device__ __forceinline__ void count_tails(const CountArgs& a, const Row& nv, const uint32_t* s_lo,
                                             unsigned long long* hist, uint2 r, uint32_t bv, uint32_t* hits,
                                             uint32_t* seg, uint32_t (&cv)[3], int lane) {
-  if (r.x >= a.n) r.y = 0;  // (here and below: only if the graph is not symmetric)
   const uint32_t my_bin = r.y ? rank_bin(s_lo, a.nb, r.x) : 0u, my_end_u = s_lo[my_bin + 1];
   const int64_t my_row_end = r.y ? __ldg(a.row_off + r.x + 1) : 0;
-  if (my_row_end > a.m || my_row_end < (int64_t)r.y) r.y = 0;
   const uint64_t my_tail = (uint64_t)(my_row_end - r.y);
   const uint32_t end_v = s_lo[bv + 1];
   uint32_t found = 0, with_u = 0, with_v = 0;  // this lane's in-edge
@@ -461,6 +465,10 @@ __global__ __launch_bounds__(EX_THREADS) void k_tri_hash_warp(CountArgs a) {
   __shared__ uint32_t s_table[EX_WARPS][WARP_SLOTS];
   __shared__ uint32_t s_hits[EX_WARPS][WARP_SLOTS];
   __shared__ uint32_t s_seg[EX_WARPS][32];
+  if (!one_way(a.in_off, a.n, a.m)) {  // (then no unit is queued either)
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, DERR_BAD_ID);
+    return;
+  }
   for (int i = threadIdx.x; i <= (int)a.nb; i += EX_THREADS) s_lo[i] = a.bin_lo[i];
   for (int i = threadIdx.x; i < (int)a.nb * 4; i += EX_THREADS) s_hist[i] = 0;
   for (int i = threadIdx.x; i < EX_WARPS * WARP_SLOTS; i += EX_THREADS) (&s_hits[0][0])[i] = 0;
@@ -479,10 +487,9 @@ __global__ __launch_bounds__(EX_THREADS) void k_tri_hash_warp(CountArgs a) {
     for (uint32_t i = first; i < last; ++i) {
       const uint32_t v = (uint32_t)a.r1 - 1u - i;
       const int64_t row = __ldg(a.row_off + v), in = __ldg(a.in_off + v);
-      // (the bounds hold by themselves unless the graph is not symmetric)
-      const int64_t d = min(a.m, __ldg(a.row_off + v + 1)) - row;
-      const int64_t k = min(in0 + a.edges, __ldg(a.in_off + v + 1)) - in;
-      if (d <= 0 || k <= 0) continue;
+      const int64_t d = __ldg(a.row_off + v + 1) - row;
+      const int64_t k = __ldg(a.in_off + v + 1) - in;
+      if (d == 0 || k == 0) continue;
       if (d > WARP_ROW || k > WARP_IN) {
         const uint32_t parts = (uint32_t)((k + UNIT_IN - 1) / UNIT_IN);
         uint32_t at = 0;
@@ -571,9 +578,9 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
     const uint32_t v = unit.x;
     const int64_t row_at = __ldg(a.row_off + v);
     const uint32_t* row = a.rows + row_at;
-    const uint32_t d = (uint32_t)(min(a.m, __ldg(a.row_off + v + 1)) - row_at);
+    const uint32_t d = (uint32_t)(__ldg(a.row_off + v + 1) - row_at);
     const int64_t in = __ldg(a.in_off + v) + (int64_t)unit.y * UNIT_IN;
-    const uint32_t k = (uint32_t)min((int64_t)UNIT_IN, min(in0 + a.edges, __ldg(a.in_off + v + 1)) - in);
+    const uint32_t k = (uint32_t)min((int64_t)UNIT_IN, __ldg(a.in_off + v + 1) - in);
     const uint32_t range = a.n - 1u - v;  // ranks above v
     const bool in_map = range <= (uint32_t)MAP_BITS && d <= (uint32_t)SLOTS;
     const bool in_table = !in_map && 2u * d <= (uint32_t)SLOTS;
@@ -635,6 +642,8 @@ int ctas_per_sm(F* f, int threads, size_t smem) {
   }
   return std::max(n, 1);
 }
+
+wedge_status not_symmetric() { return fail(WEDGE_EINVAL, "wedge_exact: the graph's CSR is not symmetric"); }
 
 unsigned blocks_for(int64_t items) { return (unsigned)((items + EX_THREADS - 1) / EX_THREADS); }
 
@@ -774,6 +783,7 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
   dfree(scratch, s);
   scratch = nullptr;
   oa.lower = taken;
+  oa.m = m;
 
   // 3-4. groups of ranks, highest first
   {
@@ -785,6 +795,9 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
     const int64_t cap = std::max<int64_t>(GROUP_EDGES, g->max_degree);
     int64_t largest = m;
     if (m > cap) {
+      int64_t all = 0;
+      EXACT_TRY(in_at(n, &all));
+      if (all != m) return done(not_symmetric());
       largest = 0;
       while (cut.back().second > 0) {
         const int64_t top = cut.back().second;
@@ -832,18 +845,17 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
       oa.r1 = r1;
       oa.keys = keys;
       oa.v_of = v_of;
-      oa.edges = (uint64_t)edges;
       EXACT_DO(launch("exact_edges", s, [&] { k_orient<true><<<tiles, EX_THREADS, 0, s>>>(oa); }));
       EXACT_DO(radix_sort_u64(keys, alt, edges, key_bits, scratch, ctl, s, &sorted, SortScratch::unused, 32));
       rec = reinterpret_cast<uint2*>(sorted == keys ? alt : keys);  // the sort's other buffer
       EXACT_DO(launch("exact_rows", s, [&] {
         const unsigned blocks = blocks_for(edges);
         if (edges == m) {
-          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, v_of, row_off, run_end, fill, rows, m, rec);
+          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, in_off, v_of, row_off, run_end, fill, rows, rec);
         } else {
-          k_run_ends<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, run_end);
-          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, v_of, row_off, run_end, fill, rows, m, rec);
-          k_run_add<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, run_end, fill);
+          k_run_ends<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end);
+          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, in_off, v_of, row_off, run_end, fill, rows, rec);
+          k_run_add<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end, fill);
         }
       }));
       CountArgs ca{};
@@ -856,11 +868,11 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
       ca.nb = nb;
       ca.n = (uint32_t)n;
       ca.m = m;
-      ca.edges = edges;
       ca.r0 = r0;
       ca.r1 = r1;
       ca.pbq = pbq;
       ca.t_i = reinterpret_cast<unsigned long long*>(t_i);
+      ca.err = ctl;
       ca.next = ctl + 1;
       ca.units = units;
       ca.max_units = (uint32_t)max_units;
@@ -889,6 +901,7 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
 #undef EXACT_TRY
 #undef EXACT_DO
   if (herr & DERR_TIMEOUT) return done(fail(WEDGE_ETIMEOUT, "wedge_exact: a look-back wait gave up"));
+  if (herr & DERR_BAD_ID) return done(not_symmetric());
   uint64_t closed = 0;
   for (uint32_t k = 0; k < inf.n_bins; ++k) {
     uint64_t sum = 0;
