@@ -218,6 +218,12 @@ __global__ __launch_bounds__(BIN_THREADS) void k_bin_guide(const uint64_t* __res
   }
 }
 
+// Shared memory of k_bin_scatter.
+constexpr size_t scatter_smem(uint32_t nb) {
+  return nb * (BIN_THREADS * sizeof(uint16_t) + sizeof(int64_t) + sizeof(uint16_t)) +
+         BIN_TILE * (sizeof(int32_t) + sizeof(uint16_t));
+}
+
 // Second pass: the vertices of degree >= 2 of each (bin, tile) go to the
 // tile's position in the bin, in id order, with their degrees beside them.
 // Each thread takes 16 consecutive ids and has a counter of its own per bin;
@@ -483,9 +489,10 @@ extern "C" wedge_status wedge_bin(const wedge_graph* g, const wedge_bin_params* 
   if ((st = dalloc_n(&b->gtab, nb, s, "wedge_bin: guide")) != WEDGE_OK) return bail(st);
   if (n2 > 0) {
     if ((st = dalloc_n(&ldeg, (size_t)n2, s, "wedge_bin")) != WEDGE_OK) return bail(st);
-    const size_t smem = nb * (BIN_THREADS * sizeof(uint16_t) + sizeof(int64_t) + sizeof(uint16_t)) +
-                        BIN_TILE * (sizeof(int32_t) + sizeof(uint16_t));
-    BIN_TRY(cudaFuncSetAttribute(k_bin_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "wedge_bin");
+    static OncePerDevice once;
+    st = once([] { return allow_shared(k_bin_scatter, scatter_smem(WEDGE_MAX_BINS), "wedge_bin: shared memory"); });
+    if (st != WEDGE_OK) return bail(st);
+    const size_t smem = scatter_smem(nb);
     st = launch("bin_scatter", s, [&] {
       k_bin_scatter<<<(unsigned)n_tiles, BIN_THREADS, smem, s>>>(g->deg, n, b->lo_dev, nb, n_tiles, pos_base,
                                                                  b->L, ldeg, n2, derr);

@@ -16,9 +16,8 @@ namespace wedge {
 namespace {
 thread_local char g_err[512] = "";
 
-constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kMaxDevices] = {};
+cudaMemPool_t g_pool[MAX_DEVICES] = {};
 
 // Test hook (wedge_test_fail_allocation): allocations that still succeed
 // before one is refused; negative when disarmed.
@@ -65,7 +64,7 @@ cudaMemPool_t pool_for_current(cudaError_t* err) {
   int dev = 0;
   *err = cudaGetDevice(&dev);
   if (*err != cudaSuccess) return nullptr;
-  if (dev < 0 || dev >= kMaxDevices) {
+  if (dev < 0 || dev >= MAX_DEVICES) {
     *err = cudaErrorInvalidDevice;
     return nullptr;
   }
@@ -325,7 +324,7 @@ void wedge_test_fail_allocation(int64_t after) { g_fail_after.store(after < 0 ? 
 
 uint64_t wedge_pool_used_bytes(void) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) {
     cudaGetLastError();
     return 0;
   }

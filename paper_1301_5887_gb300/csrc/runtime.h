@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 #include "../../include/wedge.h"
@@ -35,6 +36,41 @@ wedge_status dalloc_n(T** p, size_t n, cudaStream_t s, const char* what) {
 }
 
 int sm_count();
+
+constexpr int MAX_DEVICES = 64;
+
+// What a kernel needs done before its first launch on a device (its attributes
+// belong to the device): run where it has not succeeded on the current device yet.
+// Threads that come first at the same time all run it, so it sets constants:
+// a kernel's shared memory limit, say, is that of its largest launch, never of
+// one call's, which could come between another's limit and launch.
+class OncePerDevice {
+ public:
+  template <typename F>
+  wedge_status operator()(F&& f) {
+    int dev = -1;
+    WEDGE_CUDA_TRY(cudaGetDevice(&dev), "current device");
+    return on(dev, std::forward<F>(f));
+  }
+  template <typename F>
+  wedge_status on(int dev, F&& f) {
+    const uint64_t bit = dev >= 0 && dev < MAX_DEVICES ? uint64_t(1) << dev : 0;
+    if (done_.load(std::memory_order_acquire) & bit) return WEDGE_OK;
+    const wedge_status st = f();
+    if (st == WEDGE_OK) done_.fetch_or(bit, std::memory_order_release);
+    return st;
+  }
+
+ private:
+  std::atomic<uint64_t> done_{0};
+};
+
+// Lets a kernel be launched with up to `bytes` of dynamic shared memory on the current device.
+template <typename K>
+wedge_status allow_shared(K* kernel, size_t bytes, const char* what) {
+  WEDGE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
+  return WEDGE_OK;
+}
 
 // Pinned host blocks, cached by power-of-two size class and reused (pinning
 // and unpinning are slow and may synchronise the device).
