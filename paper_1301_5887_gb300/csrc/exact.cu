@@ -633,15 +633,26 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
 constexpr int MID_THREADS = 256, MID_SLOTS = 2048, MID_BITS = 1 << 16;    // rows up to 1024
 constexpr int BIG_THREADS = 512, BIG_SLOTS = 16384, BIG_BITS = 1 << 19;   // rows beyond (table up to 8192)
 
-template <typename F>
-int ctas_per_sm(F* f, int threads, size_t smem) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    n = 0;
+// CTAs of a kernel that the current device's SMs hold, asked for once a device.
+class CtasPerSm {
+ public:
+  template <typename F>
+  int operator()(F* f, int threads, size_t smem) {
+    int dev = -1, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) dev = 0;
+    if ((n = n_[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return 1;
+    }
+    n = std::max(n, 1);
+    n_[dev].store(n, std::memory_order_relaxed);
+    return n;
   }
-  return std::max(n, 1);
-}
+
+ private:
+  std::atomic<int> n_[MAX_DEVICES] = {};
+};
 
 wedge_status not_symmetric() { return fail(WEDGE_EINVAL, "wedge_exact: the graph's CSR is not symmetric"); }
 
@@ -829,12 +840,12 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
     constexpr auto big_kernel = k_tri_hash_cta<BIG_THREADS, BIG_SLOTS, BIG_BITS>;
     constexpr size_t mid_smem = sizeof(CtaSmem<MID_THREADS, MID_SLOTS, MID_BITS>);
     constexpr size_t big_smem = sizeof(CtaSmem<BIG_THREADS, BIG_SLOTS, BIG_BITS>);
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem);
-    EXACT_TRY(attr);
-    static const int warp_ctas = ctas_per_sm(k_tri_hash_warp, EX_THREADS, 0);
-    static const int mid_ctas = ctas_per_sm(mid_kernel, MID_THREADS, mid_smem);
-    static const int big_ctas = ctas_per_sm(big_kernel, BIG_THREADS, big_smem);
+    static OncePerDevice once;
+    static CtasPerSm warp_occupancy, mid_occupancy, big_occupancy;
+    EXACT_DO(once([&] { return allow_shared(big_kernel, big_smem, "wedge_exact: shared memory"); }));
+    const int warp_ctas = warp_occupancy(k_tri_hash_warp, EX_THREADS, 0);
+    const int mid_ctas = mid_occupancy(mid_kernel, MID_THREADS, mid_smem);
+    const int big_ctas = big_occupancy(big_kernel, BIG_THREADS, big_smem);
     const int sms = sm_count();
     for (size_t gi = 0; gi + 1 < cut.size(); ++gi) {
       const int32_t r1 = cut[gi].first, r0 = cut[gi + 1].first;

@@ -135,13 +135,12 @@ template <bool VEC, bool WRITE, int NP>
 wedge_status launch_expand(int grid, size_t smem, cudaStream_t s, const int32_t* src, const int32_t* dst, int64_t m,
                            int32_t n, uint32_t b, uint64_t sentinel, int passes, uint64_t* keys,
                            unsigned long long* hist, unsigned long long* hist_total, uint32_t* err) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_expand<VEC, WRITE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)(SORT_MAX_PASSES * 256 * HIST_COPIES * sizeof(uint32_t)));
-    if (e != cudaSuccess) return cuda_fail(e, "wedge_graph_build: shared memory");
-    attr_set = true;
-  }
+  static OncePerDevice once;
+  const wedge_status st = once([] {
+    return allow_shared(k_expand<VEC, WRITE, NP>, SORT_MAX_PASSES * 256 * HIST_COPIES * sizeof(uint32_t),
+                        "wedge_graph_build: shared memory");
+  });
+  if (st != WEDGE_OK) return st;
   k_expand<VEC, WRITE, NP><<<grid, EXPAND_THREADS, smem, s>>>(src, dst, m, n, b, sentinel, passes, keys, hist,
                                                               hist_total, err);
   return WEDGE_OK;

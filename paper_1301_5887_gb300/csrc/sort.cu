@@ -386,12 +386,12 @@ __global__ __launch_bounds__(SORT_THREADS, SORT_MIN_BLOCKS) void k_sort_pass(Pas
 template <int ITEMS, typename F>
 void for_each_pass(F&& f) {
   constexpr size_t bytes = sizeof(PassSmem<ITEMS>);
-  f(reinterpret_cast<const void*>(k_sort_pass<false, false, true, RADIX_BITS, false, ITEMS>), bytes);
-  f(reinterpret_cast<const void*>(k_sort_pass<true, false, true, RADIX_BITS, false, ITEMS>), bytes);
-  f(reinterpret_cast<const void*>(k_sort_pass<false, false, false, RADIX_BITS, false, ITEMS>), bytes);
-  f(reinterpret_cast<const void*>(k_sort_pass<true, true, true, RADIX_BITS, false, ITEMS>), bytes);
-  f(reinterpret_cast<const void*>(k_sort_pass<true, true, true, 4, false, ITEMS>), bytes);
-  f(reinterpret_cast<const void*>(k_sort_pass<false, false, false, RADIX_BITS, true, ITEMS>), bytes);
+  f(k_sort_pass<false, false, true, RADIX_BITS, false, ITEMS>, bytes);
+  f(k_sort_pass<true, false, true, RADIX_BITS, false, ITEMS>, bytes);
+  f(k_sort_pass<false, false, false, RADIX_BITS, false, ITEMS>, bytes);
+  f(k_sort_pass<true, true, true, RADIX_BITS, false, ITEMS>, bytes);
+  f(k_sort_pass<true, true, true, 4, false, ITEMS>, bytes);
+  f(k_sort_pass<false, false, false, RADIX_BITS, true, ITEMS>, bytes);
 }
 
 template <int ITEMS>
@@ -482,18 +482,18 @@ wedge_status radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, 
                    "radix sort: clear scratch");
   }
 
-  static bool attr_set = false;
-  if (!attr_set) {
+  static OncePerDevice once;
+  st = once([] {
     wedge_status fst = WEDGE_OK;
-    auto allow = [&](const void* f, size_t bytes) {
-      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      if (e != cudaSuccess && fst == WEDGE_OK) fst = cuda_fail(e, "radix sort: shared memory");
+    auto allow = [&](auto* kernel, size_t bytes) {
+      const wedge_status ast = allow_shared(kernel, bytes, "radix sort: shared memory");
+      if (fst == WEDGE_OK) fst = ast;
     };
     for_each_pass<SORT_ITEMS>(allow);
     for_each_pass<SMALL_ITEMS>(allow);
-    if (fst != WEDGE_OK) return fst;
-    attr_set = true;
-  }
+    return fst;
+  });
+  if (st != WEDGE_OK) return st;
   if (emit && emit->n_keys && !small)
     return fail(WEDGE_EINVAL, "radix sort: a number of keys on the device needs a small sort");
   if (emit && shift0 < 32) return fail(WEDGE_EINVAL, "radix sort: placement needs keys sorted from bit 32");

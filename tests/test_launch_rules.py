@@ -29,3 +29,21 @@ def test_sort_pass_waits_for_the_clear_of_its_tickets(tmp_path, ready, first):
       printf("%%d ", (int)sort_pass_chained(SortScratch::%s, p, tiles));""" % ready)
     few = [first] + [1] * 7
     assert [int(x) for x in out] == few * 3 + [0] * 8
+
+
+def test_once_per_device(tmp_path):
+    """What a kernel needs before its first launch is done on each device, and again where it failed."""
+    out = _run(tmp_path, """
+  OncePerDevice once;
+  int runs[3] = {};
+  auto on = [&](int dev, wedge_status st) {
+    once.on(dev, [&] { ++runs[dev]; return st; });
+  };
+  on(0, WEDGE_ECUDA);
+  on(0, WEDGE_OK);
+  on(0, WEDGE_OK);
+  on(2, WEDGE_OK);
+  on(1, WEDGE_OK);
+  on(2, WEDGE_ECUDA);
+  printf("%d %d %d", runs[0], runs[1], runs[2]);""")
+    assert [int(x) for x in out] == [2, 1, 1]
