@@ -116,7 +116,6 @@ __global__ __launch_bounds__(BIN_THREADS) void k_bin_count(const int32_t* __rest
 // found by one look into the guide and two or three halvings instead of
 // log2(n_b) (sampling kernel at Kronecker scale 22, 16.3 M samples: 1.24 to
 // 1.05 ms; 2 or 1 vertices a cell: no faster).
-constexpr uint32_t GUIDE_PER = 4;
 constexpr int BOUND_THREADS = WEDGE_MAX_BINS + 32;
 
 // W at the bin boundaries: bound[k] = W[start of bin k], k = 0 .. nb (bins 0
@@ -483,8 +482,7 @@ extern "C" wedge_status wedge_bin(const wedge_graph* g, const wedge_bin_params* 
 
   if ((st = dalloc_n(&b->L, (size_t)(n2 > 0 ? n2 : 1), s, "wedge_bin: L")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&b->W, (size_t)n2 + 1, s, "wedge_bin: W")) != WEDGE_OK) return bail(st);
-  // bin k's guide takes at most n_b / GUIDE_PER + 2 entries from start / GUIDE_PER + 2 k on
-  const size_t guide_len = (size_t)(n2 / GUIDE_PER) + 2 * (size_t)nb + 2;
+  const size_t guide_len = guide_alloc(n2, nb);
   if ((st = dalloc_n(&b->guide, guide_len, s, "wedge_bin: guide")) != WEDGE_OK) return bail(st);
   if ((st = dalloc_n(&b->gtab, nb, s, "wedge_bin: guide")) != WEDGE_OK) return bail(st);
   if (n2 > 0) {

@@ -429,10 +429,6 @@ struct BuildBuffers {
   }
 };
 
-// Entries to allocate for an adjacency array: whole 32-byte sectors, which
-// the closure search reads as a whole.
-size_t adj_alloc(int64_t n_adj) { return ((size_t)(n_adj > 0 ? n_adj : 1) + 7) & ~(size_t)7; }
-
 void free_graph(wedge_graph* g, cudaStream_t s) {
   if (!g) return;
   dfree(g->off, s);

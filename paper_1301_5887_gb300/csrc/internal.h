@@ -47,6 +47,15 @@ struct wedge_bins {
 
 namespace wedge {
 
+// Entries allocated for an adjacency array of n_adj: whole 32-byte sectors,
+// which the closure search reads as a whole.
+inline size_t adj_alloc(int64_t n_adj) { return ((size_t)(n_adj > 0 ? n_adj : 1) + 7) & ~(size_t)7; }
+
+// Vertices of a bin that share a cell of its guide, at least, and the guide's
+// entries: bin k's take at most n_b / GUIDE_PER + 2 from start / GUIDE_PER + 2 k on.
+constexpr uint32_t GUIDE_PER = 4;
+inline size_t guide_alloc(int64_t n2, uint32_t nb) { return (size_t)(n2 / GUIDE_PER) + 2 * (size_t)nb + 2; }
+
 // Sort-scratch size and sort (sort.cu). The scratch starts with the digit
 // histograms (8 passes x 256 unsigned long long); a caller that produces the
 // keys may accumulate them there itself: after sort_clear for that many keys

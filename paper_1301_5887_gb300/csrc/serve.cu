@@ -89,17 +89,20 @@ uint64_t request_samples(const wedge_server_request& r, const wedge_bins* b) {
   return total;
 }
 
-// (The guide over W, a byte a vertex, is left out: a budget admits what it did
-// before there was one.)
-uint64_t graph_bytes(const wedge_graph* g, const wedge_bins* b) {
-  const uint64_t n = (uint64_t)g->n;
-  uint64_t bytes = 8 * (n + 1) + 4 * n + 4 * (uint64_t)(2 * g->n_input > 0 ? 2 * g->n_input : 1);
-  if (b) bytes += 4 * (uint64_t)b->info.n_wedge_vertices + 8 * ((uint64_t)b->info.n_wedge_vertices + 1);
-  return bytes;
+// What a resident graph and its bins hold: offsets, degrees and adjacency; L,
+// W, the guide over W and, per bin, its least degree and its guide's place.
+uint64_t resident_size(int64_t n_edges, uint64_t n, uint64_t n2, uint32_t nb) {
+  return 8 * (n + 1) + 4 * n + 4 * (uint64_t)adj_alloc(2 * n_edges) + 4 * n2 + 8 * (n2 + 1) +
+         4 * (uint64_t)guide_alloc((int64_t)n2, nb) + (8 + sizeof(GuideBin)) * (uint64_t)nb;
 }
 
+uint64_t graph_bytes(const wedge_graph* g, const wedge_bins* b) {
+  return resident_size(g->n_input, (uint64_t)g->n, (uint64_t)b->info.n_wedge_vertices, b->info.n_bins);
+}
+
+// The most that can be, before the graph is built.
 uint64_t graph_bytes_estimate(int64_t n_edges, int32_t n) {
-  return 8 * (uint64_t)(n_edges > 0 ? n_edges : 1) + 24 * (uint64_t)n + 16;
+  return resident_size(n_edges, (uint64_t)n, (uint64_t)n, WEDGE_MAX_BINS);
 }
 
 // Build scratch of wedge_graph_build: key buffers and look-back words.
