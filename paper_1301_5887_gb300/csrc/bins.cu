@@ -217,6 +217,13 @@ __global__ __launch_bounds__(BIN_THREADS) void k_bin_guide(const uint64_t* __res
   }
 }
 
+// Most bins that k_bin_scatter takes; k_bin_scatter_many takes more. In 24.6 KB
+// and 522 bytes a bin, four CTAs of the first fit an SM up to 60 bins, and one at
+// 256. Both forms, us (Kronecker scale 24 / 2 M vertices of alike degrees): 20
+// bins 61, 69 (kron); 36 bins 103, 102 / 27, 27; 49 and 47 bins 129, 109 / 27,
+// 31; 62 bins 156, 111 / 41, 33; 139 bins 299, 129; 249 bins 671, 141.
+constexpr uint32_t SCATTER_BINS = 52;
+
 // Shared memory of k_bin_scatter.
 constexpr size_t scatter_smem(uint32_t nb) {
   return nb * (BIN_THREADS * sizeof(uint16_t) + sizeof(int64_t) + sizeof(uint16_t)) +
@@ -323,6 +330,61 @@ __global__ __launch_bounds__(BIN_THREADS) void k_bin_scatter(const int32_t* __re
       L[at] = (int32_t)(tbase + s_id[i]);
       ldeg[at] = x;
     }
+  }
+}
+
+// The same for many bins. The counters per thread are 512 bytes a bin to clear,
+// scan and hold; here a warp takes 32 consecutive ids at a time, the lanes of a bin
+// find each other, and a counter per warp and bin gives them their place.
+__global__ __launch_bounds__(BIN_THREADS) void k_bin_scatter_many(const int32_t* __restrict__ deg, int32_t n,
+                                                                  const uint64_t* __restrict__ lo_g, uint32_t nb,
+                                                                  int64_t n_tiles, const int64_t* __restrict__ pos_base,
+                                                                  int32_t* __restrict__ L, int32_t* __restrict__ ldeg,
+                                                                  int64_t n2, uint32_t* err) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  int64_t* s_pos = reinterpret_cast<int64_t*>(smem);  // [warp][bin]: counts, then places in L
+  __shared__ DegreeBins s_bins;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t tile = blockIdx.x;
+  const int64_t first = tile * BIN_TILE + warp * (32 * BIN_ITEMS) + lane;
+  int32_t d[BIN_ITEMS];
+#pragma unroll
+  for (int i = 0; i < BIN_ITEMS; ++i) d[i] = first + 32 * i < n ? __ldg(deg + first + 32 * i) : 0;
+  for (int i = tid; i < BIN_WARPS * (int)nb; i += BIN_THREADS) s_pos[i] = 0;
+  s_bins.load(lo_g, nb);
+  int64_t* mine = s_pos + warp * nb;
+  const uint32_t lt = lanemask_lt();
+  uint32_t bin[BIN_ITEMS], peers[BIN_ITEMS];
+#pragma unroll
+  for (int i = 0; i < BIN_ITEMS; ++i) {
+    bin[i] = d[i] >= 2 ? s_bins.of(d[i]) : 0u;
+    peers[i] = __match_any_sync(FULL_MASK, bin[i]);
+    if (bin[i] && (peers[i] & lt) == 0) mine[bin[i]] += __popc(peers[i]);
+    __syncwarp();
+  }
+  __syncthreads();
+  for (uint32_t b = 2 + tid; b < nb; b += BIN_THREADS) {
+    int64_t pos = pos_base[mat_row(b, nb) * n_tiles + tile];
+    for (int w = 0; w < BIN_WARPS; ++w) {
+      const int64_t c = s_pos[w * nb + b];
+      s_pos[w * nb + b] = pos;
+      pos += c;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < BIN_ITEMS; ++i) {
+    const int64_t p0 = bin[i] ? mine[bin[i]] : 0;
+    __syncwarp();
+    if (bin[i]) {
+      if ((peers[i] & lt) == 0) mine[bin[i]] = p0 + __popc(peers[i]);
+      const int64_t at = p0 + __popc(peers[i] & lt);
+      if (in_bounds((uint64_t)at, (uint64_t)n2, err)) {
+        L[at] = (int32_t)(first + 32 * i);
+        ldeg[at] = d[i];
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -488,12 +550,14 @@ extern "C" wedge_status wedge_bin(const wedge_graph* g, const wedge_bin_params* 
   if (n2 > 0) {
     if ((st = dalloc_n(&ldeg, (size_t)n2, s, "wedge_bin")) != WEDGE_OK) return bail(st);
     static OncePerDevice once;
-    st = once([] { return allow_shared(k_bin_scatter, scatter_smem(WEDGE_MAX_BINS), "wedge_bin: shared memory"); });
+    st = once([] { return allow_shared(k_bin_scatter, scatter_smem(SCATTER_BINS), "wedge_bin: shared memory"); });
     if (st != WEDGE_OK) return bail(st);
-    const size_t smem = scatter_smem(nb);
+    const bool many = nb > SCATTER_BINS;
+    const size_t smem = many ? BIN_WARPS * nb * sizeof(int64_t) : scatter_smem(nb);
     st = launch("bin_scatter", s, [&] {
-      k_bin_scatter<<<(unsigned)n_tiles, BIN_THREADS, smem, s>>>(g->deg, n, b->lo_dev, nb, n_tiles, pos_base,
-                                                                 b->L, ldeg, n2, derr);
+      auto* kernel = many ? k_bin_scatter_many : k_bin_scatter;
+      kernel<<<(unsigned)n_tiles, BIN_THREADS, smem, s>>>(g->deg, n, b->lo_dev, nb, n_tiles, pos_base, b->L, ldeg, n2,
+                                                          derr);
     });
     if (st != WEDGE_OK) return bail(st);
     // W = exclusive prefix of the wedge counts over L, W[n2] = p
