@@ -478,7 +478,7 @@ WEDGE_API wedge_status wedge_classify(const wedge_graph* g, const wedge_bins* b,
  * Exact counts (Sec. 2.1, 2.2): the quantities the sampler estimates, by
  * enumerating every triangle once on the device (each edge oriented from
  * the smaller to the larger (degree, id); for each edge (u, v), the rest of
- * u's oriented row is looked up in v's). For every bin b: p_b (wedges centred in b) and
+ * u's oriented row is looked up in v's, or v's row in u's). For every bin b: p_b (wedges centred in b) and
  * pbq[b][q], the closed wedges centred in b whose two endpoints include
  * q - 1 vertices of b (q = 1, 2, 3; Alg. Phase 4c's classes), with
  * pbq[b][0] = p_b - pbq[b][1] - pbq[b][2] - pbq[b][3] (open wedges). Then
@@ -486,9 +486,11 @@ WEDGE_API wedge_status wedge_classify(const wedge_graph* g, const wedge_bins* b,
  * global c = 3t/p (Eq. (CC)).
  *   t_i: optional device uint64[n_vertices] receiving the closed wedges
  *     centred at each vertex (triangles at i); NULL skips them.
- *   Synchronises s. Needs about 4m + 44n bytes of device memory beyond the
- *   graph (m undirected edges), and about 22 bytes for each of m, but at most
- *   2^27 (or the largest degree, if that is more), edges.
+ *   Synchronises s. Needs about 4m + 36n bytes of device memory beyond the
+ *   graph (m undirected edges), and about 25 bytes for each of m, but at most
+ *   2^27 (or the largest degree, if that is more), edges. Where that is refused,
+ *   and for graphs with little to look up, the triangles are found another way, in
+ *   4m + 16n bytes: the same counts, of many triangles slower.
  *   Errors: EINVAL for NULL handles or bins of another graph, or if other
  *   than half of the CSR's entries go to a larger (degree, id), which an
  *   imported CSR that is not symmetric may have (t_i is then zeros; one
@@ -637,6 +639,15 @@ WEDGE_API void wedge_test_fail_allocation(int64_t after);
  * synchronises s. Errors: EINVAL (spin_limit out of range), ENOMEM, ECUDA;
  * WEDGE_OK only if the wait unexpectedly did not time out. */
 WEDGE_API wedge_status wedge_test_lookback_timeout(uint32_t spin_limit, wedge_stream s);
+/* wedge_exact by a form of the caller's choice (0: as wedge_exact, 1: tails, 2:
+ * whole rows) and with lower limits, so that small graphs reach what else only
+ * large ones do: in-edges of a group (at least 1; a vertex's are never split), the most
+ * ranks that a CTA's bit map covers and the longest row in a CTA's hash table (longer
+ * ones are searched in memory; only with form 1). The counts are the same. Errors: as
+ * wedge_exact, and EINVAL for a form or group out of range. */
+WEDGE_API wedge_status wedge_test_exact(const wedge_graph* g, const wedge_bins* b, uint64_t* t_i, wedge_stream s,
+                                        int form, int64_t group_edges, uint32_t map_ranks, uint32_t table_row,
+                                        wedge_exact_counts* out);
 
 #ifdef __cplusplus
 }

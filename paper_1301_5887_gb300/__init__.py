@@ -174,7 +174,7 @@ EXPORTS = ["wedge_status_str", "wedge_last_error", "wedge_version", "wedge_abi_s
            "wedge_server_destroy", "wedge_server_add_graph", "wedge_server_remove_graph", "wedge_server_submit",
            "wedge_server_wait", "wedge_server_stats", "wedge_probe_random_read", "wedge_triangle_stats",
            "wedge_exact", "wedge_pool_used_bytes", "wedge_test_fail_allocation", "wedge_test_lookback_timeout",
-           "wedge_graph_from_csr"]
+           "wedge_graph_from_csr", "wedge_test_exact"]
 
 _lib = None
 
@@ -258,6 +258,7 @@ def _configure(lib):
         "wedge_test_fail_allocation": ([i64], None),
         "wedge_test_lookback_timeout": ([u32, P], st),
         "wedge_graph_from_csr": ([P, P, i32, i64, P, P], st),
+        "wedge_test_exact": ([P, P, P, P, i32, i64, ctypes.c_uint32, ctypes.c_uint32, ctypes.POINTER(ExactCounts)], st),
     }
     for name, (args, res) in sig.items():
         f = getattr(lib, name)
@@ -486,14 +487,24 @@ def classify(graph: Graph, bins: Bins, v0, v1, v2, q, stream=None):
 def exact(graph: Graph, bins: Bins, t_i=None, stream=None) -> dict:
     """Exact triangle counts (wedge_exact): t, p_b, pbq[n_bins, 4] (q = 0 open,
     1..3 closed by class); t_i: optional device uint64 tensor of n_vertices."""
-    lib = load()
+    return _exact(load().wedge_exact, graph, bins, t_i, stream)
+
+
+def force_exact(graph: Graph, bins: Bins, t_i=None, form: int = 0, group_edges: int = 1 << 27,
+                map_ranks: int = 0xFFFFFFFF, table_row: int = 0xFFFFFFFF, stream=None) -> dict:
+    """Test hook: exact() by a form of choice and with lower limits (wedge_test_exact)."""
+    return _exact(load().wedge_test_exact, graph, bins, t_i, stream, int(form), int(group_edges), int(map_ranks),
+                  int(table_row))
+
+
+def _exact(call, graph, bins, t_i, stream, *limits):
     out = ExactCounts()
     pt = 0
     if t_i is not None:
         pt, arr = _ptr(t_i)
         if int(np.prod(arr.shape)) < graph.info().n_vertices:
             raise ValueError("t_i needs n_vertices entries")
-    _check(lib.wedge_exact(graph.handle, bins.handle, pt, _stream_handle(stream), ctypes.byref(out)))
+    _check(call(graph.handle, bins.handle, pt, _stream_handle(stream), *limits, ctypes.byref(out)))
     nb = out.n_bins
     return {"triangles": int(out.triangles), "p_total": int(out.p_total), "p_b": _words(out, "p_b", nb),
             "pbq": _words(out, "pbq", nb, 4)}

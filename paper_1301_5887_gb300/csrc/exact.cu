@@ -9,7 +9,8 @@
 // in N+(v):
 //   1. ranks: a radix sort of the degrees;
 //   2. exact_orient: counts, per vertex, the neighbours of lower and of higher
-//      rank; scans give the in-lists (the u of every v) and the rows N+;
+//      rank and marks the entries that go down; a scan gives the in-lists (the u of
+//      every v) and the rows N+;
 //   3. exact_edges: the oriented edges by v, in rank order; a stable radix sort
 //      by u then yields the rows N+(u) in rank order, and exact_rows records
 //      for every edge of an in-list how many entries of N+(u) come after v;
@@ -21,26 +22,26 @@
 // times as many entries (Kronecker scale 20: 4.4e9 against 1.2e9; 34.4 ms in
 // all that way, 5.2 ms this way; scale 24: 1.11 s and 0.25 s). The count is
 // bound by instructions and, where N+ rows are short, by the chain of loads per
-// vertex; graphs with next to no triangles pay the ranks and the sort for
-// nothing (uniform, 16 M edges: 2.1 and 2.3 ms).
-// Vertices are taken in groups of at most GROUP_EDGES in-edges, highest ranks
+// vertex. Graphs that would pay the ranks and the sort for nothing stream whole rows
+// (exact_rows.cu; the rule: takes_rows), as does one whose memory is refused.
+// Vertices are taken in groups of at most 2^27 in-edges, highest ranks
 // first, so that the edges' scratch is bounded; rows fill from their ends, and
 // the tails that a group reads are there when it is counted.
 //
 // Symmetry of an imported CSR is its owner's promise. What the kernels rely on
-// is less: that m entries go to a lower rank (one_way). Every buffer of edges
-// holds m, and the second look at the entries gives each the place that the
+// is less: that m entries go to a lower rank (`down` counts them). Every buffer of
+// edges holds m, and the second look at the entries gives each the place that the
 // first counted for it, so with m of them all places of in-lists and rows are
 // filled, with ranks in order, in any CSR of strictly ascending rows. With
-// another number nothing after the scans runs, and the call fails.
+// another number nothing after the first look does anything (the sort finds its
+// histograms empty and then writes to places below m), and the call fails.
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
-#include "device.cuh"
-#include "internal.h"
-#include "runtime.h"
+#include "exact.cuh"
 
 namespace wedge {
 namespace {
@@ -48,45 +49,32 @@ namespace {
 constexpr int EX_THREADS = 256;
 constexpr int EX_WARPS = EX_THREADS / 32;
 constexpr int OR_STEPS = 16;                            // 32-entry steps of a warp at most
-constexpr int64_t GROUP_EDGES = int64_t(1) << 27;       // in-edges of a group (unless one vertex has more)
 
-// Largest u in [0, n) with off[u] <= e (off ascending, off[0] = 0 <= e).
-__device__ __forceinline__ int32_t row_of(const int64_t* __restrict__ off, int32_t n, int64_t e) {
-  int32_t lo = 0, hi = n;
-  while (hi - lo > 1) {
-    const int32_t mid = lo + ((hi - lo) >> 1);
-    if (__ldg(off + mid) <= e) lo = mid; else hi = mid;
-  }
-  return lo;
+// Adds w to the counts of the digits of x, and a CTA's counts to the sort's histograms.
+constexpr int DIGIT_COUNTS = 4 * 256;
+__device__ __forceinline__ void count_digits(uint32_t* sh, int passes, uint32_t x, uint32_t w) {
+  for (int p = 0; p < passes; ++p) atomicAdd(&sh[p * 256 + ((x >> (8 * p)) & 255u)], w);
+}
+__device__ __forceinline__ void add_counts(const uint32_t* sh, int passes, unsigned long long* __restrict__ hist) {
+  for (int i = threadIdx.x; i < passes * 256; i += EX_THREADS)
+    if (sh[i]) atomicAdd(&hist[i], (unsigned long long)sh[i]);
 }
 
-// Row of entry e, given a row u with off[u] <= e: up to 32 steps forward
-// over consecutive (cached) offsets, the common case even with isolated
-// vertices, then a binary search, so a long run of empty rows costs O(log n)
-// instead of one step each.
-__device__ __forceinline__ int32_t next_row(const int64_t* __restrict__ off, int32_t n, int32_t u, int64_t e) {
-#pragma unroll 1
-  for (int t = 0; t < 32; ++t) {
-    if (e < __ldg(off + u + 1)) return u;
-    ++u;
+// Degrees as sort keys, with the sort's histograms.
+__global__ __launch_bounds__(EX_THREADS) void k_degree_keys(const int32_t* __restrict__ deg, int32_t n, int passes,
+                                                            uint64_t* __restrict__ keys,
+                                                            unsigned long long* __restrict__ hist) {
+  __shared__ uint32_t sh[DIGIT_COUNTS];
+  for (int i = threadIdx.x; i < DIGIT_COUNTS; i += EX_THREADS) sh[i] = 0;
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * EX_THREADS;
+  for (int64_t v = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x; v < n; v += stride) {
+    const uint32_t d = (uint32_t)__ldg(deg + v);
+    keys[v] = ((uint64_t)d << 32) | (uint64_t)v;
+    count_digits(sh, passes, d, 1u);
   }
-  int32_t lo = u, hi = n;  // off[lo] <= e < off[n]
-  while (hi - lo > 1) {
-    const int32_t mid = lo + ((hi - lo) >> 1);
-    if (__ldg(off + mid) <= e) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-// Whether m entries go to a lower rank (in_off[n] is their number).
-__device__ __forceinline__ bool one_way(const int64_t* __restrict__ in_off, uint32_t n, int64_t m) {
-  return __ldg(in_off + n) == m;
-}
-
-__global__ __launch_bounds__(EX_THREADS) void k_degree_keys(const int32_t* __restrict__ deg, int32_t n,
-                                                            uint64_t* __restrict__ keys) {
-  const int64_t v = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
-  if (v < n) keys[v] = ((uint64_t)(uint32_t)deg[v] << 32) | (uint64_t)v;
+  __syncthreads();
+  add_counts(sh, passes, hist);
 }
 
 // order[r] = the vertex of rank r, rank its inverse.
@@ -140,26 +128,32 @@ struct OrientArgs {
   int steps;              // 32-entry steps of a warp
   int32_t* lower;         // by rank: neighbours of lower rank (EMIT: taken so far)
   int32_t* higher;        // by rank: neighbours of higher rank
+  uint32_t* kept;         // which entries go to a lower rank, a bit each
+  unsigned long long* down;  // their number
   const int64_t* in_off;  // EMIT: in-list offsets by rank
   int32_t r0, r1;         // EMIT: the group's ranks
   uint64_t* keys;         // EMIT: u << 32 | place in the group's in-lists
   uint32_t* v_of;         // EMIT: v by place
+  uint32_t* u_of;         // EMIT: u by place
   int64_t m;              // EMIT: places in all in-lists
 };
 
-// Every adjacency entry (v, u) with rank(u) < rank(v): counted for both ends,
-// or (EMIT) given a place in v's in-list, if v is of the group. A warp takes up to
+// Every adjacency entry (v, u) with rank(u) < rank(v): counted for both ends and
+// marked, or (EMIT) given a place in v's in-list, if v is of the group. A warp takes up to
 // 512 consecutive entries, 32 at a time; the lanes of a row share one atomic.
 template <bool EMIT>
 __global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
   const int lane = threadIdx.x & 31;
   const uint32_t le = lanemask_lt() | (1u << lane);
   const int64_t base = ((int64_t)blockIdx.x * EX_WARPS + (threadIdx.x >> 5)) * (32 * a.steps);
-  if (base >= a.n_adj || (EMIT && !one_way(a.in_off, (uint32_t)a.n, a.m))) return;
+  if (base >= a.n_adj || (EMIT && *a.down != (unsigned long long)a.m)) return;
+  uint32_t down = 0;
   int32_t x = row_of(a.off, a.n, min(base + lane, a.n_adj - 1)), rx = __ldg(a.rank + x);
   for (int i = 0; i < a.steps; ++i) {
     const int64_t e = base + i * 32 + lane;
     if (e - lane >= a.n_adj) break;  // the whole warp
+    const uint32_t marked = EMIT ? __ldg(a.kept + (e >> 5)) : FULL_MASK;  // (e - lane is a multiple of 32)
+    if (EMIT && marked == 0) continue;
     bool keep = false;
     int32_t ry = 0;
     if (e < a.n_adj) {
@@ -167,10 +161,14 @@ __global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
         x = next_row(a.off, a.n, x, e);
         rx = __ldg(a.rank + x);
       }
-      ry = __ldg(a.rank + __ldcs(a.adj + e));
-      keep = ry < rx && (!EMIT || (rx >= a.r0 && rx < a.r1));
+      if (!EMIT || ((marked >> lane & 1u) && rx >= a.r0 && rx < a.r1)) {
+        ry = __ldg(a.rank + __ldcs(a.adj + e));
+        keep = ry < rx;
+      }
     }
     const uint32_t kept = __ballot_sync(FULL_MASK, keep);
+    if (!EMIT && lane == 0) a.kept[e >> 5] = kept;
+    down += __popc(kept);
     if (kept == 0) continue;
     const int32_t before = __shfl_up_sync(FULL_MASK, rx, 1);
     const uint32_t starts = __ballot_sync(FULL_MASK, lane == 0 || before != rx);
@@ -189,9 +187,11 @@ __global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
                              __popc(mine & lanemask_lt());
         a.keys[pos] = ((uint64_t)(uint32_t)ry << 32) | pos;
         a.v_of[pos] = (uint32_t)rx;
+        a.u_of[pos] = (uint32_t)ry;
       }
     }
   }
+  if (!EMIT && lane == 0 && down) atomicAdd(a.down, (unsigned long long)down);
 }
 
 // Last place of each u's run in the group's edges sorted by u.
@@ -215,44 +215,49 @@ __global__ __launch_bounds__(EX_THREADS) void k_run_add(const uint64_t* __restri
 
 // Rows N+(u), from their ends: sorted edge i (u, and by its place the v) goes
 // before the entries of higher rank, and its in-list place learns how many
-// these are. WHOLE: the group is all there is, so i is the place in the rows,
-// and whether all of it was filled is not known to the host.
+// these are (alone: 4 bytes to random places; with u beside it, 134 MB of 16.8 M
+// edges, past L2, 529 us, so 305..323). WHOLE: the group is all there is, so i is the
+// place in the rows, and whether all of it was filled is not known to the host.
 template <bool WHOLE>
 __global__ __launch_bounds__(EX_THREADS) void k_rows(const uint64_t* __restrict__ keys, int64_t m, uint32_t n,
-                                                     const int64_t* __restrict__ in_off,
+                                                     const unsigned long long* __restrict__ down,
                                                      const uint32_t* __restrict__ v_of,
                                                      const int64_t* __restrict__ row_off,
                                                      const uint32_t* __restrict__ run_end,
                                                      const uint32_t* __restrict__ filled, uint32_t* __restrict__ rows,
-                                                     uint2* __restrict__ rec) {
+                                                     int64_t row_base, uint32_t* __restrict__ tail_of) {
   const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
-  if (i >= m || (WHOLE && !one_way(in_off, n, m))) return;
+  if (i >= m || (WHOLE && *down != (unsigned long long)m)) return;
   const uint64_t key = __ldcs(keys + i);
   const uint32_t u = (uint32_t)(key >> 32), pos = (uint32_t)key;
   const int64_t row_end = __ldg(row_off + u + 1);
-  const uint32_t after = WHOLE ? (uint32_t)(row_end - 1 - i)
+  const uint32_t after = WHOLE ? (uint32_t)(row_end - 1 - row_base - i)
                                : __ldg(filled + u) + (__ldg(run_end + u) - 1u - (uint32_t)i);
-  rows[row_end - 1 - (int64_t)after] = __ldg(v_of + pos);
-  rec[pos] = make_uint2(u, after);
+  rows[row_end - 1 - row_base - (int64_t)after] = __ldg(v_of + pos);
+  tail_of[pos] = after;
 }
 
 // ----------------------------------------------------------------- count --
 
 struct CountArgs {
-  const int64_t* row_off;  // n + 1, by rank
-  const uint32_t* rows;
   const int64_t* in_off;   // n + 1, by rank
-  const uint2* rec;        // the group's in-lists: u, entries of N+(u) after v
+  const int64_t* row_off;  // n + 1, by rank, from m on (the scan goes on from the in-lists)
+  const uint32_t* rows;
+  const uint32_t* u_of;    // the group's in-lists: u,
+  const uint32_t* tail_of; // and entries of N+(u) after v
   const int32_t* order;
   const uint32_t* bin_lo;  // first rank of each bin, then n
   uint32_t nb;
   uint32_t n;
   int64_t m;               // entries of rows
   uint32_t grab;           // vertices a warp takes per ticket
+  uint32_t map_ranks;      // most ranks of a bit map, and half the slots of a hash table, of the
+  uint32_t table_row;      // CTA kernels (as they are sized, or less)
   int32_t r0, r1;          // the group's ranks
   unsigned long long* pbq; // [nb][4] (class 1..3 used)
   unsigned long long* t_i; // per-vertex closed wedges or nullptr
-  uint32_t* err;           // DERR_BAD_ID: not one_way
+  const unsigned long long* down;  // entries that go to a lower rank
+  uint32_t* err;           // DERR_BAD_ID: they are not m
   unsigned int* next;      // work counter of the warp kernel
   uint2* units;            // (v, part of its in-list) for the CTA kernels: medium rows from the front, long from the back
   uint32_t max_units;
@@ -268,6 +273,10 @@ constexpr int UNIT_IN = 512;         // in-edges of a unit of the CTA kernels
 constexpr uint32_t GRAB = 8;         // vertices a warp takes per ticket at most
 
 __device__ __forceinline__ uint32_t slot_of(uint32_t w, uint32_t mask) { return (w * 0x9E3779B1u) >> 7 & mask; }
+
+__device__ __forceinline__ uint2 in_edge(const CountArgs& a, int64_t place) {
+  return make_uint2(__ldcs(a.u_of + place), __ldcs(a.tail_of + place));
+}
 
 // Insert key w (absent); the table has free slots (load <= 1/2).
 __device__ __forceinline__ void insert_key(uint32_t* table, uint32_t mask, uint32_t w) {
@@ -347,7 +356,7 @@ __device__ __forceinline__ void count_tails(const CountArgs& a, const Row& nv, c
                                             uint32_t* seg, uint32_t (&cv)[3], int lane) {
   const uint32_t my_bin = r.y ? rank_bin(s_lo, a.nb, r.x) : 0u, my_end_u = s_lo[my_bin + 1];
   const int64_t my_row_end = r.y ? __ldg(a.row_off + r.x + 1) : 0;
-  const uint64_t my_tail = (uint64_t)(my_row_end - r.y);
+  const uint64_t my_tail = (uint64_t)(my_row_end - a.m - r.y);
   const uint32_t end_v = s_lo[bv + 1];
   uint32_t found = 0, with_u = 0, with_v = 0;  // this lane's in-edge
   // w of a tail of a u whose bin ends at end_u: what it adds to found (low 10
@@ -465,7 +474,7 @@ __global__ __launch_bounds__(EX_THREADS) void k_tri_hash_warp(CountArgs a) {
   __shared__ uint32_t s_table[EX_WARPS][WARP_SLOTS];
   __shared__ uint32_t s_hits[EX_WARPS][WARP_SLOTS];
   __shared__ uint32_t s_seg[EX_WARPS][32];
-  if (!one_way(a.in_off, a.n, a.m)) {  // (then no unit is queued either)
+  if (*a.down != (unsigned long long)a.m) {  // (then no unit is queued either)
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, DERR_BAD_ID);
     return;
   }
@@ -486,8 +495,8 @@ __global__ __launch_bounds__(EX_THREADS) void k_tri_hash_warp(CountArgs a) {
     const uint32_t last = min(count, first + a.grab);
     for (uint32_t i = first; i < last; ++i) {
       const uint32_t v = (uint32_t)a.r1 - 1u - i;
-      const int64_t row = __ldg(a.row_off + v), in = __ldg(a.in_off + v);
-      const int64_t d = __ldg(a.row_off + v + 1) - row;
+      const int64_t row = __ldg(a.row_off + v) - a.m, in = __ldg(a.in_off + v);
+      const int64_t d = __ldg(a.row_off + v + 1) - a.m - row;
       const int64_t k = __ldg(a.in_off + v + 1) - in;
       if (d == 0 || k == 0) continue;
       if (d > WARP_ROW || k > WARP_IN) {
@@ -502,7 +511,7 @@ __global__ __launch_bounds__(EX_THREADS) void k_tri_hash_warp(CountArgs a) {
       const uint32_t bv = rank_bin(s_lo, a.nb, v);
       uint32_t cv[3] = {0, 0, 0};
       auto tails = [&](int64_t j) {
-        return j + lane < k ? __ldcs(a.rec + (in - in0) + j + lane) : make_uint2(0, 0);
+        return j + lane < k ? in_edge(a, in - in0 + j + lane) : make_uint2(0, 0);
       };
       if (d <= MEMORY_ROW) {  // a few entries are found faster than they are entered into a table
         for (int64_t j = 0; j < k; j += 32)
@@ -577,13 +586,13 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
     const uint2 unit = list[(int64_t)dir * q];
     const uint32_t v = unit.x;
     const int64_t row_at = __ldg(a.row_off + v);
-    const uint32_t* row = a.rows + row_at;
+    const uint32_t* row = a.rows + (row_at - a.m);
     const uint32_t d = (uint32_t)(__ldg(a.row_off + v + 1) - row_at);
     const int64_t in = __ldg(a.in_off + v) + (int64_t)unit.y * UNIT_IN;
     const uint32_t k = (uint32_t)min((int64_t)UNIT_IN, __ldg(a.in_off + v + 1) - in);
     const uint32_t range = a.n - 1u - v;  // ranks above v
-    const bool in_map = range <= (uint32_t)MAP_BITS && d <= (uint32_t)SLOTS;
-    const bool in_table = !in_map && 2u * d <= (uint32_t)SLOTS;
+    const bool in_map = range <= min((uint32_t)MAP_BITS, a.map_ranks) && d <= (uint32_t)SLOTS;
+    const bool in_table = !in_map && d <= min((uint32_t)SLOTS / 2u, a.table_row);
     uint32_t slots = 64;
     while (slots < 4u * d && slots < (uint32_t)SLOTS) slots <<= 1;
     if (in_map) {
@@ -608,7 +617,7 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
       if (lane == 0) j = atomicAdd(&s_batch, 32u);
       j = __shfl_sync(FULL_MASK, j, 0);
       if (j >= k) break;
-      const uint2 r = j + lane < k ? __ldcs(a.rec + (in - in0) + j + lane) : make_uint2(0, 0);
+      const uint2 r = j + lane < k ? in_edge(a, in - in0 + j + lane) : make_uint2(0, 0);
       if (in_map)
         count_tails<true>(a, BitRow{sm.map.bits, sm.map.before, v + 1u}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
       else if (in_table)
@@ -633,81 +642,110 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
 constexpr int MID_THREADS = 256, MID_SLOTS = 2048, MID_BITS = 1 << 16;    // rows up to 1024
 constexpr int BIG_THREADS = 512, BIG_SLOTS = 16384, BIG_BITS = 1 << 19;   // rows beyond (table up to 8192)
 
-// CTAs of a kernel that the current device's SMs hold, asked for once a device.
-class CtasPerSm {
- public:
-  template <typename F>
-  int operator()(F* f, int threads, size_t smem) {
-    int dev = -1, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) dev = 0;
-    if ((n = n_[dev].load(std::memory_order_relaxed)) > 0) return n;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, smem) != cudaSuccess) {
-      cudaGetLastError();
-      return 1;
-    }
-    n = std::max(n, 1);
-    n_[dev].store(n, std::memory_order_relaxed);
-    return n;
-  }
-
- private:
-  std::atomic<int> n_[MAX_DEVICES] = {};
-};
-
-wedge_status not_symmetric() { return fail(WEDGE_EINVAL, "wedge_exact: the graph's CSR is not symmetric"); }
-
 unsigned blocks_for(int64_t items) { return (unsigned)((items + EX_THREADS - 1) / EX_THREADS); }
 
+// What the neighbours of higher rank say before the edges are looked at again: the
+// digit histograms of the sort by u, and whether any rank has neighbours on both
+// sides (any[0]) and any two of higher rank (any[1]): without both there is no tail to
+// look up.
+__global__ __launch_bounds__(EX_THREADS) void k_row_sums(const int32_t* __restrict__ lower,
+                                                         const int32_t* __restrict__ higher, int32_t n, int passes,
+                                                         const unsigned long long* __restrict__ down, int64_t m,
+                                                         unsigned long long* __restrict__ hist,
+                                                         uint32_t* __restrict__ any) {
+  __shared__ uint32_t sh[DIGIT_COUNTS];
+  if (*down != (unsigned long long)m) return;  // (no counts: see above)
+  for (int i = threadIdx.x; i < DIGIT_COUNTS; i += EX_THREADS) sh[i] = 0;
+  __syncthreads();
+  bool both = false, two = false;
+  const int64_t stride = (int64_t)gridDim.x * EX_THREADS;
+  for (int64_t r = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x; r < n; r += stride) {
+    const int32_t h = __ldg(higher + r);
+    if (h == 0) continue;
+    both = both || __ldg(lower + r) > 0;
+    two = two || h > 1;
+    count_digits(sh, passes, (uint32_t)r, (uint32_t)h);
+  }
+  both = __syncthreads_or(both);
+  two = __syncthreads_or(two);
+  if (threadIdx.x == 0 && both) any[0] = 1u;
+  if (threadIdx.x == 0 && two) any[1] = 1u;
+  add_counts(sh, passes, hist);
+}
+
+// For a graph of this many entries the host waits for `any` (while the offsets
+// are scanned) before its edges are looked at again: 20 M edges between 1,000 and
+// 20,000 vertices 1,108 -> 327 us, 2 M between 20 and 100,000 364 -> 177.
+constexpr int64_t ASK_ENTRIES = int64_t(1) << 20;
+
+// A few words read back while later work runs.
+struct ReadBack {
+  cudaEvent_t done = nullptr;
+  uint32_t* words = nullptr;
+  static constexpr size_t BYTES = 64;
+  ~ReadBack() {
+    if (done) {
+      cudaEventSynchronize(done);  // the copy is no longer under way
+      cudaEventDestroy(done);
+    }
+    pinned_free(words, BYTES);
+  }
+  cudaError_t start(const uint32_t* from, size_t n, cudaStream_t s) {
+    words = static_cast<uint32_t*>(pinned_alloc(BYTES));
+    if (!words) return cudaErrorMemoryAllocation;
+    cudaError_t e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(words, from, n * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaEventRecord(done, s);
+    return e;
+  }
+  cudaError_t wait() { return cudaEventSynchronize(done); }
+};
+
+unsigned some_blocks(int64_t items) {
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + EX_THREADS - 1) / EX_THREADS, (int64_t)sm_count() * 8));
+}
+
 }  // namespace
-}  // namespace wedge
 
-using namespace wedge;
-
-extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, uint64_t* t_i, wedge_stream stream,
-                                    wedge_exact_counts* out) {
-  clear_error();
-  if (!g || !b || !out) return fail(WEDGE_EINVAL, "wedge_exact: NULL argument");
-  if (b->graph_uid != g->uid) return fail(WEDGE_EINVAL, "wedge_exact: bins were built from another graph");
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned long long* t_i, cudaStream_t s,
+                         const ExactLimits& lim, unsigned long long* pbq_out) {
   const wedge_bins_info& inf = b->info;
-  memset(out, 0, sizeof(*out));
-  out->n_bins = inf.n_bins;
-  out->p_total = inf.p_total;
-  for (uint32_t k = 0; k < inf.n_bins; ++k) out->p_b[k] = inf.p_b[k];
   const int32_t n = g->n;
   const int64_t n_adj = g->n_adj;
-  if (t_i) WEDGE_CUDA_TRY(cudaMemsetAsync(t_i, 0, (size_t)n * sizeof(uint64_t), s), "wedge_exact");
-  if (n_adj == 0) {
-    for (uint32_t k = 0; k < inf.n_bins; ++k) out->pbq[k][0] = inf.p_b[k];
-    return WEDGE_OK;
-  }
   const int64_t m = n_adj / 2;
   if (n_adj / (EX_WARPS * 32 * OR_STEPS) >= (int64_t)INT32_MAX) return fail(WEDGE_EINVAL, "wedge_exact: graph too large");
 
+  // edges are taken in groups of at most `cap`
+  const int64_t cap = std::max<int64_t>(lim.group_edges, g->max_degree);
+  const bool grouped = m > cap, few = n <= FEW_VERTICES;
+  const int64_t most = std::min(m, cap);
+  const size_t n_keys = (size_t)(few ? most : std::max<int64_t>(most, n));
+  const uint32_t nb = inf.n_bins;
+  const size_t n_cnt = (size_t)nb * 4;
+  // ranks, vertices by rank, per rank: lower and higher neighbours, entries taken; with groups also row entries, run
+  // ends; then a bit per adjacency entry
+  const size_t n_words = (grouped ? 7 : 5) * (size_t)n + (size_t)((n_adj + 31) / 32);
+
+  // control words (error bits, warp ticket, 2 unit counts, 2 CTA tickets, any[2]; entries down), pbq [nb*4], the
+  // bins' first ranks
+  unsigned long long* cnt = nullptr;
+  int32_t* words = nullptr;
+  int64_t* offs = nullptr;  // in-list, then row offsets by rank, one scan (2n + 1)
   uint64_t* keys = nullptr;
   uint64_t* alt = nullptr;
-  void* scratch = nullptr;
-  int32_t* rank = nullptr;     // ranks, then vertices by rank (2n)
-  int32_t* counts = nullptr;   // per rank: lower and higher neighbours, entries taken, row entries, run ends (5n)
-  int64_t* offs = nullptr;     // in-list, then row offsets by rank (2(n + 1))
-  uint32_t* rows = nullptr;
-  uint32_t* v_of = nullptr;
-  uint2* rec = nullptr;
+  char* scratch = nullptr;   // of a sort, then of the scan
+  uint32_t* rows = nullptr;  // m, and v and u by place of a group's edges
   uint2* units = nullptr;
-  // control words (error bits, warp ticket, 2 unit counts, 2 CTA tickets), pbq [nb*4], the bins' first ranks
-  unsigned long long* cnt = nullptr;
+  ReadBack any;
   auto done = [&](wedge_status st) {
+    dfree(cnt, s);
+    dfree(words, s);
+    dfree(offs, s);
     dfree(keys, s);
     dfree(alt, s);
     dfree(scratch, s);
-    dfree(rank, s);
-    dfree(counts, s);
-    dfree(offs, s);
     dfree(rows, s);
-    dfree(v_of, s);
-    dfree(rec, s);
     dfree(units, s);
-    dfree(cnt, s);
     return st;
   };
 #define EXACT_TRY(expr)                                                        \
@@ -721,13 +759,48 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
     if (st__ != WEDGE_OK) return done(st__);               \
   } while (0)
 
-  // control words and histogram, then the bins as ranges of ranks (bin_lo, n)
-  const uint32_t nb = inf.n_bins;
-  const size_t n_cnt = (size_t)nb * 4;
-  EXACT_DO(dalloc_n(&cnt, 4 + n_cnt + nb / 2 + 1, s, "wedge_exact"));
-  EXACT_TRY(cudaMemsetAsync(cnt, 0, (4 + n_cnt) * sizeof(unsigned long long), s));
+  const size_t sort_bytes = std::max(sort_scratch_bytes((int64_t)n_keys, (int)g->id_bits),
+                                     few ? 0 : sort_scratch_bytes(n, 31));
+  EXACT_DO(dalloc_n(&cnt, 5 + n_cnt + nb / 2 + 1, s, "wedge_exact"));
+  EXACT_DO(dalloc_n(&words, n_words, s, "wedge_exact: ranks and counts"));
+  EXACT_DO(dalloc_n(&keys, n_keys, s, "wedge_exact: edges"));
+  EXACT_DO(dalloc_n(&alt, n_keys, s, "wedge_exact: edges"));
+  EXACT_DO(dalloc(reinterpret_cast<void**>(&scratch), sort_bytes + scan_scratch_bytes(2 * (int64_t)n), s, "wedge_exact"));
+  const uint64_t max_units = (uint64_t)most / UNIT_IN + (uint64_t)most / WARP_IN + (uint64_t)m / WARP_ROW + 64;
+  if (most > (int64_t)UINT32_MAX || max_units > UINT32_MAX)
+    return done(fail(WEDGE_EINVAL, "wedge_exact: graph too large"));
+  EXACT_TRY(cudaMemsetAsync(cnt, 0, (5 + n_cnt) * sizeof(unsigned long long), s));
   uint32_t* ctl = reinterpret_cast<uint32_t*>(cnt);
-  unsigned long long* pbq = cnt + 4;
+  unsigned long long* down = cnt + 4;
+  unsigned long long* pbq = cnt + 5;
+  int32_t* rank = words;
+  int32_t* order = rank + n;
+  int32_t* lower = order + n;
+  int32_t* higher = lower + n;
+  int32_t* taken = higher + n;  // of a vertex's in-list
+  uint32_t* kept = reinterpret_cast<uint32_t*>(taken + n);
+  uint32_t* fill = kept + (n_adj + 31) / 32;  // entries per row so far
+  uint32_t* run_end = fill + n;
+  void* scan_scratch = scratch + sort_bytes;
+
+  // 1. ranks (launched before what comes later is allocated)
+  uint64_t* sorted = nullptr;
+  if (few) {
+    EXACT_DO(launch("exact_ranks", s, [&] {
+      k_ranks_few<<<(unsigned)((n + 31) / 32), EX_THREADS, 0, s>>>(g->deg, n, order, rank);
+    }));
+  } else {
+    int deg_bits = 1;
+    while (deg_bits < 31 && (g->max_degree >> deg_bits) != 0) ++deg_bits;
+    EXACT_DO(sort_clear(scratch, n, s));
+    EXACT_DO(launch("exact_ranks", s, [&] {
+      k_degree_keys<<<some_blocks(n), EX_THREADS, 0, s>>>(g->deg, n, (deg_bits + 7) / 8, keys, sort_hist_area(scratch));
+    }));
+    EXACT_DO(radix_sort_u64(keys, alt, n, deg_bits, scratch, ctl, s, &sorted, SortScratch::cleared, 32));
+    EXACT_DO(launch("exact_ranks", s, [&] { k_ranks<<<blocks_for(n), EX_THREADS, 0, s>>>(sorted, n, order, rank); }));
+  }
+
+  // the bins as ranges of ranks (bin_lo, n)
   std::vector<uint32_t> bin_lo(nb + 1, 0);  // bin 0: degree 0
   uint64_t below = (uint64_t)n;
   for (uint32_t k = 0; k < nb; ++k) below -= inf.n_b[k];
@@ -739,42 +812,16 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
   uint32_t* d_bin_lo = reinterpret_cast<uint32_t*>(pbq + n_cnt);
   EXACT_TRY(cudaMemcpyAsync(d_bin_lo, bin_lo.data(), (nb + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
 
-  // 1. ranks
-  EXACT_DO(dalloc_n(&rank, 2 * (size_t)n, s, "wedge_exact: ranks"));
-  int32_t* order = rank + n;
-  uint64_t* sorted = nullptr;
-  if (n <= FEW_VERTICES) {
-    EXACT_DO(launch("exact_ranks", s, [&] {
-      k_ranks_few<<<(unsigned)((n + 31) / 32), EX_THREADS, 0, s>>>(g->deg, n, order, rank);
-    }));
-  } else {
-    int deg_bits = 1;
-    while (deg_bits < 31 && (g->max_degree >> deg_bits) != 0) ++deg_bits;
-    EXACT_DO(dalloc_n(&keys, (size_t)n, s, "wedge_exact: ranks"));
-    EXACT_DO(dalloc_n(&alt, (size_t)n, s, "wedge_exact: ranks"));
-    EXACT_DO(dalloc(&scratch, sort_scratch_bytes(n, deg_bits), s, "wedge_exact: ranks"));
-    EXACT_DO(launch("exact_ranks", s, [&] { k_degree_keys<<<blocks_for(n), EX_THREADS, 0, s>>>(g->deg, n, keys); }));
-    EXACT_DO(radix_sort_u64(keys, alt, n, deg_bits, scratch, ctl, s, &sorted, SortScratch::unused, 32));
-    EXACT_DO(launch("exact_ranks", s, [&] { k_ranks<<<blocks_for(n), EX_THREADS, 0, s>>>(sorted, n, order, rank); }));
-    dfree(keys, s);
-    dfree(alt, s);
-    dfree(scratch, s);
-    keys = alt = nullptr;
-    scratch = nullptr;
-  }
-
   // 2. neighbours of lower and higher rank, in-list and row offsets
-  EXACT_DO(dalloc_n(&counts, 5 * (size_t)n, s, "wedge_exact: counts"));
-  EXACT_DO(dalloc_n(&offs, 2 * ((size_t)n + 1), s, "wedge_exact: offsets"));
-  EXACT_DO(dalloc(&scratch, scan_scratch_bytes(n), s, "wedge_exact"));
-  int32_t* lower = counts;
-  int32_t* higher = counts + n;
-  int32_t* taken = counts + 2 * (size_t)n;  // of a vertex's in-list
-  uint32_t* fill = reinterpret_cast<uint32_t*>(counts + 3 * (size_t)n);  // entries per row so far
-  uint32_t* run_end = reinterpret_cast<uint32_t*>(counts + 4 * (size_t)n);
+  EXACT_DO(dalloc_n(&offs, 2 * (size_t)n + 1, s, "wedge_exact: offsets"));
+  EXACT_DO(dalloc_n(&rows, (size_t)m + 2 * (size_t)most, s, "wedge_exact: rows"));
+  EXACT_DO(dalloc_n(&units, (size_t)max_units, s, "wedge_exact: units"));
   int64_t* in_off = offs;
-  int64_t* row_off = offs + (n + 1);
-  EXACT_TRY(cudaMemsetAsync(counts, 0, 4 * (size_t)n * sizeof(int32_t), s));
+  int64_t* row_off = offs + n;  // (row_off[0] = in_off[n] = m)
+  uint32_t* v_of = rows + m;
+  uint32_t* u_of = v_of + most;
+  EXACT_TRY(cudaMemsetAsync(lower, 0, 3 * (size_t)n * sizeof(int32_t), s));
+  if (grouped) EXACT_TRY(cudaMemsetAsync(fill, 0, (size_t)n * sizeof(int32_t), s));
   // a warp takes fewer entries where there are too few for all warps
   const int steps = (int)std::max<int64_t>(1, std::min<int64_t>(OR_STEPS, n_adj / ((int64_t)sm_count() * 64 * 32)));
   const int64_t tile = (int64_t)EX_WARPS * 32 * steps;
@@ -788,11 +835,29 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
   oa.steps = steps;
   oa.lower = lower;
   oa.higher = higher;
+  oa.kept = kept;
+  oa.down = down;
   EXACT_DO(launch("exact_orient", s, [&] { k_orient<false><<<tiles, EX_THREADS, 0, s>>>(oa); }));
-  EXACT_DO(scan_i32_to_i64(higher, row_off, n, row_off + n, nullptr, scratch, ctl, s));
-  EXACT_DO(scan_counts_to_i64(lower, in_off, n, in_off + n, scratch, ctl, s, "scan_in_counts"));
-  dfree(scratch, s);
-  scratch = nullptr;
+  const int key_bits = (int)g->id_bits;
+  if (!grouped) {
+    EXACT_DO(sort_clear(scratch, m, s));
+    EXACT_DO(launch("exact_row_sums", s, [&] {
+      k_row_sums<<<some_blocks(n), EX_THREADS, 0, s>>>(lower, higher, n, (key_bits + 7) / 8, down, m,
+                                                       sort_hist_area(scratch), ctl + 6);
+    }));
+  }
+  const bool ask = !grouped && n_adj >= ASK_ENTRIES;
+  if (ask) EXACT_TRY(any.start(ctl + 6, 4, s));
+  EXACT_DO(scan_i32_to_i64(lower, offs, 2 * (int64_t)n, offs + 2 * (size_t)n, nullptr, scan_scratch, ctl, s));
+  if (ask) {
+    EXACT_TRY(any.wait());
+    const bool half = any.words[2] == (uint32_t)m && any.words[3] == (uint32_t)(m >> 32);
+    if (half && (!any.words[0] || !any.words[1])) {
+      std::fill(pbq_out, pbq_out + n_cnt, 0ULL);
+      EXACT_TRY(cudaStreamSynchronize(s));
+      return done(WEDGE_OK);
+    }
+  }
   oa.lower = taken;
   oa.m = m;
 
@@ -803,13 +868,10 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
       return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
     };
     std::vector<std::pair<int32_t, int64_t>> cut{{n, m}};  // ends of the groups, from the top: rank, in_off there
-    const int64_t cap = std::max<int64_t>(GROUP_EDGES, g->max_degree);
-    int64_t largest = m;
-    if (m > cap) {
+    if (grouped) {
       int64_t all = 0;
       EXACT_TRY(in_at(n, &all));
-      if (all != m) return done(not_symmetric());
-      largest = 0;
+      if (all != m) return done(exact_not_symmetric());
       while (cut.back().second > 0) {
         const int64_t top = cut.back().second;
         int32_t lo = 0, hi = cut.back().first - 1;  // least rank whose group [rank, end) is at most cap
@@ -820,22 +882,11 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
           if (top - at <= cap) hi = mid; else lo = mid + 1;
         }
         EXACT_TRY(in_at(lo, &at));
-        largest = std::max(largest, top - at);
         cut.push_back({lo, at});
       }
     } else {
       cut.push_back({0, 0});
     }
-    const uint64_t max_units = (uint64_t)largest / UNIT_IN + (uint64_t)largest / WARP_IN + (uint64_t)m / WARP_ROW + 64;
-    if (largest > (int64_t)UINT32_MAX || max_units > UINT32_MAX)
-      return done(fail(WEDGE_EINVAL, "wedge_exact: graph too large"));
-    const int key_bits = (int)g->id_bits;
-    EXACT_DO(dalloc_n(&keys, (size_t)largest, s, "wedge_exact: edges"));
-    EXACT_DO(dalloc_n(&alt, (size_t)largest, s, "wedge_exact: edges"));
-    EXACT_DO(dalloc(&scratch, sort_scratch_bytes(largest, key_bits), s, "wedge_exact: edges"));
-    EXACT_DO(dalloc_n(&rows, (size_t)m, s, "wedge_exact: rows"));
-    EXACT_DO(dalloc_n(&v_of, (size_t)largest, s, "wedge_exact: edges"));
-    EXACT_DO(dalloc_n(&units, (size_t)max_units, s, "wedge_exact: units"));
     constexpr auto mid_kernel = k_tri_hash_cta<MID_THREADS, MID_SLOTS, MID_BITS>;
     constexpr auto big_kernel = k_tri_hash_cta<BIG_THREADS, BIG_SLOTS, BIG_BITS>;
     constexpr size_t mid_smem = sizeof(CtaSmem<MID_THREADS, MID_SLOTS, MID_BITS>);
@@ -847,6 +898,7 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
     const int mid_ctas = mid_occupancy(mid_kernel, MID_THREADS, mid_smem);
     const int big_ctas = big_occupancy(big_kernel, BIG_THREADS, big_smem);
     const int sms = sm_count();
+    const int64_t longest = longest_row(inf, g->max_degree);
     for (size_t gi = 0; gi + 1 < cut.size(); ++gi) {
       const int32_t r1 = cut[gi].first, r0 = cut[gi + 1].first;
       const int64_t edges = cut[gi].second - cut[gi + 1].second;
@@ -856,24 +908,27 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
       oa.r1 = r1;
       oa.keys = keys;
       oa.v_of = v_of;
+      oa.u_of = u_of;
       EXACT_DO(launch("exact_edges", s, [&] { k_orient<true><<<tiles, EX_THREADS, 0, s>>>(oa); }));
-      EXACT_DO(radix_sort_u64(keys, alt, edges, key_bits, scratch, ctl, s, &sorted, SortScratch::unused, 32));
-      rec = reinterpret_cast<uint2*>(sorted == keys ? alt : keys);  // the sort's other buffer
+      EXACT_DO(radix_sort_u64(keys, alt, edges, key_bits, scratch, ctl, s, &sorted,
+                              grouped ? SortScratch::unused : SortScratch::cleared, 32));
+      uint32_t* tail_of = reinterpret_cast<uint32_t*>(sorted == keys ? alt : keys);  // the sort's other buffer
       EXACT_DO(launch("exact_rows", s, [&] {
         const unsigned blocks = blocks_for(edges);
         if (edges == m) {
-          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, in_off, v_of, row_off, run_end, fill, rows, rec);
+          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of);
         } else {
           k_run_ends<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end);
-          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, in_off, v_of, row_off, run_end, fill, rows, rec);
+          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of);
           k_run_add<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end, fill);
         }
       }));
       CountArgs ca{};
+      ca.in_off = in_off;
       ca.row_off = row_off;
       ca.rows = rows;
-      ca.in_off = in_off;
-      ca.rec = rec;
+      ca.u_of = u_of;
+      ca.tail_of = tail_of;
       ca.order = order;
       ca.bin_lo = d_bin_lo;
       ca.nb = nb;
@@ -882,47 +937,147 @@ extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, u
       ca.r0 = r0;
       ca.r1 = r1;
       ca.pbq = pbq;
-      ca.t_i = reinterpret_cast<unsigned long long*>(t_i);
+      ca.t_i = t_i;
+      ca.down = down;
       ca.err = ctl;
       ca.next = ctl + 1;
+      ca.map_ranks = lim.map_ranks;
+      ca.table_row = lim.table_row;
       ca.units = units;
       ca.max_units = (uint32_t)max_units;
       ca.n_units = ctl + 2;
-      rec = nullptr;
-      // few vertices to a ticket where there are few for each warp
-      const int64_t warps = (int64_t)sms * warp_ctas * EX_WARPS;
-      ca.grab = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(GRAB, (r1 - r0) / (4 * warps)));
+      ca.grab = vertices_per_ticket(r1 - r0, (int64_t)sms * warp_ctas * EX_WARPS, GRAB);
       if (gi > 0) EXACT_TRY(cudaMemsetAsync(ctl + 1, 0, 5 * sizeof(uint32_t), s));
       EXACT_DO(launch("exact_hash_warp", s, [&] { k_tri_hash_warp<<<sms * warp_ctas, EX_THREADS, 0, s>>>(ca); }));
-      // (their work lists are on the device; a kernel without work ends at once)
-      EXACT_DO(launch("exact_hash_cta", s, [&] {
-        mid_kernel<<<sms * mid_ctas, MID_THREADS, mid_smem, s>>>(ca, units, 1, ctl + 2, ctl + 4);
-      }));
-      if (g->max_degree > MID_ROW)
+      // (their work lists are on the device; not launched where nothing can be in them)
+      if (g->max_degree > WARP_IN)
+        EXACT_DO(launch("exact_hash_cta", s, [&] {
+          mid_kernel<<<sms * mid_ctas, MID_THREADS, mid_smem, s>>>(ca, units, 1, ctl + 2, ctl + 4);
+        }));
+      if (longest > MID_ROW)
         EXACT_DO(launch("exact_hash_cta_long", s, [&] {
           big_kernel<<<sms * big_ctas, BIG_THREADS, big_smem, s>>>(ca, units + (max_units - 1), -1, ctl + 3, ctl + 5);
         }));
     }
   }
-  std::vector<unsigned long long> h(n_cnt);
   uint32_t herr = 0;
-  EXACT_TRY(cudaMemcpyAsync(h.data(), pbq, n_cnt * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  EXACT_TRY(cudaMemcpyAsync(pbq_out, pbq, n_cnt * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   EXACT_TRY(cudaMemcpyAsync(&herr, ctl, sizeof(herr), cudaMemcpyDeviceToHost, s));
   EXACT_TRY(cudaStreamSynchronize(s));
 #undef EXACT_TRY
 #undef EXACT_DO
   if (herr & DERR_TIMEOUT) return done(fail(WEDGE_ETIMEOUT, "wedge_exact: a look-back wait gave up"));
-  if (herr & DERR_BAD_ID) return done(not_symmetric());
+  if (herr & DERR_BAD_ID) return done(exact_not_symmetric());
+  return done(WEDGE_OK);
+}
+
+namespace {
+
+// Entries of whole rows N+(v) that exact_rows would stream per edge (u, v), by the
+// bins: in a bin of mean degree d (of its wedges), a vertex has about d / 2 edges from
+// below and as many to above, but no more than there are vertices in its bin and
+// those after.
+double streamed_per_edge(const wedge_bins_info& inf, int64_t m) {
+  double entries = 0, above = -1;
+  for (uint32_t k = inf.n_bins; k-- > 1;) {
+    const double n_b = (double)inf.n_b[k];
+    if (n_b == 0) continue;
+    above += n_b;
+    const double d = k == 1 ? 1.0 : 0.5 * (1.0 + std::sqrt(1.0 + 8.0 * (double)inf.p_b[k] / n_b));
+    entries += n_b * d * std::min(d, above) / 4.0;
+  }
+  return entries / (double)m;
+}
+
+// Whether whole rows are streamed (exact_rows.cu) and not tails. Whole rows need no
+// ranks and no sort of the edges, about 80 ps an edge and 50 us, but twice
+// the entries where degrees are alike and up to four times where they are not, and
+// a found triangle costs more. Both forms, us (16.8 M edges unless stated):
+//   next to nothing to stream (R <= 2.25 entries an edge): path of 4.2 M 390, 1,430; star
+//     1,450, 4,450; grid of 9 M vertices 4,850, 4,840; ring of 1 M with 2 neighbours a side 760, 930;
+//   few edges: 0.26 M, power law 3.0 (R = 5) 200, 257, ring (R = 8) 255, 266; 0.52 M, ring
+//     (R = 8) 397, 370; uniform (R = 4.5) of 1 M 360, 364; all of 16.8 M 3,990, 3,010;
+//   many, degrees alike, next to no triangles: uniform, R = 16 2,190, 2,370; R = 32 2,770, 3,105
+//     (67 M 12,140, 15,240: rows, lists and tails are past L2); R = 8 2,630, 2,515. With triangles, a
+//     ring of 16 neighbours a side, 13,380, 5,450: so these are asked first, 2,048
+//     wedges for 40 us (the forms meet at about one closed in sixty).
+bool takes_rows(const wedge_graph* g, const wedge_bins* b, wedge_stream stream) {
+  const wedge_bins_info& inf = b->info;
+  const int64_t m = g->n_adj / 2;
+  const double per_edge = streamed_per_edge(inf, m);
+  if (per_edge <= 2.25 || (per_edge <= 9.0 && m <= (1 << 19))) return true;
+  const double pairs_per_edge = (double)inf.p_total / (double)m;  // twice R where degrees are alike
+  if (m < (1 << 23) || per_edge < 12.0 || pairs_per_edge > 2.3 * per_edge) return false;
+  wedge_sample_params sp;
+  memset(&sp, 0, sizeof(sp));
+  sp.k_global = 2048;
+  sp.flags = WEDGE_FLAG_NO_BINS;
+  wedge_counts c;
+  if (wedge_sample(g, b, &sp, stream, &c) != WEDGE_OK) {
+    clear_error();
+    return false;
+  }
+  return c.closed_global <= 20;
+}
+
+}  // namespace
+}  // namespace wedge
+
+using namespace wedge;
+
+// form: 0 by the rule, 1 tails, 2 whole rows.
+static wedge_status exact_counts(const wedge_graph* g, const wedge_bins* b, uint64_t* t_i, wedge_stream stream, int form,
+                                 const ExactLimits& lim, wedge_exact_counts* out) {
+  clear_error();
+  if (!g || !b || !out) return fail(WEDGE_EINVAL, "wedge_exact: NULL argument");
+  if (b->graph_uid != g->uid) return fail(WEDGE_EINVAL, "wedge_exact: bins were built from another graph");
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const wedge_bins_info& inf = b->info;
+  memset(out, 0, sizeof(*out));
+  out->n_bins = inf.n_bins;
+  out->p_total = inf.p_total;
+  for (uint32_t k = 0; k < inf.n_bins; ++k) out->p_b[k] = inf.p_b[k];
+  if (t_i) WEDGE_CUDA_TRY(cudaMemsetAsync(t_i, 0, (size_t)g->n * sizeof(uint64_t), s), "wedge_exact");
+  if (g->n_adj == 0) {
+    for (uint32_t k = 0; k < inf.n_bins; ++k) out->pbq[k][0] = inf.p_b[k];
+    return WEDGE_OK;
+  }
+  unsigned long long pbq[WEDGE_MAX_BINS * 4];
+  unsigned long long* ti = reinterpret_cast<unsigned long long*>(t_i);
+  const bool rows = form == 0 ? takes_rows(g, b, stream) : form == 2;
+  wedge_status st = rows ? exact_rows(g, b, ti, s, pbq) : exact_tails(g, b, ti, s, lim, pbq);
+  if (st == WEDGE_ENOMEM && !rows && form == 0) {  // the other form needs less
+    clear_error();
+    st = exact_rows(g, b, ti, s, pbq);
+  }
+  if (st != WEDGE_OK) return st;
   uint64_t closed = 0;
   for (uint32_t k = 0; k < inf.n_bins; ++k) {
     uint64_t sum = 0;
     for (int q = 1; q <= 3; ++q) {
-      out->pbq[k][q] = h[(size_t)k * 4 + q];
+      out->pbq[k][q] = pbq[(size_t)k * 4 + q];
       sum += out->pbq[k][q];
     }
     out->pbq[k][0] = inf.p_b[k] - sum;
     closed += sum;
   }
   out->triangles = closed / 3;
-  return done(WEDGE_OK);
+  return WEDGE_OK;
+}
+
+extern "C" wedge_status wedge_exact(const wedge_graph* g, const wedge_bins* b, uint64_t* t_i, wedge_stream stream,
+                                    wedge_exact_counts* out) {
+  return exact_counts(g, b, t_i, stream, 0, ExactLimits(), out);
+}
+
+extern "C" wedge_status wedge_test_exact(const wedge_graph* g, const wedge_bins* b, uint64_t* t_i, wedge_stream stream,
+                                         int form, int64_t group_edges, uint32_t map_ranks, uint32_t table_row,
+                                         wedge_exact_counts* out) {
+  clear_error();
+  if (form < 0 || form > 2 || group_edges < 1) return fail(WEDGE_EINVAL, "wedge_test_exact: form or group out of range");
+  ExactLimits lim;
+  lim.group_edges = std::min(group_edges, lim.group_edges);
+  lim.map_ranks = map_ranks;
+  lim.table_row = table_row;
+  return exact_counts(g, b, t_i, stream, form, lim, out);
 }
