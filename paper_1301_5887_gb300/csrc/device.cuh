@@ -34,6 +34,13 @@ __device__ __forceinline__ bool in_bounds(uint64_t i, uint64_t n, uint32_t* err)
 #endif
 }
 
+// Debug-build read of a[i] for i < n; an index outside reads a[0] instead
+// (n >= 1 wherever a gather happens) after recording DERR_BOUNDS.
+template <typename T>
+__device__ __forceinline__ T checked_ldg(const T* a, int64_t i, int64_t n, uint32_t* err) {
+  return __ldg(a + (in_bounds((uint64_t)i, (uint64_t)n, err) ? i : 0));
+}
+
 // A look-back wait polls at most this many times (with nanosleep back-off,
 // about a second) before it records DERR_TIMEOUT and stops waiting.
 constexpr uint32_t SPIN_LIMIT = 1u << 22;

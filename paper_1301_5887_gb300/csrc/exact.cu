@@ -136,6 +136,8 @@ struct OrientArgs {
   uint32_t* v_of;         // EMIT: v by place
   uint32_t* u_of;         // EMIT: u by place
   int64_t m;              // EMIT: places in all in-lists
+  int64_t places;         // and room for a group's (checked by the debug build, as below)
+  uint32_t* err;
 };
 
 // Every adjacency entry (v, u) with rank(u) < rank(v): counted for both ends and
@@ -185,9 +187,11 @@ __global__ __launch_bounds__(EX_THREADS) void k_orient(OrientArgs a) {
       if (keep) {
         const uint64_t pos = (uint64_t)(__ldg(a.in_off + rx) - __ldg(a.in_off + a.r0)) + (uint32_t)at +
                              __popc(mine & lanemask_lt());
-        a.keys[pos] = ((uint64_t)(uint32_t)ry << 32) | pos;
-        a.v_of[pos] = (uint32_t)rx;
-        a.u_of[pos] = (uint32_t)ry;
+        if (in_bounds(pos, (uint64_t)a.places, a.err)) {
+          a.keys[pos] = ((uint64_t)(uint32_t)ry << 32) | pos;
+          a.v_of[pos] = (uint32_t)rx;
+          a.u_of[pos] = (uint32_t)ry;
+        }
       }
     }
   }
@@ -225,15 +229,19 @@ __global__ __launch_bounds__(EX_THREADS) void k_rows(const uint64_t* __restrict_
                                                      const int64_t* __restrict__ row_off,
                                                      const uint32_t* __restrict__ run_end,
                                                      const uint32_t* __restrict__ filled, uint32_t* __restrict__ rows,
-                                                     int64_t row_base, uint32_t* __restrict__ tail_of) {
+                                                     int64_t row_base, uint32_t* __restrict__ tail_of,
+                                                     uint32_t* err) {
   const int64_t i = (int64_t)blockIdx.x * EX_THREADS + threadIdx.x;
   if (i >= m || (WHOLE && *down != (unsigned long long)m)) return;
   const uint64_t key = __ldcs(keys + i);
   const uint32_t u = (uint32_t)(key >> 32), pos = (uint32_t)key;
+  if (!in_bounds(u, n, err)) return;
   const int64_t row_end = __ldg(row_off + u + 1);
   const uint32_t after = WHOLE ? (uint32_t)(row_end - 1 - row_base - i)
                                : __ldg(filled + u) + (__ldg(run_end + u) - 1u - (uint32_t)i);
-  rows[row_end - 1 - row_base - (int64_t)after] = __ldg(v_of + pos);
+  const int64_t at = row_end - 1 - row_base - (int64_t)after;
+  if (!in_bounds(pos, (uint64_t)m, err) || !in_bounds((uint64_t)at, (uint64_t)row_base, err)) return;
+  rows[at] = __ldg(v_of + pos);
   tail_of[pos] = after;
 }
 
@@ -250,6 +258,7 @@ struct CountArgs {
   uint32_t nb;
   uint32_t n;
   int64_t m;               // entries of rows
+  int64_t places;          // entries of u_of and tail_of (checked by the debug build)
   uint32_t grab;           // vertices a warp takes per ticket
   uint32_t map_ranks;      // most ranks of a bit map, and half the slots of a hash table, of the
   uint32_t table_row;      // CTA kernels (as they are sized, or less)
@@ -275,7 +284,9 @@ constexpr uint32_t GRAB = 8;         // vertices a warp takes per ticket at most
 __device__ __forceinline__ uint32_t slot_of(uint32_t w, uint32_t mask) { return (w * 0x9E3779B1u) >> 7 & mask; }
 
 __device__ __forceinline__ uint2 in_edge(const CountArgs& a, int64_t place) {
-  return make_uint2(__ldcs(a.u_of + place), __ldcs(a.tail_of + place));
+  if (!in_bounds((uint64_t)place, (uint64_t)a.places, a.err)) return make_uint2(0, 0);
+  const uint2 r = make_uint2(__ldcs(a.u_of + place), __ldcs(a.tail_of + place));
+  return in_bounds(r.x, a.n, a.err) ? r : make_uint2(0, 0);
 }
 
 // Insert key w (absent); the table has free slots (load <= 1/2).
@@ -314,7 +325,10 @@ struct BitRow {  // one bit per rank above v; the counter is w's place in the ro
   const uint32_t* bits;
   const uint16_t* before;  // row entries before the word's first
   uint32_t above;          // v + 1
+  uint32_t range;          // ranks of the map (checked by the debug build)
+  uint32_t* err;
   __device__ __forceinline__ bool find(uint32_t w, uint32_t& slot) const {
+    if (!in_bounds(w - above, range, err)) return false;
     const uint32_t i = w - above, word = bits[i >> 5], rest = word >> (i & 31u);
     if (!(rest & 1u)) return false;
     slot = before[i >> 5] + __popc(word) - __popc(rest);
@@ -395,7 +409,7 @@ __device__ __forceinline__ void count_tails(const CountArgs& a, const Row& nv, c
       const uint64_t first = __shfl_sync(FULL_MASK, my_first, l);
       const uint32_t end_u = __shfl_sync(FULL_MASK, my_end_u, l);
       if (t0 + lane < total) {
-        const uint32_t add = look(__ldg(a.rows + first + t), end_u);
+        const uint32_t add = look(checked_ldg(a.rows, (int64_t)(first + t), a.m, a.err), end_u);
         if (add) atomicAdd(seg + l, add);
       }
     }
@@ -408,7 +422,9 @@ __device__ __forceinline__ void count_tails(const CountArgs& a, const Row& nv, c
     for (; todo; todo &= todo - 1) {
       const int l = __ffs(todo) - 1;
       const uint32_t len = __shfl_sync(FULL_MASK, r.y, l), end_u = __shfl_sync(FULL_MASK, my_end_u, l);
-      const uint32_t* tail = a.rows + __shfl_sync(FULL_MASK, my_tail, l);
+      const uint64_t at = __shfl_sync(FULL_MASK, my_tail, l);
+      if (len && !in_bounds(at + len - 1, (uint64_t)a.m, a.err)) continue;  // (the whole warp)
+      const uint32_t* tail = a.rows + at;
       for (uint32_t k0 = 0; k0 < len; k0 += 30 * 32) {  // (sums of 30 x 32 fit their 10 bits)
         uint32_t mine = 0;
         const uint32_t k1 = min(len, k0 + 30 * 32);
@@ -600,6 +616,7 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
       __syncthreads();
       for (uint32_t i = tid; i < d; i += THREADS) {
         const uint32_t x = __ldg(row + i) - (v + 1u), y = i ? __ldg(row + i - 1) - (v + 1u) : ~0u;
+        if (!in_bounds(x, range, a.err)) continue;
         atomicOr(&sm.map.bits[x >> 5], 1u << (x & 31u));
         if ((x >> 5) != (y >> 5)) sm.map.before[x >> 5] = (uint16_t)i;
       }
@@ -619,7 +636,7 @@ __global__ __launch_bounds__(THREADS) void k_tri_hash_cta(CountArgs a, const uin
       if (j >= k) break;
       const uint2 r = j + lane < k ? in_edge(a, in - in0 + j + lane) : make_uint2(0, 0);
       if (in_map)
-        count_tails<true>(a, BitRow{sm.map.bits, sm.map.before, v + 1u}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
+        count_tails<true>(a, BitRow{sm.map.bits, sm.map.before, v + 1u, range, a.err}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
       else if (in_table)
         count_tails<true>(a, HashRow{sm.table, slots - 1}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
       else count_tails<false>(a, MemoryRow{row, d}, s_lo, s_hist, r, bv, sm.hits, s_seg[tid >> 5], cv, lane);
@@ -860,6 +877,8 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
   }
   oa.lower = taken;
   oa.m = m;
+  oa.places = most;
+  oa.err = ctl;
 
   // 3-4. groups of ranks, highest first
   {
@@ -916,10 +935,12 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
       EXACT_DO(launch("exact_rows", s, [&] {
         const unsigned blocks = blocks_for(edges);
         if (edges == m) {
-          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of);
+          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of,
+                                                          ctl);
         } else {
           k_run_ends<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end);
-          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of);
+          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of,
+                                                          ctl);
           k_run_add<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end, fill);
         }
       }));
@@ -928,6 +949,7 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
       ca.row_off = row_off;
       ca.rows = rows;
       ca.u_of = u_of;
+      ca.places = most;
       ca.tail_of = tail_of;
       ca.order = order;
       ca.bin_lo = d_bin_lo;
@@ -967,6 +989,7 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
 #undef EXACT_TRY
 #undef EXACT_DO
   if (herr & DERR_TIMEOUT) return done(fail(WEDGE_ETIMEOUT, "wedge_exact: a look-back wait gave up"));
+  if (herr & DERR_BOUNDS) return done(exact_out_of_bounds());
   if (herr & DERR_BAD_ID) return done(exact_not_symmetric());
   return done(WEDGE_OK);
 }

@@ -32,6 +32,10 @@ inline wedge_status exact_not_symmetric() {
   return fail(WEDGE_EINVAL, "wedge_exact: the graph's CSR is not symmetric");
 }
 
+inline wedge_status exact_out_of_bounds() {
+  return fail(WEDGE_ECUDA, "wedge_exact: an index outside its buffer (bounds-checked build)");
+}
+
 // The most neighbours of higher (degree, id) that a vertex can have, by the bins.
 inline int64_t longest_row(const wedge_bins_info& inf, int32_t max_degree) {
   int64_t longest = 0, above = -1;  // vertices of the bin and those after it, but for one

@@ -328,7 +328,7 @@ __global__ __launch_bounds__(TC_THREADS) void k_rows_warp(CountArgs a) {
           tv.bin = sm.vbin[wid][i];
           cur = i;
         }
-        const int32_t w = __ldg(a.adjp + sm.voff[wid][i] + (t - pre[i]));
+        const int32_t w = checked_ldg(a.adjp, sm.voff[wid][i] + (t - pre[i]), a.m, a.err);
         const int h = find_key(table, WARP_SLOTS - 1, w);
         if (h >= 0) count_triangle(tu, tv, hits, h, tbin[h]);
       }
@@ -460,7 +460,7 @@ __global__ __launch_bounds__(THREADS) void k_rows_cta(CountArgs a, const int32_t
               tv[r].vertex = wv[r];
               tv[r].bin = bin_of(bt, (uint64_t)__ldg(a.deg + wv[r]));
             }
-            w[r] = __ldg(a.adjp + wlo[r] + (t - pre[wi[r]]));
+            w[r] = checked_ldg(a.adjp, wlo[r] + (t - pre[wi[r]]), a.m, a.err);
           }
         }
 #pragma unroll
@@ -615,6 +615,7 @@ wedge_status exact_rows(const wedge_graph* g, const wedge_bins* b, unsigned long
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return done(cuda_fail(e, "wedge_exact"));
   if (herr & DERR_TIMEOUT) return done(fail(WEDGE_ETIMEOUT, "wedge_exact: a look-back wait gave up"));
+  if (herr & DERR_BOUNDS) return done(exact_out_of_bounds());
   if (herr & DERR_BAD_ID) return done(exact_not_symmetric());
   return done(WEDGE_OK);
 }

@@ -68,7 +68,7 @@ struct SampleArgs {
   unsigned long long* stats;   // [WEDGE_STAT_BINS][WEDGE_STAT_BINS]
   wedge_record* records;       // global stream records or nullptr
   bool whole_records;          // records are aligned to their size
-  int64_t n, n_adj, n_L;       // sizes for the bounds-checked debug build
+  int64_t n, n_adj, n_L, n_guide;  // sizes for the bounds-checked debug build
   uint32_t* err;
 };
 
@@ -107,7 +107,7 @@ __global__ __launch_bounds__(SAMPLE_THREADS) void k_sample(SampleArgs a) {
   __syncthreads();
   const StreamDesc desc = s_desc;
   const BinTable bt{s_lo, a.nb, a.pow2};
-  const GraphView gv{a.off, a.adj, a.L, a.W, a.guide, 1.0f / (float)a.n, a.n, a.n_adj, a.n_L, a.err};
+  const GraphView gv{a.off, a.adj, a.L, a.W, a.guide, 1.0f / (float)a.n, a.n, a.n_adj, a.n_L, a.n_guide, a.err};
   const bool global = desc.tag != 0;
   const GuideRange gr{s_gtab, global ? 2u : desc.bin, global ? a.nb : desc.bin + 1u};
   const uint64_t first = ((uint64_t)blockIdx.x - desc.tile_begin) * (uint32_t)(SAMPLE_THREADS * a.per_thread);
@@ -332,6 +332,7 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
   a.n = g->n;
   a.n_adj = g->n_adj;
   a.n_L = inf.n_wedge_vertices;
+  a.n_guide = (int64_t)guide_alloc(inf.n_wedge_vertices, inf.n_bins);
   a.err = reinterpret_cast<uint32_t*>(d_cnt + n_cnt - 1);
   st = launch("sample_closure", s, [&] { k_sample<<<(unsigned)tiles, SAMPLE_THREADS, 0, s>>>(a); });
   if (st != WEDGE_OK) return done(st);

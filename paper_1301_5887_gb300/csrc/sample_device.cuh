@@ -14,7 +14,7 @@
 namespace wedge {
 
 // One sampling stream: a bin of one graph (tag 0) or all of its wedges (tag 1).
-// n, n_adj, n_L and err are read only by the bounds-checked debug build
+// n, n_adj, n_L, n_guide and err are read only by the bounds-checked debug build
 // (err == nullptr: unchecked).
 struct GraphView {
   const int64_t* off;
@@ -26,15 +26,9 @@ struct GraphView {
   int64_t n = 0;
   int64_t n_adj = 0;
   int64_t n_L = 0;
+  int64_t n_guide = 0;
   uint32_t* err = nullptr;
 };
-
-// Debug-build read of a[i] for i < n; an index outside reads a[0] instead
-// (n >= 1 wherever a gather happens) after recording DERR_BOUNDS.
-template <typename T>
-__device__ __forceinline__ T checked_ldg(const T* a, int64_t i, int64_t n, uint32_t* err) {
-  return __ldg(a + (in_bounds((uint64_t)i, (uint64_t)n, err) ? i : 0));
-}
 
 // u / d, in 32 bits where both fit (the degrees of all but the largest hubs):
 // a 64-bit division is several times the instructions.
@@ -210,9 +204,9 @@ __device__ __forceinline__ void centre_cell(const GraphView& g, const GuideRange
     if (gr.tab[mid].wlo <= T) b = mid; else e = mid;
   }
   const GuideBin t = gr.tab[b];
-  const uint32_t* c = g.guide + t.at + ((T - t.wlo) >> t.shift);
-  lo = __ldg(c);
-  hi = (int64_t)__ldg(c + 1) + 1;
+  const int64_t c = (int64_t)(t.at + ((T - t.wlo) >> t.shift));
+  lo = checked_ldg(g.guide, c, g.n_guide, g.err);
+  hi = (int64_t)checked_ldg(g.guide, c + 1, g.n_guide, g.err) + 1;
 }
 
 // Centre and endpoints (no closure) for random words r of a stream of the bins
@@ -227,7 +221,7 @@ __device__ __forceinline__ Wedge draw_pair_thread(const GraphView& g, const Guid
   centre_cell(g, gr, T, lo, hi);
   while (hi - lo > 1) {
     const int64_t mid = lo + ((hi - lo) >> 1);
-    if (__ldg(g.W + mid) <= T) lo = mid; else hi = mid;
+    if (checked_ldg(g.W, mid, g.n_L + 1, g.err) <= T) lo = mid; else hi = mid;
   }
   w.v0 = checked_ldg(g.L, lo, g.n_L, g.err);
   const int64_t o0 = checked_ldg(g.off, w.v0, g.n + 1, g.err);
@@ -276,7 +270,7 @@ __device__ __forceinline__ void draw_wedge_thread2(const GraphView& g, const Gui
     const bool sa = ha - la > 1, sb = hb - lb > 1;
     const int64_t ma = sa ? la + ((ha - la) >> 1) : la;
     const int64_t mb = sb ? lb + ((hb - lb) >> 1) : lb;
-    const uint64_t xa = __ldg(g.W + ma), xb = __ldg(g.W + mb);
+    const uint64_t xa = checked_ldg(g.W, ma, g.n_L + 1, g.err), xb = checked_ldg(g.W, mb, g.n_L + 1, g.err);
     if (sa) {
       if (xa <= Ta) la = ma; else ha = ma;
     }
