@@ -865,7 +865,7 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
   }
   const bool ask = !grouped && n_adj >= ASK_ENTRIES;
   if (ask) EXACT_TRY(any.start(ctl + 6, 4, s));
-  EXACT_DO(scan_i32_to_i64(lower, offs, 2 * (int64_t)n, offs + 2 * (size_t)n, nullptr, scan_scratch, ctl, s));
+  EXACT_DO(scan_i32_to_i64(lower, offs, 2 * (int64_t)n, offs + 2 * (size_t)n, scan_scratch, ctl, s));
   if (ask) {
     EXACT_TRY(any.wait());
     const bool half = any.words[2] == (uint32_t)m && any.words[3] == (uint32_t)(m >> 32);

@@ -564,7 +564,7 @@ wedge_status exact_rows(const wedge_graph* g, const wedge_bins* b, unsigned long
   oa.dplus = dplus;
   st = launch("exact_orient", s, [&] { k_orient<<<(unsigned)tiles, OR_THREADS, 0, s>>>(oa); });
   if (st != WEDGE_OK) return done(st);
-  if ((st = scan_i32_to_i64(dplus, offp, n, offp + n, nullptr, scratch, ctl, s)) != WEDGE_OK) return done(st);
+  if ((st = scan_i32_to_i64(dplus, offp, n, offp + n, scratch, ctl, s)) != WEDGE_OK) return done(st);
 
   constexpr auto mid_kernel = k_rows_cta<MID_THREADS, MID_SLOTS>;
   constexpr auto big_kernel = k_rows_cta<BIG_THREADS, BIG_SLOTS>;

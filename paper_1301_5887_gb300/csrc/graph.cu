@@ -717,7 +717,7 @@ extern "C" wedge_status wedge_graph_build(const int32_t* src, const int32_t* dst
     // 4. forward offsets; transposed sort on the larger endpoint's bits, its
     //    last pass placing each backward entry u of row w at j + foff[w] (j
     //    its sorted position) and counting the backward entries per row
-    st = scan_i32_to_i64(bb.fdeg, bb.foff, n_vertices, bb.foff + n_vertices, nullptr,
+    st = scan_i32_to_i64(bb.fdeg, bb.foff, n_vertices, bb.foff + n_vertices,
                          static_cast<char*>(bb.scratch) + hist_bytes, bb.derr, s);
     if (st != WEDGE_OK) return bail(st);
     if (m_unique >= 2) {

@@ -130,12 +130,8 @@ wedge_status merge_two_runs(const uint64_t* in, uint64_t* out, int64_t p0, int64
 // Exclusive scans with decoupled look-back (scan.cu).
 size_t scan_scratch_bytes(int64_t n);
 // out[i] = sum in[0..i) for i < n; if total != nullptr, *total = sum of all.
-// If maxv != nullptr, atomicMax(maxv, max input) (inputs interpreted as int32).
-wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, int32_t* maxv, void* scratch,
-                             uint32_t* derr, cudaStream_t s);
-// The same under a name of its own.
-wedge_status scan_counts_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch,
-                                uint32_t* derr, cudaStream_t s, const char* name);
+wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch, uint32_t* derr,
+                             cudaStream_t s);
 // boff: exclusive scan of bdeg (n + 1); off = foff + boff (n + 1), deg = fdeg +
 // bdeg, *maxdeg raised to the largest; n >= 1.
 wedge_status scan_rows(const int32_t* fdeg, const int32_t* bdeg, const int64_t* foff, int64_t* boff, int64_t n,

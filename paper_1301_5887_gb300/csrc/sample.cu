@@ -39,10 +39,8 @@ constexpr int SAMPLE_PER_THREAD = 8;
 constexpr int SAMPLE_MIN_CTAS = 4;
 
 struct StreamDesc {
-  int64_t start;        // first index of the stream's vertices in L
-  int64_t len;          // number of vertices
   uint64_t p;           // wedges in the stream
-  uint64_t wbase;       // W[start]
+  uint64_t wbase;       // wedges before them (W at the bin's start)
   uint64_t k;           // samples to draw
   uint64_t first;       // first sample index
   uint64_t tile_begin;  // first CTA of this stream
@@ -247,11 +245,9 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
   std::vector<StreamDesc> streams;
   std::vector<int> stream_bin;
   uint64_t tiles = 0;
-  auto add = [&](int64_t start, int64_t len, uint64_t p, uint64_t k, uint32_t bin, uint32_t tag, uint64_t wbase) {
-    if (k == 0 || p == 0 || len == 0) return;
+  auto add = [&](uint64_t p, uint64_t k, uint32_t bin, uint32_t tag, uint64_t wbase) {
+    if (k == 0 || p == 0) return;
     StreamDesc d;
-    d.start = start;
-    d.len = len;
     d.p = p;
     d.wbase = wbase;
     d.k = k;
@@ -265,10 +261,10 @@ static wedge_status sample_streams(const wedge_graph* g, const wedge_bins* b, co
   uint64_t wacc = 0;
   for (uint32_t k = 2; k < inf.n_bins; ++k) {
     const uint64_t kb = !want_bins ? 0 : (sp->k_bin ? sp->k_bin[k] : k_bin);
-    add(inf.start[k], inf.start[k + 1] - inf.start[k], inf.p_b[k], kb, k, 0u, wacc);
+    add(inf.p_b[k], kb, k, 0u, wacc);
     wacc += inf.p_b[k];
   }
-  add(0, inf.n_wedge_vertices, inf.p_total, k_glob, 0u, 1u, 0ULL);
+  add(inf.p_total, k_glob, 0u, 1u, 0ULL);
   double budget = 0;
   for (const StreamDesc& d : streams) budget += (double)d.k;
   const double fills = budget / ((double)SAMPLE_THREADS * SAMPLE_MIN_CTAS * sm_count());

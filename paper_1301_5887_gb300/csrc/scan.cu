@@ -34,7 +34,7 @@ struct Pairs {
 template <typename Tin, typename Tout, bool CHECK = false>
 __global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restrict__ in, Tout* __restrict__ out,
                                                             int64_t n, uint64_t* status, uint32_t* tile_ctr,
-                                                            uint32_t* err, Tout* total, int32_t* maxv,
+                                                            uint32_t* err, Tout* total,
                                                             uint32_t spin_limit = SPIN_LIMIT,
                                                             int64_t prefetch_tiles = 0) {
   __shared__ Tout s_buf[SCAN_TILE + SCAN_TILE / 32];
@@ -55,7 +55,6 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restric
                    "r"((uint32_t)(SCAN_TILE * sizeof(Tin)))
                    : "memory");
   }
-  int32_t local_max = INT32_MIN;
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
     const int idx = i * SCAN_THREADS + tid;
@@ -64,7 +63,6 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restric
     if (g < n) {
       const Tin x = in[g];
       v = (Tout)x;
-      if (maxv) local_max = max(local_max, (int32_t)v);
       if (CHECK && v < (Tout)0) atomicOr(err, DERR_NEGATIVE);
     }
     s_buf[pad(idx)] = v;
@@ -85,11 +83,6 @@ __global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restric
     if (lane >= o) incl += y;
   }
   if (lane == 31) s_wsum[warp] = incl;
-  if (maxv) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) local_max = max(local_max, __shfl_xor_sync(FULL_MASK, local_max, o));
-    if (lane == 0 && local_max != INT32_MIN) atomicMax(maxv, local_max);
-  }
   __syncthreads();
   Tout wpre = 0, tile_total = 0;
 #pragma unroll
@@ -222,8 +215,8 @@ __global__ __launch_bounds__(SCAN_THREADS, 5) void k_scan_rows(const int32_t* __
 }
 
 template <typename Tin, typename Tout>
-wedge_status run_scan(const Tin* in, Tout* out, int64_t n, Tout* total, int32_t* maxv, void* scratch, uint32_t* derr,
-                      cudaStream_t s, const char* name) {
+wedge_status run_scan(const Tin* in, Tout* out, int64_t n, Tout* total, void* scratch, uint32_t* derr, cudaStream_t s,
+                      const char* name) {
   if (n <= 0) {
     if (total) WEDGE_CUDA_TRY(cudaMemsetAsync(total, 0, sizeof(Tout), s), name);
     return WEDGE_OK;
@@ -234,11 +227,12 @@ wedge_status run_scan(const Tin* in, Tout* out, int64_t n, Tout* total, int32_t*
   uint32_t* ctr = tiles > 1 ? static_cast<uint32_t*>(scratch) : nullptr;
   uint64_t* status = reinterpret_cast<uint64_t*>(static_cast<char*>(scratch) + 256);
   if (tiles > 1) WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, 256 + (size_t)tiles * sizeof(uint64_t), s), name);
-  // L2 prefetch about one wave of CTAs ahead (six 34 KB tile buffers fit an SM)
+  // L2 prefetch six tiles an SM ahead: one and a half to three waves, as 64 to 114
+  // registers a thread leave an SM four CTAs or two
   const int64_t prefetch = (reinterpret_cast<uintptr_t>(in) & 15) == 0 ? 6 * (int64_t)sm_count() : 0;
   return launch(name, s, [&] {
-    k_scan_excl<Tin, Tout><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, out, n, status, ctr, derr, total, maxv,
-                                                                    SPIN_LIMIT, prefetch);
+    k_scan_excl<Tin, Tout><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, out, n, status, ctr, derr, total, SPIN_LIMIT,
+                                                                    prefetch);
   });
 }
 
@@ -249,14 +243,9 @@ size_t scan_scratch_bytes(int64_t n) {
   return 256 + (size_t)(tiles + 1) * sizeof(uint64_t);
 }
 
-wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, int32_t* maxv, void* scratch,
-                             uint32_t* derr, cudaStream_t s) {
-  return run_scan<int32_t, int64_t>(in, out, n, total, maxv, scratch, derr, s, "scan_degrees");
-}
-
-wedge_status scan_counts_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch,
-                                uint32_t* derr, cudaStream_t s, const char* name) {
-  return run_scan<int32_t, int64_t>(in, out, n, total, nullptr, scratch, derr, s, name);
+wedge_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* total, void* scratch, uint32_t* derr,
+                             cudaStream_t s) {
+  return run_scan<int32_t, int64_t>(in, out, n, total, scratch, derr, s, "scan_degrees");
 }
 
 wedge_status scan_rows(const int32_t* fdeg, const int32_t* bdeg, const int64_t* foff, int64_t* boff, int64_t n,
@@ -273,17 +262,17 @@ wedge_status scan_rows(const int32_t* fdeg, const int32_t* bdeg, const int64_t* 
 
 wedge_status scan_u32_with_total(const uint32_t* in, int64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s) {
-  return run_scan<uint32_t, int64_t>(in, out, n, out + n, nullptr, scratch, derr, s, "scan_bin_counts");
+  return run_scan<uint32_t, int64_t>(in, out, n, out + n, scratch, derr, s, "scan_bin_counts");
 }
 
 wedge_status scan_u64_with_total(const uint64_t* in, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                  cudaStream_t s, const char* name) {
-  return run_scan<uint64_t, uint64_t>(in, out, n, out + n, nullptr, scratch, derr, s, name);
+  return run_scan<uint64_t, uint64_t>(in, out, n, out + n, scratch, derr, s, name);
 }
 
 wedge_status scan_pairs_with_total(const int32_t* deg, uint64_t* out, int64_t n, void* scratch, uint32_t* derr,
                                    cudaStream_t s, const char* name) {
-  return run_scan<Pairs, uint64_t>(reinterpret_cast<const Pairs*>(deg), out, n, out + n, nullptr, scratch, derr, s,
+  return run_scan<Pairs, uint64_t>(reinterpret_cast<const Pairs*>(deg), out, n, out + n, scratch, derr, s,
                                    name);
 }
 
@@ -361,7 +350,7 @@ extern "C" wedge_status wedge_degree_offsets_noalloc(const int32_t* deg, int64_t
   WEDGE_CUDA_TRY(cudaMemsetAsync(b, 0, NOALLOC_HEADER + (size_t)tiles * sizeof(uint64_t), s),
                  "wedge_degree_offsets_noalloc");
   k_scan_excl<int32_t, int64_t, true><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(deg, off, n, status, ctr, err,
-                                                                                 off + n, nullptr);
+                                                                                 off + n);
   WEDGE_CUDA_TRY(cudaGetLastError(), "wedge_degree_offsets_noalloc: launch");
   uint32_t herr = 0;
   WEDGE_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s),
@@ -413,7 +402,7 @@ extern "C" wedge_status wedge_test_lookback_timeout(uint32_t spin_limit, wedge_s
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctr, &one, sizeof(one), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return done(cuda_fail(e, "wedge_test_lookback_timeout"));
   st = launch("test_lookback_timeout", s, [&] {
-    k_scan_excl<int32_t, int64_t><<<1, SCAN_THREADS, 0, s>>>(in, out, n, status, ctr, derr, out + n, nullptr,
+    k_scan_excl<int32_t, int64_t><<<1, SCAN_THREADS, 0, s>>>(in, out, n, status, ctr, derr, out + n,
                                                              spin_limit);
   });
   if (st != WEDGE_OK) return done(st);

@@ -37,8 +37,7 @@ constexpr int CL_ITEMS = 8;
 constexpr uint64_t BLOCK_BYTES = 32 << 20;
 
 struct KeyStream {
-  int64_t start, len;   // the bin's vertices in L
-  uint64_t p, wbase;    // wedges in the bin, W[start]
+  uint64_t p, wbase;    // wedges in the bin, and before it (W at its start)
   uint64_t k, first;    // samples, first sample index
   uint64_t key_base;    // first key slot of the stream
   uint64_t tile_begin;  // first CTA
@@ -154,11 +153,8 @@ wedge_status sample_sorted_closure(const wedge_graph* g, const wedge_bins* b, ui
     for (int c = 0; c < 4; ++c) out->q[k][c] = 0;
   }
   for (uint32_t k = 2; k < nb; ++k) {
-    const int64_t len = inf.start[k + 1] - inf.start[k];
-    if (k_of_bin[k] == 0 || inf.p_b[k] == 0 || len == 0) continue;
+    if (k_of_bin[k] == 0 || inf.p_b[k] == 0) continue;
     KeyStream d;
-    d.start = inf.start[k];
-    d.len = len;
     d.p = inf.p_b[k];
     d.wbase = 0;
     for (uint32_t j = 2; j < k; ++j) d.wbase += inf.p_b[j];
