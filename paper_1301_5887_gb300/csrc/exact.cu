@@ -273,6 +273,13 @@ struct CountArgs {
   unsigned int* n_units;   // [0] medium, [1] long
 };
 
+// Times of the whole call in us, each constant alone changed, on Kronecker scale
+// 20 / scale 16 / power law of 1 M, gamma 2.3, 20 a vertex / uniform, 16.8 M edges of 4 M:
+//   as they are 5,124 / 535 / 1,774 / 3,013
+//   WARP_IN 32: 5,510 / 510 / 1,944 / 3,009; 128: 5,152 / 751 / 1,708 / 3,022
+//   MEMORY_ROW 4: 5,129 / 534 / 1,797 / 3,127; 16: 5,131 / 532 / 1,763 / 3,013 (and a ring
+//     with 16 neighbours a side, nearly all of whose looks find: 4,446, 5,483 with 8, 8,427)
+//   UNIT_IN 256: 5,635 / 529 / 1,852 / 3,014; 1,024: 4,870 / 541 / 1,755 / 3,016
 constexpr int WARP_ROW = 128;        // rows N+(v) up to this length ...
 constexpr int WARP_IN = 64;          // ... with in-lists up to this: one warp
 constexpr int WARP_SLOTS = 512;
