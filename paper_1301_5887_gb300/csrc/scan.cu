@@ -31,8 +31,11 @@ struct Pairs {
 
 // CHECK: inputs must be >= 0 (DERR_NEGATIVE otherwise) and every prefix must
 // fit the look-back words' 58-bit value field (DERR_OVERFLOW otherwise).
+// Bound by latency, so by the CTAs an SM holds: four at 64 registers (200 M
+// counts 697 us, 53 M degrees' wedges 193; left to itself the compiler takes
+// 116 registers for two CTAs, 1,113 and 304; three at 72, 845 and 230; five spill).
 template <typename Tin, typename Tout, bool CHECK = false>
-__global__ __launch_bounds__(SCAN_THREADS) void k_scan_excl(const Tin* __restrict__ in, Tout* __restrict__ out,
+__global__ __launch_bounds__(SCAN_THREADS, 4) void k_scan_excl(const Tin* __restrict__ in, Tout* __restrict__ out,
                                                             int64_t n, uint64_t* status, uint32_t* tile_ctr,
                                                             uint32_t* err, Tout* total,
                                                             uint32_t spin_limit = SPIN_LIMIT,
@@ -227,8 +230,7 @@ wedge_status run_scan(const Tin* in, Tout* out, int64_t n, Tout* total, void* sc
   uint32_t* ctr = tiles > 1 ? static_cast<uint32_t*>(scratch) : nullptr;
   uint64_t* status = reinterpret_cast<uint64_t*>(static_cast<char*>(scratch) + 256);
   if (tiles > 1) WEDGE_CUDA_TRY(cudaMemsetAsync(scratch, 0, 256 + (size_t)tiles * sizeof(uint64_t), s), name);
-  // L2 prefetch six tiles an SM ahead: one and a half to three waves, as 64 to 114
-  // registers a thread leave an SM four CTAs or two
+  // L2 prefetch six tiles an SM ahead, a wave and a half
   const int64_t prefetch = (reinterpret_cast<uintptr_t>(in) & 15) == 0 ? 6 * (int64_t)sm_count() : 0;
   return launch(name, s, [&] {
     k_scan_excl<Tin, Tout><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, out, n, status, ctr, derr, total, SPIN_LIMIT,
