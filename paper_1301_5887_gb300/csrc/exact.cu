@@ -726,7 +726,8 @@ struct ReadBack {
 };
 
 unsigned some_blocks(int64_t items) {
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + EX_THREADS - 1) / EX_THREADS, (int64_t)sm_count() * 8));
+  const int64_t blocks = (items + EX_THREADS - 1) / EX_THREADS;
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sm_count() * 8));
 }
 
 }  // namespace
@@ -789,7 +790,8 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
   EXACT_DO(dalloc_n(&words, n_words, s, "wedge_exact: ranks and counts"));
   EXACT_DO(dalloc_n(&keys, n_keys, s, "wedge_exact: edges"));
   EXACT_DO(dalloc_n(&alt, n_keys, s, "wedge_exact: edges"));
-  EXACT_DO(dalloc(reinterpret_cast<void**>(&scratch), sort_bytes + scan_scratch_bytes(2 * (int64_t)n), s, "wedge_exact"));
+  EXACT_DO(dalloc(reinterpret_cast<void**>(&scratch), sort_bytes + scan_scratch_bytes(2 * (int64_t)n), s,
+                  "wedge_exact"));
   const uint64_t max_units = (uint64_t)most / UNIT_IN + (uint64_t)most / WARP_IN + (uint64_t)m / WARP_ROW + 64;
   if (most > (int64_t)UINT32_MAX || max_units > UINT32_MAX)
     return done(fail(WEDGE_EINVAL, "wedge_exact: graph too large"));
@@ -942,12 +944,12 @@ wedge_status exact_tails(const wedge_graph* g, const wedge_bins* b, unsigned lon
       EXACT_DO(launch("exact_rows", s, [&] {
         const unsigned blocks = blocks_for(edges);
         if (edges == m) {
-          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of,
-                                                          ctl);
+          k_rows<true><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill,
+                                                     rows, m, tail_of, ctl);
         } else {
           k_run_ends<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end);
-          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill, rows, m, tail_of,
-                                                          ctl);
+          k_rows<false><<<blocks, EX_THREADS, 0, s>>>(sorted, edges, (uint32_t)n, down, v_of, row_off, run_end, fill,
+                                                      rows, m, tail_of, ctl);
           k_run_add<<<blocks, EX_THREADS, 0, s>>>(sorted, edges, run_end, fill);
         }
       }));

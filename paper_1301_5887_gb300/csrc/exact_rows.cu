@@ -15,7 +15,7 @@
 //      a found triangle costs one shared-memory atomic.
 // No ranks and no sort of the edges: 16n + 4m bytes, and less time than exact.cu
 // takes to prepare its tails where there is next to nothing to look up (a path of 4.2 M
-// vertices, us: 404 here, 1,472 there; the rule stands in exact.cu).
+// vertices, us: 391 here, 1,472 there; the rule stands in exact.cu).
 #include <string.h>
 
 #include <vector>
